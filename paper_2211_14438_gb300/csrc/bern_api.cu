@@ -47,6 +47,7 @@ struct TableSet {
   std::map<std::pair<int, int>, std::pair<DevBuf, DevBuf>> prod;
   std::vector<ProdTable> prod_host;
   DevBuf prod_arr;
+  std::vector<LexView> lex;         // by order, host array of Tables::lex
 };
 
 struct GraphEntry {
@@ -205,6 +206,40 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
     ts.view.lines[l] = (const int2*)bl.p;
     ts.bufs.push_back(bg);
     ts.bufs.push_back(bl);
+  }
+  // the slab enclosure's tables, all arrays of one order in one buffer
+  if (n >= 4) {
+    ts.lex.assign(kSlabMaxOrder + 1, LexView{});
+    for (int l = 2; l <= std::min(kSlabMaxOrder, ts.view.rscale_max); ++l) {
+      std::vector<uint32_t> pos;
+      std::vector<std::vector<int32_t>> off;
+      std::vector<std::vector<float>> wt;
+      build_lex_tables(n, l, pos, off, wt);
+      std::vector<uint32_t> img;
+      auto put = [&](const void* src, size_t words) {
+        const size_t at = img.size();
+        img.resize(at + words);
+        if (words) std::memcpy(img.data() + at, src, words * sizeof(uint32_t));
+        return at;
+      };
+      size_t at_off[kMaxVars + 1], at_wt[kMaxVars + 1];
+      const size_t at_pos = put(pos.data(), pos.size());
+      for (int m = 0; m <= n; ++m) {
+        at_off[m] = put(off[m].data(), off[m].size());
+        at_wt[m] = put(wt[m].data(), wt[m].size());
+      }
+      DevBuf b;
+      if ((e = b.reserve(img.size() * sizeof(uint32_t))) != cudaSuccess) return map_cuda(e);
+      cudaMemcpy(b.p, img.data(), img.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+      ts.bufs.push_back(b);
+      const uint32_t* d = (const uint32_t*)b.p;
+      ts.lex[l].pos = d + at_pos;
+      for (int m = 0; m <= n; ++m) {
+        if (!off[m].empty()) ts.lex[l].off[m] = (const int32_t*)(d + at_off[m]);
+        if (!wt[m].empty()) ts.lex[l].wt[m] = (const float*)(d + at_wt[m]);
+      }
+    }
+    ts.view.lex = ts.lex.data();
   }
   ts.view.row_dmax = std::min(kMaxRowDegree, row_path_max_degree(n));
   for (int D = 0; D <= ts.view.row_dmax; ++D) {

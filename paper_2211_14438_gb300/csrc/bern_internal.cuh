@@ -91,6 +91,19 @@ struct ProdTable {
 };
 constexpr int kProdStride = kMaxTableDegree + 1;   // prod[Dq * kProdStride + Ds]
 
+// Lexicographic layout of the monomials of total degree <= l (the last
+// exponent running), for the slab enclosure of four and more variables: pos[r]
+// the position of graded rank r, with a bit per variable it contains from bit
+// 24 on; off[m] the C(m-1+l, m-1) + 1 row offsets of m variables (a row: the
+// monomials sharing all exponents but the last); wt[m] the products
+// prod_k C(l, j_k) of m variables, rounded up.
+constexpr int kSlabMaxOrder = 10;
+struct LexView {
+  const uint32_t* pos = nullptr;
+  const int32_t* off[kMaxVars + 1] = {};
+  const float* wt[kMaxVars + 1] = {};
+};
+
 struct Tables {
   int n;
   int dmax;                        // degrees 0..dmax have square tables
@@ -112,6 +125,9 @@ struct Tables {
   int row_dmax;
   // product tables of the Horner kernel (device array of kProdStride^2)
   const ProdTable* prod;
+  // host array [kSlabMaxOrder + 1] of the slab enclosure's tables by order
+  // (null: none were built, as in the allocation-free path)
+  const LexView* lex;
 };
 
 // Largest Bernstein order whose grid fits the shared-memory limit for n vars.
@@ -127,6 +143,10 @@ void build_rscale(int n, int l, std::vector<float>& out);
 // the lines' base offsets and prefix digit sums; two int32 per line).
 void build_enclose_tables(int n, int l, std::vector<int32_t>& gidx, std::vector<int32_t>& lines,
                           bool with_lines = true);
+// Host images of the slab enclosure's tables for (n, l), n >= 4: pos, and
+// off[m] (m = 4..n) and wt[m] (m = 3..n-1).
+void build_lex_tables(int n, int l, std::vector<uint32_t>& pos,
+                      std::vector<std::vector<int32_t>>& off, std::vector<std::vector<float>>& wt);
 
 // ------------------------------------------------------------ launchers
 // Autotuning.  Launchers that have several valid variants for a shape ask
@@ -314,6 +334,14 @@ cudaError_t launch_enclose_blk(const Launch& L, const Tables& T, int lb, int G, 
                                int h, const float* pre_up, const float* pre_lo, int64_t ld,
                                const int32_t* nterms, float* lo, float* hi, const int* list,
                                const int* count, bool wide);
+
+// Four and more variables at orders 2..kSlabMaxOrder (k_enclose_slab.cu), lo/hi
+// only; needs T.lex.
+bool enclose_slab_ok(const Tables& T, int lb);
+cudaError_t launch_enclose_slab(const Launch& L, const Tables& T, int lb, int64_t n_items, int h,
+                                const float* pre_up, const float* pre_lo, int64_t ld,
+                                const int32_t* nterms, float* lo, float* hi, const int* list,
+                                const int* count);
 
 // The square of dense Bernstein tensors by Prod_Bern (k_bern_tensor.cu):
 // a [n_polys][(l+1)^n] -> coefficient intervals [c_lo, c_hi] of the square at

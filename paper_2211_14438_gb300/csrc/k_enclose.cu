@@ -4,7 +4,7 @@
 // runtime-order kernel below.
 #include <string>
 
-#include "enclose_impl.cuh"
+#include "enclose_tail.cuh"
 
 namespace bern {
 
@@ -122,11 +122,16 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
   int G;
   const int lb = effective_order(T.n, order, budget, &G, L.ews != nullptr);
   if (lb > T.rscale_max || T.rscale[lb] == nullptr) return cudaErrorInvalidValue;
+  // Order 1, and two and three variables up to order kTailMaxOrder: the last two
+  // passes in registers (k_enclose_tail.cu)
+  if (enclose_tail_ok(T.n, lb))
+    return launch_enclose_tail(L, T, lb, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
   // Shared-memory grids of at least 256 cells: a block per polynomial
   // (variants 3 and 4 of the enclosure tuner: 128 or 320 threads; 3 is the
   // default from kEncloseBlkGrid cells) or a warp per polynomial (variants
   // 0-2, items per block)
-  const bool blk_ok = G >= 256 && G <= kEncloseGridMax && lb >= 3 && lb <= 16;
+  const bool slab = enclose_slab_ok(T, lb);   // four and more variables: no grid
+  const bool blk_ok = !slab && G >= 256 && G <= kEncloseGridMax && lb >= 3 && lb <= 16;
   bool blk = false, blk_wide = false;
   TuneTimer tt;
   std::string key;
@@ -137,12 +142,14 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
     blk = v >= 3;
     blk_wide = v == 4;
   }
-  if (G > kEncloseGridMax || blk) {
-    // global-memory grids, or a block per polynomial: lo/hi, then the ReLU
-    // step on the same items
+  if (slab || G > kEncloseGridMax || blk) {
+    // slabs, global-memory grids, or a block per polynomial: lo/hi, then the
+    // ReLU step on the same items
     if (blk) tune_begin(L, "enclose", tt);
     cudaError_t e =
-        G > kEncloseGridMax
+        slab ? launch_enclose_slab(L, T, lb, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi,
+                                   ro.list, ro.count)
+        : G > kEncloseGridMax
             ? launch_enclose_big(L, T, lb, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi,
                                  ro.list, ro.count)
             : launch_enclose_blk(L, T, lb, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi,

@@ -1,0 +1,301 @@
+// a2 (Sec. 5.1 Step 1 with Def. 2) for two and three variables at the orders
+// whose last two passes fit a thread's registers, and for order 1.
+//
+// The passes of enclose_impl.cuh run from the last variable to the first, so
+// once the digits of the variables above the second are fixed, what is left
+// is a polynomial in t_1, t_2 of at most (l+1)(l+2)/2 coefficients: a thread
+// holds those in registers and runs the passes of variables 2 and 1 on
+// compile-time indices (line_transform's FMAs, in its order, so every
+// coefficient is bit for bit that of the grid kernels).  The lower bound is
+// the negated upper bound of the negated polynomial (RD(x) = -RU(-x)), so
+// one instruction stream serves both.
+//
+// Bound: FP32 issue.  The grid in shared memory that it replaces cost a
+// shared-memory access for every two FMAs; here the only shared-memory traffic
+// is the first pass (three variables: (l+1)(l+2)(l+3)/6 loads, mostly
+// broadcasts, per (l+1)(l+2)/2 register coefficients), 1 load to 4 FMAs at
+// order 8.
+#include <string>
+
+#include "enclose_tail.cuh"
+
+namespace bern {
+
+namespace {
+
+// Threads of a block of the three-variable kernel; a block takes as many items
+// as give every thread one (item, digit of t_3) task.
+constexpr int kTailThreads = 128;
+template <int LB>
+constexpr int tail_items() {
+  return kTailThreads / (LB + 1);
+}
+
+// Three variables: the scaled coefficients of the block's items sit in shared
+// memory in lexicographic order (rows of t_3), a thread takes one digit i_3
+// of one item's two polynomials.
+template <int LB>
+__global__ void __launch_bounds__(kTailThreads, (LB >= 7 ? 4 : (LB >= 5 ? 6 : 8)))
+k_enclose_tail3(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
+                const float* __restrict__ pre_up, const float* __restrict__ pre_lo, int64_t ld,
+                const int32_t* __restrict__ nterms, float* __restrict__ lo,
+                float* __restrict__ hi, EncloseOpts ro, int* status) {
+  constexpr int R = LB + 1, M3 = R * (R + 1) * (R + 2) / 6, MS = M3 | 1;
+  constexpr int IB = tail_items<LB>(), RB = kTailThreads / IB;   // rows loaded at a time
+  __shared__ p2 s_c[IB * MS];
+  __shared__ p2 s_bin[R * R];
+  __shared__ float2 s_sc[M3];
+  __shared__ int s_at[M3];                     // graded rank -> lexicographic position
+  __shared__ int s_bl[IB], s_bu[IB];
+  __shared__ float s_rl[IB], s_ru[IB];
+  __shared__ int64_t s_item[IB], s_base[IB];
+  __shared__ int s_nt[IB], s_any;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int x = tid; x < R * R; x += kTailThreads)
+    s_bin[x] = pack2(binomf(x / R, x % R), binomf(x / R, x % R));
+  for (int r = tid; r < M3; r += kTailThreads) {
+    const int g = __ldg(T.gidx[LB] + r), j1 = g / (R * R), j2 = g / R % R;
+    s_at[r] = lex3(LB, j1, j2) + g % R;
+    s_sc[r] = __ldg(rs + r);
+  }
+  const int my = tid % IB, my_r = tid / IB;    // this thread's item and first row in loads
+  const int64_t n_list = ro.list ? (int64_t)*ro.count : n_items;
+  for (int64_t i0 = (int64_t)blockIdx.x * IB; i0 < n_list; i0 += (int64_t)gridDim.x * IB) {
+    __syncthreads();                           // the previous items are finished
+    if (tid == 0) s_any = 0;
+    if (tid < IB) {
+      const int64_t item = i0 + tid < n_list ? (ro.list ? (int64_t)ro.list[i0 + tid] : i0 + tid)
+                                             : -1;
+      int nt = item >= 0 ? nterms[item] : 0;
+      if (nt < 0 || nt > ld || nt > T.mexps) {
+        atomicOr(status, kStatusInvalid);
+        nt = 0;
+      }
+      const int64_t b = item >= 0 ? item / h : 0;
+      s_item[tid] = item;
+      s_base[tid] = item >= 0 ? (b * ld) * h + (item - b * h) : 0;
+      s_nt[tid] = nt;
+      s_bl[tid] = float_key(-CUDART_INF_F);
+      s_bu[tid] = float_key(-CUDART_INF_F);
+      s_rl[tid] = 0.0f;
+      s_ru[tid] = 0.0f;
+    }
+    __syncthreads();
+    if (my_r < RB) {
+      // neighbouring threads take neighbouring neurons of one coefficient; all
+      // loads of a thread are independent
+      const int nt = s_nt[my];
+      const float* pu = pre_up + s_base[my];
+      const float* pl = pre_lo + s_base[my];
+      p2* dst = s_c + my * MS;
+#pragma unroll 8
+      for (int r = my_r; r < M3; r += RB) {
+        const float u = r < nt ? pu[(int64_t)r * h] : 0.0f;
+        const float l = r < nt ? -pl[(int64_t)r * h] : 0.0f;
+        dst[s_at[r]] = scale_pair(l, u, s_sc[r]);
+      }
+      if (my_r == 0 && nt > M3) s_any = 1;
+    }
+    __syncthreads();
+    if (s_any) {
+      // terms above the order: their one-sided ranges, a warp per item
+      for (int i = warp; i < IB; i += kTailThreads / 32) {
+        float ru = 0.0f, rl = 0.0f;
+        for (int r = lane; r < s_nt[i]; r += 32) {
+          if (r < M3) continue;
+          ru = __fadd_ru(ru, fmaxf(pre_up[s_base[i] + (int64_t)r * h], 0.0f));
+          rl = __fadd_ru(rl, fmaxf(-pre_lo[s_base[i] + (int64_t)r * h], 0.0f));
+        }
+        ru = warp_dsum<true>(ru);
+        rl = warp_dsum<true>(rl);
+        if (lane == 0) {
+          s_ru[i] = ru;
+          s_rl[i] = rl;
+        }
+      }
+    }
+    if (tid < IB * R && i0 + tid / R < n_list) {
+      float bl = -CUDART_INF_F, bu = -CUDART_INF_F;
+      tail_max<LB>(s_c + tid / R * MS, tid % R, s_bin, bl, bu);
+      atomicMax(&s_bl[tid / R], float_key(bl));
+      atomicMax(&s_bu[tid / R], float_key(bu));
+    }
+    __syncthreads();
+    if (tid < IB && s_item[tid] >= 0) {
+      const int64_t it = s_item[tid];
+      const float l = -__fadd_ru(key_float(s_bl[tid]), s_rl[tid]);
+      const float u = __fadd_ru(key_float(s_bu[tid]), s_ru[tid]);
+      lo[it] = l;
+      hi[it] = u;
+      if (!(isfinite(l) && isfinite(u))) atomicOr(status, kStatusNonFinite);
+      if (ro.kind != nullptr) {
+        const int d = ro.degrees ? (int)ro.degrees[it] : ro.global_d;
+        ro.kind[it] = (int8_t)relu_item(l, u, d, ro.coef + it * kCoefStride, ro.eps + it, status);
+      }
+    }
+  }
+}
+
+// Two variables: a thread per item, its coefficients straight into registers
+// (rank of (j_1, j_2): s (s + 1) / 2 + j_2, s = j_1 + j_2).  Neighbouring
+// threads take neighbouring items.
+template <int LB>
+__global__ void __launch_bounds__(128)
+k_enclose_tail2(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
+                const float* __restrict__ pre_up, const float* __restrict__ pre_lo, int64_t ld,
+                const int32_t* __restrict__ nterms, float* __restrict__ lo,
+                float* __restrict__ hi, EncloseOpts ro, int* status) {
+  constexpr int R = LB + 1, M2 = R * (R + 1) / 2;
+  const int64_t n_list = ro.list ? (int64_t)*ro.count : n_items;
+  for (int64_t at = (int64_t)blockIdx.x * 128 + threadIdx.x; at < n_list;
+       at += (int64_t)gridDim.x * 128) {
+    const int64_t item = ro.list ? (int64_t)ro.list[at] : at;
+    int nt = nterms[item];
+    if (nt < 0 || nt > ld || nt > T.mexps) {
+      atomicOr(status, kStatusInvalid);
+      nt = 0;
+    }
+    const int64_t b = item / h;
+    const float* pu = pre_up + (b * ld) * h + (item - b * h);
+    const float* pl = pre_lo + (b * ld) * h + (item - b * h);
+    p2 q[M2];
+#pragma unroll
+    for (int s = 0; s <= LB; ++s)
+#pragma unroll
+      for (int j = 0; j <= s; ++j) {
+        const int r = s * (s + 1) / 2 + j;
+        q[lex2(LB, s - j) + j] = r < nt ? pack2(-pl[(int64_t)r * h], pu[(int64_t)r * h])
+                                        : pack2(0.0f, 0.0f);
+      }
+#pragma unroll
+    for (int s = 0; s <= LB; ++s)
+#pragma unroll
+      for (int j = 0; j <= s; ++j) {
+        float l, u;
+        unpack2(q[lex2(LB, s - j) + j], l, u);
+        q[lex2(LB, s - j) + j] = scale_pair(l, u, __ldg(rs + s * (s + 1) / 2 + j));
+      }
+    float ru = 0.0f, rl = 0.0f;
+    for (int r = M2; r < nt; ++r) {
+      ru = __fadd_ru(ru, fmaxf(pu[(int64_t)r * h], 0.0f));
+      rl = __fadd_ru(rl, fmaxf(-pl[(int64_t)r * h], 0.0f));
+    }
+    float bl = -CUDART_INF_F, bu = -CUDART_INF_F;
+    pair_max<LB>(q, bl, bu);
+    const float l = -__fadd_ru(bl, rl), u = __fadd_ru(bu, ru);
+    lo[item] = l;
+    hi[item] = u;
+    if (!(isfinite(l) && isfinite(u))) atomicOr(status, kStatusNonFinite);
+    if (ro.kind != nullptr) {
+      const int d = ro.degrees ? (int)ro.degrees[item] : ro.global_d;
+      ro.kind[item] = (int8_t)relu_item(l, u, d, ro.coef + item * kCoefStride, ro.eps + item,
+                                        status);
+    }
+  }
+}
+
+// Order 1: the coefficients are the values at the vertices, and with the
+// passes' rounding from the last variable to the first the largest is
+// a_0 plus the positive linear coefficients in that order.  A thread per
+// item.
+__global__ void __launch_bounds__(256)
+k_enclose_order1(Tables T, int64_t n_items, int h, const float* __restrict__ pre_up,
+                 const float* __restrict__ pre_lo, int64_t ld,
+                 const int32_t* __restrict__ nterms, float* __restrict__ lo,
+                 float* __restrict__ hi, EncloseOpts ro, int* status) {
+  const int n = T.n;
+  const int64_t n_list = ro.list ? (int64_t)*ro.count : n_items;
+  for (int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; at < n_list;
+       at += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t item = ro.list ? (int64_t)ro.list[at] : at;
+    int nt = nterms[item];
+    if (nt < 0 || nt > ld || nt > T.mexps) {
+      atomicOr(status, kStatusInvalid);
+      nt = 0;
+    }
+    const int64_t b = item / h;
+    const int64_t base = (b * ld) * h + (item - b * h);
+    float u = 0.0f, l = 0.0f;
+    if (nt > 0) {
+      u = pre_up[base];
+      l = pre_lo[base];
+    }
+    float cu[kMaxVars], cl[kMaxVars];
+#pragma unroll
+    for (int k = 0; k < kMaxVars; ++k) {   // rank 1 + k: t_(k+1)
+      const bool live = k < n && 1 + k < nt;
+      cu[k] = live ? pre_up[base + (int64_t)(1 + k) * h] : 0.0f;
+      cl[k] = live ? pre_lo[base + (int64_t)(1 + k) * h] : 0.0f;
+    }
+#pragma unroll
+    for (int k = kMaxVars - 1; k >= 0; --k) {
+      u = __fadd_ru(u, fmaxf(cu[k], 0.0f));
+      l = __fadd_rd(l, fminf(cl[k], 0.0f));
+    }
+    float ru = 0.0f, rl = 0.0f;
+    for (int r = n + 1; r < nt; ++r) {
+      ru = __fadd_ru(ru, fmaxf(pre_up[base + (int64_t)r * h], 0.0f));
+      rl = __fadd_rd(rl, fminf(pre_lo[base + (int64_t)r * h], 0.0f));
+    }
+    u = __fadd_ru(u, ru);
+    l = __fadd_rd(l, rl);
+    lo[item] = l;
+    hi[item] = u;
+    if (!(isfinite(l) && isfinite(u))) atomicOr(status, kStatusNonFinite);
+    if (ro.kind != nullptr) {
+      const int d = ro.degrees ? (int)ro.degrees[item] : ro.global_d;
+      ro.kind[item] = (int8_t)relu_item(l, u, d, ro.coef + item * kCoefStride, ro.eps + item,
+                                        status);
+    }
+  }
+}
+
+}  // namespace
+
+bool enclose_tail_ok(int n, int lb) {
+  return lb == 1 || (n == 2 && lb >= 2 && lb <= kTailMaxOrder) ||
+         (n == 3 && lb >= 2 && lb <= kTailMaxOrder);
+}
+
+cudaError_t launch_enclose_tail(const Launch& L, const Tables& T, int lb, int64_t n_items, int h,
+                                const float* pre_up, const float* pre_lo, int64_t ld,
+                                const int32_t* nterms, float* lo, float* hi,
+                                const EncloseOpts& ro) {
+  const int64_t sms = device_sms(L);
+  ++*L.launches;
+  if (lb == 1) {
+    const int64_t blocks = std::min<int64_t>((n_items + 255) / 256, sms * 8);
+    k_enclose_order1<<<(unsigned)blocks, 256, 0, L.stream>>>(T, n_items, h, pre_up, pre_lo, ld,
+                                                             nterms, lo, hi, ro, L.status);
+    return cudaGetLastError();
+  }
+  if (T.n == 2) {
+    const int64_t blocks = std::min<int64_t>((n_items + 127) / 128, sms * 16);
+#define BERN_T2(X)                                                                              \
+  case X:                                                                                       \
+    k_enclose_tail2<X><<<(unsigned)blocks, 128, 0, L.stream>>>(T, T.rscale[X], n_items, h, pre_up, \
+                                                               pre_lo, ld, nterms, lo, hi, ro,  \
+                                                               L.status);                       \
+    return cudaGetLastError();
+    switch (lb) {
+      BERN_T2(2) BERN_T2(3) BERN_T2(4) BERN_T2(5) BERN_T2(6) BERN_T2(7) BERN_T2(8)
+      default: return cudaErrorInvalidValue;
+    }
+#undef BERN_T2
+  }
+#define BERN_T3(X)                                                                              \
+  case X: {                                                                                     \
+    const int64_t need = (n_items + tail_items<X>() - 1) / tail_items<X>();                     \
+    k_enclose_tail3<X><<<(unsigned)std::min<int64_t>(need, sms * 16), kTailThreads, 0,           \
+                         L.stream>>>(T, T.rscale[X], n_items, h, pre_up, pre_lo, ld, nterms, lo, \
+                                     hi, ro, L.status);                                         \
+    return cudaGetLastError();                                                                  \
+  }
+  switch (lb) {
+    BERN_T3(2) BERN_T3(3) BERN_T3(4) BERN_T3(5) BERN_T3(6) BERN_T3(7) BERN_T3(8)
+    default: return cudaErrorInvalidValue;
+  }
+#undef BERN_T3
+}
+
+}  // namespace bern

@@ -286,6 +286,63 @@ void build_rscale(int n, int l, std::vector<float>& out) {
   }
 }
 
+// Lexicographic exponents of total degree <= l in m variables.
+static void lex_monomials(int m, int l, std::vector<uint8_t>& ex) {
+  ex.clear();
+  std::vector<int> e(m, 0);
+  int left = l;
+  for (;;) {
+    for (int k = 0; k < m; ++k) ex.push_back((uint8_t)e[k]);
+    int k = m - 1;
+    if (left == 0) {
+      // the last non-zero exponent gives way to its left neighbour
+      while (k >= 0 && e[k] == 0) --k;
+      if (k <= 0) return;
+      left += e[k];
+      e[k] = 0;
+      --k;
+    }
+    ++e[k];
+    --left;
+  }
+}
+
+void build_lex_tables(int n, int l, std::vector<uint32_t>& pos,
+                      std::vector<std::vector<int32_t>>& off, std::vector<std::vector<float>>& wt) {
+  off.assign(n + 1, {});
+  wt.assign(n + 1, {});
+  double binom[kMaxTableDegree + 1];
+  binom[0] = 1.0;
+  for (int j = 1; j <= l; ++j) binom[j] = binom[j - 1] * (l - j + 1) / j;
+  std::map<uint64_t, uint32_t> at;
+  for (int m = 3; m <= n; ++m) {
+    std::vector<uint8_t> ex;
+    lex_monomials(m, l, ex);
+    const size_t rows = ex.size() / m;
+    for (size_t r = 0; r < rows; ++r) {
+      const uint8_t* e = &ex[r * m];
+      if (m < n) {
+        double w = 1.0;
+        for (int k = 0; k < m; ++k) w *= binom[e[k]];
+        float f = (float)w;
+        if ((double)f < w) f = std::nextafterf(f, INFINITY);
+        wt[m].push_back(f);
+      }
+      if (m >= 4 && e[m - 1] == 0) off[m].push_back((int32_t)r);
+      if (m == n) {
+        uint32_t mask = 0;
+        for (int k = 0; k < n; ++k) mask |= (e[k] ? 1u : 0u) << k;
+        at[pack_key(e, n)] = (uint32_t)r | mask << 24;
+      }
+    }
+    if (m >= 4) off[m].push_back((int32_t)rows);
+  }
+  std::vector<uint8_t> ex;
+  graded_monomials(n, l, ex);
+  pos.resize((size_t)num_monomials(n, l));
+  for (size_t r = 0; r < pos.size(); ++r) pos[r] = at[pack_key(&ex[r * n], n)];
+}
+
 }  // namespace bern
 
 namespace bern {
