@@ -33,7 +33,15 @@
 // three-variable slab and runs the last two passes in registers.
 //
 // Bound: FP32 issue in the register passes (610 of about 1000 instructions of
-// a digit at order 8 are packed FMAs).
+// a digit at order 8 are packed FMAs; the FP32 pipe is 48% busy).
+//
+// Three forms, by what fits where (launch_enclose_slab): order 2, and orders 3
+// and 4 of few variables, fix every digit above t_3 in registers
+// (k_enclose_regs); up to the shared memory of a quarter SM all slabs of a
+// level are made at once, without bounds (k_enclose_expand); above, digit by
+// digit with pruning (k_enclose_slab).  Measured against the grid kernels on
+// the layers of the [6,100x3,2] network, 2048 boxes: order 2 344 -> 85 us,
+// order 4 31.5 -> 1.82 ms (slabs: 3.35 ms), order 8 17.1 -> 2.15 ms.
 #include "enclose_tail.cuh"
 
 namespace bern {
@@ -337,6 +345,410 @@ cudaError_t launch_slab(const Launch& L, const Tables& T, const LexView& X, int6
   return cudaGetLastError();
 }
 
+// ------------------------------------------------------------ registers
+// Order 2 from four variables on, order 3 up to six and order 4 in four: at
+// most 84 coefficients, so a thread fixes all digits above t_3 in registers
+// (each level by the same FMAs as slab_row) and runs the digits of t_3; no
+// level is stored at all.  64,000 items of four variables at order 4: 64 us
+// with the levels in shared memory, 27 us here.
+template <int M, int LB>
+struct LexRows {
+  static constexpr int count() {
+    int c = 1;
+    for (int i = 1; i < M; ++i) c = c * (LB + i) / i;   // C(M-1+LB, M-1)
+    return c;
+  }
+  int off[count() + 1];
+  constexpr LexRows() : off() {
+    // rows: the exponents of the first M-1 variables, lexicographic; a row of
+    // degree d holds LB - d + 1 coefficients
+    int e[M] = {};
+    int left = LB, at = 0;
+    for (int r = 0; r < count(); ++r) {
+      off[r] = at;
+      at += left + 1;
+      int k = M - 2;
+      if (left == 0) {
+        while (k > 0 && e[k] == 0) --k;
+        left += e[k];
+        e[k] = 0;
+        --k;
+      }
+      if (k >= 0) {
+        ++e[k];
+        --left;
+      }
+    }
+    off[count()] = at;
+  }
+};
+
+// Digit d of the last of M variables: src (M variables) -> dst (M - 1).
+template <int M, int LB, class Src>
+__device__ __forceinline__ void fix_digit(const Src& src, int d, const p2* bin,
+                                          p2 (&dst)[LexRows<M, LB>::count()]) {
+  constexpr LexRows<M, LB> t{};
+#pragma unroll
+  for (int r = 0; r < LexRows<M, LB>::count(); ++r) dst[r] = src[t.off[r]];
+#pragma unroll
+  for (int j = 1; j <= LB; ++j)
+    if (j <= d) {
+      const p2 w = bin[d * (LB + 1) + j];
+#pragma unroll
+      for (int r = 0; r < LexRows<M, LB>::count(); ++r)
+        if (t.off[r + 1] - t.off[r] > j) dst[r] = fma2_ru(w, src[t.off[r] + j], dst[r]);
+    }
+}
+
+// The largest coefficients over the digits of t_3 of three-variable slab q.
+template <int LB>
+__device__ __forceinline__ void slab_max(const p2 (&q)[LexRows<4, LB>::count()], float& bl,
+                                         float& bu) {
+  constexpr LexRows<3, LB> t{};
+#pragma unroll
+  for (int i3 = 0; i3 <= LB; ++i3) {
+    p2 x[LexRows<3, LB>::count()];
+#pragma unroll
+    for (int r = 0; r < LexRows<3, LB>::count(); ++r) {
+      p2 acc = q[t.off[r]];
+#pragma unroll
+      for (int j = 1; j <= LB; ++j)
+        if (j <= i3 && j < t.off[r + 1] - t.off[r])
+          acc = i3 == j ? add2_ru(q[t.off[r] + j], acc)
+                        : fma2_ru(pack2(cbin(i3, j), cbin(i3, j)), q[t.off[r] + j], acc);
+      x[r] = acc;
+    }
+    pair_max<LB>(x, bl, bu);
+  }
+}
+
+// The digits of t_M .. t_4 in mixed radix from `digits`, then t_3 .. t_1.
+template <int M, int LB, class Src>
+__device__ __forceinline__ void fix_all(const Src& src, int digits, const p2* bin, float& bl,
+                                        float& bu) {
+  p2 dst[LexRows<M, LB>::count()];
+  fix_digit<M, LB>(src, digits % (LB + 1), bin, dst);
+  if constexpr (M > 4)
+    fix_all<M - 1, LB>(dst, digits / (LB + 1), bin, bl, bu);
+  else
+    slab_max<LB>(dst, bl, bu);
+}
+
+constexpr int kRegThreads = 128;
+template <int N, int LB>
+__global__ void __launch_bounds__(kRegThreads, N >= 8 || LB >= 3 ? 4 : 5)
+k_enclose_regs(Tables T, LexView X, const float2* __restrict__ rs, int64_t n_items, int h,
+               const float* __restrict__ pre_up, const float* __restrict__ pre_lo, int64_t ld,
+               const int32_t* __restrict__ nterms, float* __restrict__ lo, float* __restrict__ hi,
+               const int* list, const int* count, int* status) {
+  constexpr int R = LB + 1, MN = LexRows<N + 1, LB>::count(), MS = MN | 1;
+  constexpr int TASKS = cipow(R, N - 3);                      // per item
+  constexpr int IB = TASKS < kRegThreads ? kRegThreads / TASKS : 1;
+  constexpr int RB = kRegThreads / IB;
+  __shared__ p2 s_c[IB * MS];
+  __shared__ p2 s_bin[R * R];
+  __shared__ float2 s_sc[MN];
+  __shared__ int s_at[MN];
+  __shared__ int s_bl[IB], s_bu[IB];
+  __shared__ float s_rl[IB], s_ru[IB];
+  __shared__ int64_t s_item[IB], s_base[IB];
+  __shared__ int s_nt[IB];
+  const int tid = threadIdx.x;
+  for (int x = tid; x < R * R; x += kRegThreads)
+    s_bin[x] = pack2(binomf(x / R, x % R), binomf(x / R, x % R));
+  for (int r = tid; r < MN; r += kRegThreads) {
+    s_at[r] = (int)(__ldg(X.pos + r) & 0xffffffu);
+    s_sc[r] = __ldg(rs + r);
+  }
+  const int my = tid % IB, my_r = tid / IB;
+  const int64_t n_list = list ? (int64_t)*count : n_items;
+  for (int64_t i0 = (int64_t)blockIdx.x * IB; i0 < n_list; i0 += (int64_t)gridDim.x * IB) {
+    __syncthreads();                                 // the previous items are finished
+    if (tid < IB) {
+      const int64_t item = i0 + tid < n_list ? (list ? (int64_t)list[i0 + tid] : i0 + tid) : -1;
+      int nt = item >= 0 ? nterms[item] : 0;
+      if (nt < 0 || nt > ld || nt > T.mexps) {
+        atomicOr(status, kStatusInvalid);
+        nt = 0;
+      }
+      const int64_t b = item >= 0 ? item / h : 0;
+      s_item[tid] = item;
+      s_base[tid] = item >= 0 ? (b * ld) * h + (item - b * h) : 0;
+      s_nt[tid] = nt;
+      s_bl[tid] = float_key(-CUDART_INF_F);
+      s_bu[tid] = float_key(-CUDART_INF_F);
+      // terms above the order: their one-sided ranges
+      float ru = 0.0f, rl = 0.0f;
+      for (int r = MN; r < nt; ++r) {
+        ru = __fadd_ru(ru, fmaxf(pre_up[s_base[tid] + (int64_t)r * h], 0.0f));
+        rl = __fadd_ru(rl, fmaxf(-pre_lo[s_base[tid] + (int64_t)r * h], 0.0f));
+      }
+      s_rl[tid] = rl;
+      s_ru[tid] = ru;
+    }
+    __syncthreads();
+    if (my_r < RB) {
+      const int nt = s_nt[my];
+      const float* pu = pre_up + s_base[my];
+      const float* pl = pre_lo + s_base[my];
+#pragma unroll 4
+      for (int r = my_r; r < MN; r += RB) {
+        const float u = r < nt ? pu[(int64_t)r * h] : 0.0f;
+        const float l = r < nt ? -pl[(int64_t)r * h] : 0.0f;
+        s_c[my * MS + s_at[r]] = scale_pair(l, u, s_sc[r]);
+      }
+    }
+    __syncthreads();
+    for (int t = tid; t < IB * TASKS; t += kRegThreads) {
+      const int i = t / TASKS;
+      if (i0 + i >= n_list) break;
+      float bl = -CUDART_INF_F, bu = -CUDART_INF_F;
+      const p2* src = s_c + i * MS;
+      fix_all<N, LB>(src, t - i * TASKS, s_bin, bl, bu);
+      atomicMax(&s_bl[i], float_key(bl));
+      atomicMax(&s_bu[i], float_key(bu));
+    }
+    __syncthreads();
+    if (tid < IB && s_item[tid] >= 0) {
+      const int64_t it = s_item[tid];
+      const float l = -__fadd_ru(key_float(s_bl[tid]), s_rl[tid]);
+      const float u = __fadd_ru(key_float(s_bu[tid]), s_ru[tid]);
+      lo[it] = l;
+      hi[it] = u;
+      if (!(isfinite(l) && isfinite(u))) atomicOr(status, kStatusNonFinite);
+    }
+  }
+}
+
+template <int N, int LB>
+cudaError_t launch_regs(const Launch& L, const Tables& T, const LexView& X, int64_t n_items, int h,
+                        const float* pre_up, const float* pre_lo, int64_t ld,
+                        const int32_t* nterms, float* lo, float* hi, const int* list,
+                        const int* count) {
+  constexpr int TASKS = cipow(LB + 1, N - 3);
+  constexpr int IB = TASKS < kRegThreads ? kRegThreads / TASKS : 1;
+  const int64_t blocks = std::min<int64_t>((n_items + IB - 1) / IB, (int64_t)device_sms(L) * 16);
+  k_enclose_regs<N, LB><<<(unsigned)blocks, kRegThreads, 0, L.stream>>>(
+      T, X, T.rscale[LB], n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, list, count, L.status);
+  ++*L.launches;
+  return cudaGetLastError();
+}
+
+// ------------------------------------------------------------ expansion
+// The same levels without pruning, all slabs of a level at once and several
+// items per block, for the shapes whose last level fits shared memory: small
+// grids have too few slabs per item to fill a block, and too little behind a
+// slab to pay for its bound.
+constexpr int64_t kExpandBytes = 52 * 1024;   // shared memory of a block: four per SM
+
+struct ExpandShape {
+  int n, ib;                   // items per block
+  int M[kMaxVars + 1];
+  int stride[kMaxVars + 1];    // pairs between the slabs of a level
+  int off_tab[kMaxVars + 1];   // row offsets of level m (uint16) in the table area
+  int slabs;                   // slabs of the last level per item, R^(n - BOT)
+  int off_a, off_b;            // the two level buffers (pairs)
+  int total;
+};
+
+// BOT: the variables of the last level: three, whose digits run tail_max, or
+// four up to order 4, where a thread fixes the digit of t_4 in registers and
+// runs all digits of t_3 (fix_all).
+template <int LB>
+constexpr int expand_bottom() { return LB <= 4 ? 4 : 3; }
+
+template <int LB, int NT>
+__global__ void __launch_bounds__(NT, (LB <= 4 ? 4 : 2))
+k_enclose_expand(Tables T, LexView X, ExpandShape sh, const float2* __restrict__ rs,
+                 int64_t n_items, int h, const float* __restrict__ pre_up,
+                 const float* __restrict__ pre_lo, int64_t ld, const int32_t* __restrict__ nterms,
+                 float* __restrict__ lo, float* __restrict__ hi, const int* list, const int* count,
+                 int* status) {
+  constexpr int R = LB + 1, NW = NT / 32, IBMAX = NT / R, BOT = expand_bottom<LB>();
+  extern __shared__ p2 sm[];
+  __shared__ p2 s_bin[R * R];
+  __shared__ int s_bl[IBMAX], s_bu[IBMAX], s_nt[IBMAX], s_any;
+  __shared__ float s_rl[IBMAX], s_ru[IBMAX];
+  __shared__ int64_t s_item[IBMAX], s_base[IBMAX];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = sh.n, ib = sh.ib, Mn = sh.M[n];
+  uint16_t* tab = reinterpret_cast<uint16_t*>(sm);
+  for (int x = tid; x < R * R; x += NT) s_bin[x] = pack2(binomf(x / R, x % R), binomf(x / R, x % R));
+  for (int m = 4; m <= n; ++m)
+    for (int x = tid; x <= sh.M[m - 1]; x += NT)
+      tab[sh.off_tab[m] + x] = (uint16_t)__ldg(X.off[m] + x);
+  const int my = tid % ib, my_r = tid / ib, rb = NT / ib;
+  const int64_t n_list = list ? (int64_t)*count : n_items;
+  for (int64_t i0 = (int64_t)blockIdx.x * ib; i0 < n_list; i0 += (int64_t)gridDim.x * ib) {
+    __syncthreads();                                 // the previous items are finished
+    if (tid == 0) s_any = 0;
+    if (tid < ib) {
+      const int64_t item = i0 + tid < n_list ? (list ? (int64_t)list[i0 + tid] : i0 + tid) : -1;
+      int nt = item >= 0 ? nterms[item] : 0;
+      if (nt < 0 || nt > ld || nt > T.mexps) {
+        atomicOr(status, kStatusInvalid);
+        nt = 0;
+      }
+      const int64_t b = item >= 0 ? item / h : 0;
+      s_item[tid] = item;
+      s_base[tid] = item >= 0 ? (b * ld) * h + (item - b * h) : 0;
+      s_nt[tid] = nt;
+      s_bl[tid] = float_key(-CUDART_INF_F);
+      s_bu[tid] = float_key(-CUDART_INF_F);
+      s_rl[tid] = 0.0f;
+      s_ru[tid] = 0.0f;
+    }
+    __syncthreads();
+    p2* cur = sm + sh.off_a;
+    p2* nxt = sm + sh.off_b;
+    if (my_r < rb) {
+      const int nt = s_nt[my];
+      const float* pu = pre_up + s_base[my];
+      const float* pl = pre_lo + s_base[my];
+      p2* dst = cur + my * sh.stride[n];
+#pragma unroll 4
+      for (int r = my_r; r < Mn; r += rb) {
+        const float u = r < nt ? pu[(int64_t)r * h] : 0.0f;
+        const float l = r < nt ? -pl[(int64_t)r * h] : 0.0f;
+        dst[__ldg(X.pos + r) & 0xffffffu] = scale_pair(l, u, __ldg(rs + r));
+      }
+      if (my_r == 0 && nt > Mn) s_any = 1;
+    }
+    __syncthreads();
+    if (s_any) {
+      // terms above the order: their one-sided ranges, a warp per item
+      for (int i = warp; i < ib; i += NW) {
+        float ru = 0.0f, rl = 0.0f;
+        for (int r = lane; r < s_nt[i]; r += 32) {
+          if (r < Mn) continue;
+          ru = __fadd_ru(ru, fmaxf(pre_up[s_base[i] + (int64_t)r * h], 0.0f));
+          rl = __fadd_ru(rl, fmaxf(-pre_lo[s_base[i] + (int64_t)r * h], 0.0f));
+        }
+        ru = warp_dsum<true>(ru);
+        rl = warp_dsum<true>(rl);
+        if (lane == 0) {
+          s_ru[i] = ru;
+          s_rl[i] = rl;
+        }
+      }
+    }
+    int ns = ib;                                     // slabs of the level above
+    for (int m = n - 1; m >= BOT; --m) {
+      const int rows = sh.M[m], sa = sh.stride[m + 1], sb = sh.stride[m];
+      const uint16_t* off = tab + sh.off_tab[m + 1];
+      const int dq = NT / rows, dr = NT - dq * rows;
+      int s = tid / rows, r = tid - s * rows;
+      while (s < ns) {
+        p2 y[R];
+        const int o = off[r];
+        slab_row<LB>(cur + s * sa + o, off[r + 1] - o, y);
+        p2* dst = nxt + (s * R) * sb + r;
+#pragma unroll
+        for (int i = 0; i < R; ++i) dst[i * sb] = y[i];
+        s += dq;
+        r += dr;
+        if (r >= rows) {
+          r -= rows;
+          ++s;
+        }
+      }
+      __syncthreads();
+      p2* t = cur;
+      cur = nxt;
+      nxt = t;
+      ns *= R;
+    }
+    const int per = sh.slabs * R, tasks = ib * per;
+    for (int t0 = 0; t0 < tasks; t0 += NT) {
+      const int t = t0 + tid;
+      const int i = t < tasks ? t / per : -1;
+      float bl = -CUDART_INF_F, bu = -CUDART_INF_F;
+      if (t < tasks) {
+        const p2* slab = cur + t / R * sh.stride[BOT];
+        if constexpr (BOT == 4)
+          fix_all<4, LB>(slab, t % R, s_bin, bl, bu);
+        else
+          tail_max<LB>(slab, t % R, s_bin, bl, bu);
+      }
+      // one update per warp where its lanes share an item
+      const int i_first = __shfl_sync(0xffffffffu, i, 0);
+      if (__all_sync(0xffffffffu, i == i_first || i < 0)) {
+        const int kl = __reduce_max_sync(0xffffffffu, float_key(bl));
+        const int ku = __reduce_max_sync(0xffffffffu, float_key(bu));
+        if (lane == 0 && i >= 0) {
+          atomicMax(&s_bl[i], kl);
+          atomicMax(&s_bu[i], ku);
+        }
+      } else if (i >= 0) {
+        atomicMax(&s_bl[i], float_key(bl));
+        atomicMax(&s_bu[i], float_key(bu));
+      }
+    }
+    __syncthreads();
+    if (tid < ib && s_item[tid] >= 0) {
+      const int64_t it = s_item[tid];
+      const float l = -__fadd_ru(key_float(s_bl[tid]), s_rl[tid]);
+      const float u = __fadd_ru(key_float(s_bu[tid]), s_ru[tid]);
+      lo[it] = l;
+      hi[it] = u;
+      if (!(isfinite(l) && isfinite(u))) atomicOr(status, kStatusNonFinite);
+    }
+  }
+}
+
+// Items per block and shared memory; false where one item does not fit.
+template <int LB, int NT>
+bool expand_shape(int n, ExpandShape* s) {
+  constexpr int R = LB + 1, BOT = expand_bottom<LB>();
+  s->n = n;
+  int64_t tab = 0;
+  for (int m = 0; m <= kMaxVars; ++m) {
+    s->M[m] = m == 0 || m > n ? 1 : (int)num_monomials(m, LB);
+    s->stride[m] = s->M[m] | 1;
+    s->off_tab[m] = (int)tab;
+    if (m >= 4 && m <= n) tab += s->M[m - 1] + 1;
+  }
+  tab = (tab + 3) / 4;                               // pairs
+  if (s->M[n] > 65535) return false;
+  int64_t a = 0, b = 0, slabs = 1;                   // pairs per item: levels n, n-2, ..; n-1, n-3, ..
+  for (int m = n; m >= BOT; --m) {
+    int64_t& x = (n - m) & 1 ? b : a;
+    x = std::max<int64_t>(x, slabs * s->stride[m]);
+    if (m > BOT) slabs *= R;
+    if (slabs > 4096) return false;
+  }
+  s->slabs = (int)slabs;
+  const int64_t fit = (kExpandBytes / (int64_t)sizeof(p2) - tab) / (a + b);
+  if (fit < 1) return false;
+  const int64_t fill = std::max<int64_t>(1, NT / (slabs * R));   // items whose tasks fill the block
+  s->ib = (int)std::min<int64_t>(fit, fill);
+  s->off_a = (int)tab;
+  s->off_b = (int)(tab + s->ib * a);
+  s->total = (int)(tab + s->ib * (a + b));
+  return true;
+}
+
+template <int LB, int NT>
+cudaError_t launch_expand(const Launch& L, const Tables& T, const LexView& X, const ExpandShape& sh,
+                          int64_t n_items, int h, const float* pre_up, const float* pre_lo,
+                          int64_t ld, const int32_t* nterms, float* lo, float* hi, const int* list,
+                          const int* count) {
+  const size_t smem = (size_t)sh.total * sizeof(p2);
+  auto kern = k_enclose_expand<LB, NT>;
+  if (smem > 40 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t need = (n_items + sh.ib - 1) / sh.ib;
+  const int64_t blocks = std::min<int64_t>((int64_t)device_sms(L) * 8, need);
+  kern<<<(unsigned)blocks, NT, smem, L.stream>>>(T, X, sh, T.rscale[LB], n_items, h, pre_up,
+                                                 pre_lo, ld, nterms, lo, hi, list, count,
+                                                 L.status);
+  ++*L.launches;
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 #define BERN_SLAB_CASES                                                                       \
@@ -358,6 +770,25 @@ cudaError_t launch_enclose_slab(const Launch& L, const Tables& T, int lb, int64_
                                 const float* pre_up, const float* pre_lo, int64_t ld,
                                 const int32_t* nterms, float* lo, float* hi, const int* list,
                                 const int* count) {
+  // orders whose levels fit a thread's registers
+#define BERN_REGS(N, X)                                                                        \
+  if (T.n == N && lb == X)                                                                     \
+    return launch_regs<N, X>(L, T, T.lex[X], n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, list, \
+                             count);
+  BERN_REGS(4, 2) BERN_REGS(5, 2) BERN_REGS(6, 2) BERN_REGS(7, 2) BERN_REGS(8, 2)
+  BERN_REGS(4, 3) BERN_REGS(5, 3) BERN_REGS(6, 3) BERN_REGS(4, 4)
+#undef BERN_REGS
+  // the expansion where its levels fit; the slabs above
+#define BERN_EXPAND(X, NT)                                                                     \
+  if (lb == X) {                                                                               \
+    ExpandShape es;                                                                            \
+    if (expand_shape<X, NT>(T.n, &es))                                                         \
+      return launch_expand<X, NT>(L, T, T.lex[X], es, n_items, h, pre_up, pre_lo, ld, nterms,  \
+                                  lo, hi, list, count);                                        \
+  }
+  BERN_EXPAND(2, 128) BERN_EXPAND(3, 128) BERN_EXPAND(4, 128) BERN_EXPAND(5, 128)
+  BERN_EXPAND(6, 256) BERN_EXPAND(7, 256) BERN_EXPAND(8, 256)
+#undef BERN_EXPAND
   switch (lb) {
 #define BERN_SLAB(X, NT) \
   case X: return launch_slab<X, NT>(L, T, T.lex[X], n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, \
