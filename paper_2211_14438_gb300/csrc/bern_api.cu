@@ -81,6 +81,7 @@ struct bern_ctx {
   DevBuf ws, stage_in, stage_out, qbuf, mlp_ws, hbuf;
   DevBuf ctr;                       // box counters of the fused layer kernels
   DevBuf ebuf;                      // grids of enclosures above shared memory
+  DevBuf sqbuf;                     // scaled inputs of the long squares
   DevBuf btnt;                      // term counts of the Bernstein-basis layer sum
   int fused = 0;                    // fused layer kernels where a plan allows them
   std::vector<GraphEntry> graphs;
@@ -264,6 +265,27 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
     if ((e = up(ri.pairs, (const void**)&rt.pairs)) != cudaSuccess) return map_cuda(e);
     if ((e = up(ri.out_ranks, (const void**)&rt.out_ranks)) != cudaSuccess) return map_cuda(e);
   }
+  // squaring units up to the largest degree asked for, or what shared memory
+  // holds
+  ts.view.sqt_dmax = std::max(square_smem_degree(n), std::min(dmax, square_max_degree(n)));
+  for (int D = 0; D <= ts.view.sqt_dmax; ++D) {
+    SquareImage im;
+    if (!build_square_table(n, D, im)) return BERN_E_UNSUPPORTED;
+    // units first: they are read as int4
+    const size_t wu = im.units.size(), wp = im.pos.size(), ww = im.words.size();
+    DevBuf b;
+    if ((e = b.reserve((wu + wp + ww + im.ranks.size() + 4) * sizeof(int32_t))) != cudaSuccess)
+      return map_cuda(e);
+    ts.bufs.push_back(b);
+    int32_t* d = (int32_t*)b.p;
+    cudaMemcpy(d, im.units.data(), wu * sizeof(int32_t), cudaMemcpyHostToDevice);
+    cudaMemcpy(d + wu, im.pos.data(), wp * sizeof(int32_t), cudaMemcpyHostToDevice);
+    cudaMemcpy(d + wu + wp, im.words.data(), ww * sizeof(int32_t), cudaMemcpyHostToDevice);
+    cudaMemcpy(d + wu + wp + ww, im.ranks.data(), im.ranks.size() * sizeof(int32_t),
+               cudaMemcpyHostToDevice);
+    ts.view.sqt[D] = SquareTable{im.m_pad, im.n_units, d + wu, (const int4*)d,
+                                 (const uint32_t*)(d + wu + wp), d + wu + wp + ww};
+  }
   for (int D = 0; D <= dmax; ++D) {
     PairList pl;
     if (!build_square_pairs(n, D, pl)) return BERN_E_UNSUPPORTED;
@@ -351,7 +373,8 @@ int ensure_prod_tables(bern_ctx* c, int n, int Dmax, int dmax, int cap) {
 }
 
 // Composition work queues for up to `items` items.
-int ensure_queues(bern_ctx* c, int64_t items, ComposeScratch* out, size_t horner_floats = 0) {
+int ensure_queues(bern_ctx* c, int64_t items, ComposeScratch* out, size_t horner_floats = 0,
+                  size_t square_bytes = 0) {
   // *out is part of the graph key byte for byte: zero its padding too
   std::memset(out, 0, sizeof *out);
   const size_t bytes = 256 + (size_t)kQueueLists * items * sizeof(int);
@@ -368,6 +391,13 @@ int ensure_queues(bern_ctx* c, int64_t items, ComposeScratch* out, size_t horner
     if ((e = c->hbuf.reserve(horner_floats * sizeof(float))) != cudaSuccess) return map_cuda(e);
     out->hws = (float*)c->hbuf.p;
     out->hws_floats = (int64_t)(c->hbuf.bytes / sizeof(float));
+  }
+  out->tws = nullptr;
+  out->tws_bytes = 0;
+  if (square_bytes) {
+    if ((e = c->sqbuf.reserve(square_bytes)) != cudaSuccess) return map_cuda(e);
+    out->tws = c->sqbuf.p;
+    out->tws_bytes = (int64_t)c->sqbuf.bytes;
   }
   return BERN_OK;
 }
@@ -839,6 +869,7 @@ int bern_destroy(bern_ctx* c) {
   c->hbuf.release();
   c->ctr.release();
   c->ebuf.release();
+  c->sqbuf.release();
   c->btnt.release();
   if (c->d_status) cudaFree(c->d_status);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -1164,7 +1195,11 @@ int bern_compose(bern_ctx* c, int n, int64_t n_boxes, int h, int degree_cap, flo
                                          kHornerGlobalPerSM * std::max(1, c->sms));
   }
   ComposeScratch CS;
-  if ((rc = ensure_queues(c, std::max<int64_t>(1, n_boxes * h), &CS, horner_floats))) return rc;
+  const size_t square_bytes =
+      prune_tau == 0.0f && global_d >= 2 ? square_scratch_bytes(n, Dmax, n_boxes * h) : 0;
+  if ((rc = ensure_queues(c, std::max<int64_t>(1, n_boxes * h), &CS, horner_floats,
+                          square_bytes)))
+    return rc;
   return map_cuda(launch_compose(c->launch(), *T, CS, n_boxes, h, degree_cap, prune_tau, kind,
                                  coef, eps, degrees, global_d, lo, hi, pre_up, pre_lo, pre_ld,
                                  pre_nterms, post_up, post_lo, post_ld, post_nterms));
@@ -1280,7 +1315,11 @@ int bern_propagate_traced(bern_ctx* c, const bern_net* net, const float* boxes,
   int hmax = 1;
   for (const auto& l : P.L) hmax = std::max(hmax, l.h_out);
   ComposeScratch CS;
-  if ((rc = ensure_queues(c, chunk * hmax, &CS, horner_floats))) return rc;
+  size_t square_bytes = 0;
+  for (const auto& l : P.L)
+    if (l.hidden && P.tau == 0.0f && l.d >= 2 && !l.fused)
+      square_bytes = std::max(square_bytes, square_scratch_bytes(P.n, l.D_pre, chunk * l.h_out));
+  if ((rc = ensure_queues(c, chunk * hmax, &CS, horner_floats, square_bytes))) return rc;
 
   // autotune once per plan shape: probe every variant of every tunable kind
   // on the first chunk (plain launches, timed per launch), keep the fastest

@@ -46,7 +46,7 @@ bool build_square_pairs(int n, int D, PairList& out);
 bool build_product_table(int n, int Dq, int Ds, int64_t max_pairs, std::vector<int32_t>& ptr,
                          std::vector<int32_t>& pairs);
 
-// Row decomposition for the squaring kernel.  A "row" is the set of
+// Row decomposition of the fused layer's squares.  A "row" is the set of
 // monomials sharing the exponents of t_1..t_{n-1} (its prefix) and varying
 // the exponent c of t_n.  The square of a degree-D polynomial is, per output
 // row P, the sum over input-row pairs (p, q), p + q = P, of the 1-D
@@ -70,6 +70,47 @@ struct RowImage {
 };
 bool build_row_table(int n, int D, RowImage& out);
 
+// Units of the squaring kernel (k_compose_square.cu).  Input position of a
+// monomial: the tiles (all monomials sharing the exponents of t_1..t_(n-2), a
+// triangle in t_(n-1), t_n, rows of t_n) in graded order of those exponents, every
+// row padded to an even length; in one variable the powers of t_1.
+constexpr int kTileDegree = 5;            // largest degree of an output tile in registers
+constexpr int kSquareSmemTerms = 750;     // inputs held in shared memory, 32 lanes a group
+constexpr int kSquareMaxTerms = 8191;     // 13 bits of positions / 2
+constexpr int64_t kSquareScratchBytes = (int64_t)512 << 20;
+// Offset of row r in a padded triangle of degree d, and its size (r = d + 1):
+// the sum of the even numbers >= d + 1, d, .., d - r + 2.
+__host__ __device__ constexpr int pad_row(int d, int r) {
+  // rows of length L and L - 1 take 2 ceil(L/2) + 2 ceil((L-1)/2) = 2 L
+  const int L = d + 1, h = r / 2;
+  return 2 * h * L - 2 * h * (h - 1) + ((r & 1) ? (L - 2 * h + 1) / 2 * 2 : 0);
+}
+// Dense index 0..14 of a pair of row half lengths 1 <= h1 <= h2 <= 5.
+__host__ __device__ constexpr int row_half_case(int h1, int h2) {
+  return (h1 - 1) * 5 - (h1 - 1) * (h1 - 2) / 2 + (h2 - h1);
+}
+struct SquareImage {
+  int m_in = 0, m_pad = 0, n_units = 0;
+  std::vector<int32_t> pos;        // graded rank -> input position, then the padding's
+  // per unit: first word, end of its words, first output rank, and
+  // (tile: output degree; row: output length) | row << 5 | diagonal pair last
+  // << 6 | (tile: degree + 1, row: length of the input of the same prefix, 0:
+  // none) << 8 | half its position << 16.  Unit 0 holds the constant term, the
+  // others follow by falling cost.
+  std::vector<int32_t> units;
+  std::vector<uint32_t> words;     // half positions of the smaller and the larger part (13
+                                   // bits each), case << 26; tile: the smaller degree; row:
+                                   // row_half_case (diagonal: half length)
+  std::vector<int32_t> ranks;      // graded ranks of the output elements
+};
+bool build_square_table(int n, int D, SquareImage& out);
+int square_padded_terms(int n, int D);
+// Largest degree whose inputs fit the shared-memory / the scratch kernels.
+int square_smem_degree(int n);
+int square_max_degree(int n);
+// Scratch of the long inputs for items of degree <= Dmax (0: none needed).
+size_t square_scratch_bytes(int n, int Dmax, int64_t n_items);
+
 // ------------------------------------------------------------ device views
 struct RowTable {
   int m_in, n_out_rows, row_split;
@@ -78,6 +119,14 @@ struct RowTable {
   const int32_t* in_off;
   const int4* pairs;
   const int32_t* out_ranks;
+};
+
+struct SquareTable {
+  int m_pad, n_units;
+  const int32_t* pos;
+  const int4* units;
+  const uint32_t* words;
+  const int32_t* ranks;
 };
 
 struct PairTable {
@@ -120,9 +169,12 @@ struct Tables {
   // and per (variable k, line) the line's (base offset, prefix digit sum)
   const int32_t* gidx[kMaxEncloseOrder + 1];
   const int2* lines[kMaxEncloseOrder + 1];
-  // row tables for squaring, input degrees 0..row_dmax (row_dmax <= 8)
+  // row tables of the fused layer, input degrees 0..row_dmax (row_dmax <= 8)
   RowTable row[kMaxRowDegree + 1];
   int row_dmax;
+  // units for squaring, input degrees 0..sqt_dmax
+  SquareTable sqt[kMaxRowDegree + 1];
+  int sqt_dmax;
   // product tables of the Horner kernel (device array of kProdStride^2)
   const ProdTable* prod;
   // host array [kSlabMaxOrder + 1] of the slab enclosure's tables by order
@@ -270,6 +322,8 @@ struct ComposeScratch {
   int64_t hws_floats = 0;    // large for shared memory), hws_blocks slices
   int hws_blocks = 0;        // blocks of the global-workspace Horner launch
   int64_t horner_smem_limit = 200 * 1024;   // bytes of shared memory before hws is used
+  void* tws = nullptr;       // scratch of the long squares (null: they take the pair lists)
+  int64_t tws_bytes = 0;
 };
 // Blocks of the global-workspace Horner launch: two per multiprocessor.
 constexpr int kHornerGlobalPerSM = 2;

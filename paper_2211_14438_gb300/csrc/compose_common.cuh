@@ -9,7 +9,7 @@ namespace bern {
 constexpr float kU = 0x1p-24f;   // unit roundoff of float32
 constexpr int kQIdent = kMaxRowDegree + 1;   // identity copies
 constexpr int kQLinear = kMaxRowDegree + 2;  // order-1 items
-constexpr int kQPairs = kMaxRowDegree + 3;   // order-2 items outside the row path
+constexpr int kQPairs = kMaxRowDegree + 3;   // order-2 items outside the squaring kernels
 constexpr int kQHorner = kMaxRowDegree + 4;  // Horner items in float32 (order >= 3, or pruning)
 constexpr int kQHorner64 = kMaxRowDegree + 5;  // Horner items in float64 (order >= kHornerF64Order)
 static_assert(kQHorner64 + 1 == kComposeQueues, "queue ids");
@@ -54,6 +54,11 @@ __device__ __forceinline__ int degree_of(const Tables& T, int m) {
   while (D < kMaxTableDegree && T.mcount[D] < m) ++D;
   return D;
 }
+
+// The squaring kernels (k_compose_square.cu) over queues 0..min(Dmax, degrees
+// that fit): order-2 items by input degree.
+cudaError_t launch_compose_square(const Launch& L, const Tables& T, const ComposeScratch& S,
+                                  const ComposeArgs& A, int64_t n_items, int Dmax);
 
 // The Horner kernels (k_horner.cu) over queues kQHorner (float32) and
 // kQHorner64 (float64), for inputs of degree <= Dmax, ReLU orders <= d and

@@ -20,12 +20,12 @@
 // Work layout.  A classification kernel puts each item (box, neuron) into a
 // queue: zero items only get a term count of 0; identity items and order-1
 // items go to an elementwise kernel; order-2 items of input degree D <= 8 go
-// to queue D of the row-convolution kernel (one lane per item, 32 items of
-// equal structure per warp), the rest to a per-item pair-list kernel.
+// to queue D of the squaring kernels (k_compose_square.cu: one lane per item,
+// 32 items of equal structure per warp), the rest to a per-item pair-list
+// kernel.
 #include <algorithm>
 
 #include "compose_common.cuh"
-#include "row_conv.cuh"
 
 namespace bern {
 
@@ -36,7 +36,7 @@ namespace bern {
 // of sorted runs, and a warp's 32 consecutive entries are mostly neighbouring
 // neurons of one box.
 __global__ void __launch_bounds__(1024)
-k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int row_dmax, ComposeScratch S,
+k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int sq_dmax, ComposeScratch S,
                 int* status) {
   __shared__ int s_wcnt[32][kComposeQueues];
   __shared__ int s_base[kComposeQueues];
@@ -71,7 +71,7 @@ k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int row_dmax, ComposeS
         } else if (d == 1) {
           q = kQLinear;
           nt = Mout;
-        } else if (D <= row_dmax) {
+        } else if (D <= sq_dmax) {
           q = D;
           nt = Mout;
         } else if (D <= T.dmax) {
@@ -103,169 +103,6 @@ k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int row_dmax, ComposeS
   }
   __syncthreads();
   if (q >= 0) S.queue[(int64_t)q * S.qcap + s_base[q] + s_wcnt[warp][q] + rank_in_warp] = (int)item;
-}
-
-// ------------------------------------------------------------ row convolution
-constexpr int kRowWarps = 4;    // warps sharing one 32-item group
-constexpr int kRowBlocks = 8;   // resident blocks per SM (registers and shared memory)
-
-// Load one bound of the 32 items of a lane group into row layout:
-// s = (pre - lo*[K=0]) / (hi - lo) in round-to-nearest; returns this warp's
-// share of sum|s| (rounded up).  Warp `half` (of kRowWarps) takes every
-// kRowWarps-th group
-// of 8 input monomials.
-__device__ float load_rows(const ComposeArgs& A, const RowTable& R, const float* P, int Mpre,
-                           float Lo, float inv, int half, float* s) {
-  const int h = A.h;
-  float l1 = 0.0f;
-  for (int r0 = 8 * half; r0 < R.m_in; r0 += 8 * kRowWarps) {
-    float v[8];
-    int pos[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = r0 + i;
-      v[i] = r < Mpre ? __ldg(P + (int64_t)r * h) : 0.0f;
-      pos[i] = r < R.m_in ? __ldg(R.pos_in + r) : -1;
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (pos[i] < 0) continue;
-      float x = v[i];
-      if (r0 + i == 0) x = __fsub_rn(x, Lo);
-      x = __fmul_rn(x, inv);
-      s[pos[i]] = x;
-      l1 = __fadd_ru(l1, fabsf(x));
-    }
-  }
-  return l1;
-}
-
-// Output rows [row_b, row_e) of one bound (UP: upper polynomial) of the
-// items of a warp: per row, the row-pair convolutions, then the coefficients
-// a1*s + a2*s^2 of the row's monomials (the constant term only in c0).
-template <bool UP>
-__device__ void rows_range(const Tables& T, const ComposeArgs& A, const RowTable& R, int D,
-                           int row_b, int row_e, int row_step, bool valid, float a1, float a2,
-                           const float* s, float* Q, float* c0_out, float* rem_out) {
-  const int h = A.h;
-  const int Mout = T.mcount[min(2 * D, A.cap)];
-  const bool no_trunc = 2 * D <= A.cap;   // every output monomial is kept
-  float rem = 0.0f;
-  for (int row = row_b; row < row_e; row += row_step) {
-    const int4 hd = __ldg(R.hdr + row);
-    const int Lout = hd.w & 0xff, in_len = (hd.w >> 8) & 0xff;
-    const int in_off = __ldg(R.in_off + row);
-    float acc[2 * kRowLen - 1];
-#pragma unroll
-    for (int c = 0; c < 2 * kRowLen - 1; ++c) acc[c] = 0.0f;
-    const int has_diag = (hd.w >> 16) & 1;
-    const int off_end = hd.y - has_diag;
-    if (hd.x < off_end) {
-      int4 pr = __ldg(R.pairs + hd.x);
-      for (int k = hd.x; k < off_end; ++k) {
-        const int4 nx = k + 1 < off_end ? __ldg(R.pairs + k + 1) : pr;   // prefetch
-        switch (pr.w) {
-          BERN_CONV_ALL_CASES
-          default: break;
-        }
-        pr = nx;
-      }
-    }
-    if (has_diag) {
-      const int4 pr = __ldg(R.pairs + off_end);
-      switch (pr.z & 15) {
-        BERN_DIAG_CASES
-        default: break;
-      }
-    }
-    const int* __restrict__ rk = R.out_ranks + hd.z;   // the row's output ranks
-#pragma unroll
-    for (int c = 0; c < 2 * kRowLen - 1; ++c) {
-      if (c >= Lout) break;
-      const float sq = acc[c];            // (s^2)_K, directed
-      const float lin = c < in_len ? s[in_off + c] : 0.0f;
-      const float v = dfma<UP>(a2, sq, UP ? __fmul_ru(a1, lin) : __fmul_rd(a1, lin));
-      if (row == 0 && c == 0) {
-        *c0_out = v;                      // the constant term is finished by the caller
-      } else if (no_trunc || __ldg(rk + c) < Mout) {
-        if (valid) Q[(int64_t)__ldg(rk + c) * h] = v;
-      } else {
-        rem = UP ? __fadd_ru(rem, fmaxf(v, 0.0f)) : __fadd_rd(rem, fminf(v, 0.0f));
-      }
-    }
-  }
-  *rem_out = rem;
-}
-
-// A block of kRowWarps warps squares one bound (UP: upper) of 32 queued items
-// (one lane per item); the warps share the items' inputs in shared memory and
-// take the output rows in turn.
-template <bool UP>
-__global__ void __launch_bounds__(32 * kRowWarps, kRowBlocks)
-k_compose_rows(Tables T, ComposeArgs A, ComposeScratch S, int row_dmax, int sstride,
-               int* status) {
-  extern __shared__ float smem[];
-  __shared__ float s_l1[kRowWarps][32], s_rem[kRowWarps][32], s_c0[32];
-  const int lane = threadIdx.x & 31, half = threadIdx.x >> 5;
-  float* s = smem + (size_t)lane * sstride;
-  for (int task = blockIdx.x;; task += gridDim.x) {
-    int D = -1, chunk = task;
-    for (int d = 0; d <= row_dmax; ++d) {
-      const int nc = (S.qcount[d] + 31) >> 5;
-      if (chunk < nc) {
-        D = d;
-        break;
-      }
-      chunk -= nc;
-    }
-    if (D < 0) break;
-    const int idx = chunk * 32 + lane;
-    const bool valid = idx < S.qcount[D];
-    const int64_t item = valid ? S.queue[(int64_t)D * S.qcap + idx] : 0;
-    const RowTable R = T.row[D];
-    const float Lo = valid ? A.lo[item] : -1.0f;
-    const float Hi = valid ? A.hi[item] : 1.0f;
-    const float inv = 1.0f / (Hi - Lo);
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
-    if (valid) {
-      const float* cf = A.coef + item * kCoefStride;
-      a0 = cf[0];
-      a1 = cf[1];
-      a2 = cf[2];
-      if (a2 < 0.0f) atomicOr(status, kStatusUnsupported);   // excluded by convexity
-    }
-    const int Mpre = valid ? A.pre_nterms[item] : 0;
-    const float* P = (UP ? A.pre_up : A.pre_lo) + A.base(valid ? item : 0, A.pre_ld);
-    s_l1[half][lane] = load_rows(A, R, P, Mpre, Lo, inv, half, s);
-    __syncthreads();
-    float* Q = (UP ? A.post_up : A.post_lo) + A.base(valid ? item : 0, A.post_ld);
-    float c0 = 0.0f, rem = 0.0f;
-    rows_range<UP>(T, A, R, D, half, R.n_out_rows, kRowWarps, valid, a1, a2, s, Q, &c0, &rem);
-    s_rem[half][lane] = rem;
-    if (!half) s_c0[lane] = c0;
-    __syncthreads();
-    if (!half && valid) {
-      // constant term: a0 + (the row-0 value without a0) + Lip*eta + remainder
-      float l1 = s_l1[0][lane], remt = s_rem[0][lane];
-#pragma unroll
-      for (int w = 1; w < kRowWarps; ++w) {
-        l1 = __fadd_ru(l1, s_l1[w][lane]);
-        remt = UP ? __fadd_ru(remt, s_rem[w][lane]) : __fadd_rd(remt, s_rem[w][lane]);
-      }
-      const float eta = __fmul_ru(5.0f * kU, l1);
-      const float lip = __fmaf_ru(2.0f * a2, __fadd_ru(1.0f, eta), fabsf(a1));
-      float v;
-      if (UP) {
-        v = __fadd_ru(__fadd_ru(__fadd_ru(s_c0[lane], a0), __fmul_ru(lip, eta)), remt);
-      } else {
-        v = __fsub_rd(__fadd_rd(s_c0[lane], a0), __fmul_ru(lip, eta));
-        v = __fadd_rd(__fsub_rd(v, A.eps[item]), remt);
-      }
-      Q[0] = v;
-      if (!isfinite(v)) atomicOr(status, kStatusNonFinite);
-    }
-    __syncthreads();   // the next task reuses the shared inputs
-  }
 }
 
 // ------------------------------------------------------------ elementwise items
@@ -364,7 +201,7 @@ k_compose_linear(ComposeArgs A, ComposeScratch S, int* status) {
 }
 
 // ------------------------------------------------------------ pair-list squaring
-// Order-2 items outside the row path: one block per item, threads over output
+// Order-2 items outside the squaring kernels: one block per item, threads over output
 // monomials, symmetric pair lists (I <= J, I + J = K) from the host tables.
 __global__ void __launch_bounds__(256)
 k_compose_pairs(Tables T, ComposeArgs A, ComposeScratch S, int* status) {
@@ -484,36 +321,20 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
   while (Dmax < kMaxTableDegree && num_monomials(T.n, Dmax + 1) >= 0 &&
          num_monomials(T.n, Dmax + 1) <= pre_cap)
     ++Dmax;
-  const int row_dmax = std::min(std::min(T.row_dmax, row_path_max_degree(T.n)), Dmax);
+  // long inputs take the squaring kernels where the caller gave them a scratch
+  const int sq_dmax = std::min(std::min(T.sqt_dmax, Dmax),
+                               S.tws ? square_max_degree(T.n) : square_smem_degree(T.n));
   cudaError_t e = cudaMemsetAsync(S.qcount, 0, kComposeQueues * sizeof(int), L.stream);
   if (e != cudaSuccess) return e;
   k_compose_queue<<<(unsigned)((n_items + 1023) / 1024), 1024, 0, L.stream>>>(
-      T, A, n_items, row_dmax, S, L.status);
+      T, A, n_items, sq_dmax, S, L.status);
   ++*L.launches;
   // order-2 items exist only with order 2 somewhere in the plan (with pruning
   // they go to the Horner kernel)
   const bool order2 = tau == 0.0f && (degrees != nullptr || global_d == 2);
-  // row-convolution kernels (one per bound): persistent blocks of 2 warps
-  // per 32 items; the per-lane stride is odd so that lanes reading the same
-  // offset hit distinct banks
-  const int sstride = (int)num_monomials(T.n, row_dmax) | 1;
-  const size_t smem = (size_t)32 * sstride * sizeof(float);
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_compose_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_compose_rows<false>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  const int64_t tasks = n_items / 32 + row_dmax + 1;
-  const int blocks = (int)std::min<int64_t>(tasks, device_sms(L) * kRowBlocks);
   if (order2) {
-    k_compose_rows<true><<<blocks, 32 * kRowWarps, smem, L.stream>>>(T, A, S, row_dmax, sstride,
-                                                                     L.status);
-    k_compose_rows<false><<<blocks, 32 * kRowWarps, smem, L.stream>>>(T, A, S, row_dmax,
-                                                                      sstride, L.status);
-    *L.launches += 2;
+    e = launch_compose_square(L, T, S, A, n_items, sq_dmax);
+    if (e != cudaSuccess) return e;
   }
   if (!in_place) {   // in place, an identity item's outputs are its inputs
     k_compose_copy<<<(unsigned)std::min<int64_t>((n_items + 31) / 32, device_sms(L) * 16), 256, 0,
@@ -527,8 +348,8 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
                        0, L.stream>>>(A, S, L.status);
     ++*L.launches;
   }
-  // pair-list kernel for order-2 items beyond the row path
-  if (order2 && Dmax > row_dmax) {
+  // pair-list kernel for order-2 items beyond the squaring kernels
+  if (order2 && Dmax > sq_dmax) {
     const size_t psmem = 2 * (size_t)pre_cap * sizeof(float);
     if (psmem > 200 * 1024) return cudaErrorInvalidValue;
     if (psmem > 48 * 1024) {

@@ -110,20 +110,18 @@ int upload_tables(DeviceSlot& s, int n, int dmax, int deg_exps, cudaStream_t str
     off_li[l] = put(li.data(), li.size() * sizeof(int32_t));
     if (img.size() > kNoAllocTableBytes) return BERN_E_UNSUPPORTED;
   }
-  const int row_dmax = std::min(bern::kMaxRowDegree, bern::row_path_max_degree(n));
-  struct RowOff { size_t pos_in, hdr, in_off, pairs, out_ranks; int m_in, n_out_rows, row_split; };
-  std::vector<RowOff> roff(row_dmax + 1);
-  for (int D = 0; D <= row_dmax; ++D) {
-    bern::RowImage ri;
-    if (!bern::build_row_table(n, D, ri)) return BERN_E_UNSUPPORTED;
-    roff[D].m_in = ri.m_in;
-    roff[D].n_out_rows = ri.n_out_rows;
-    roff[D].row_split = ri.row_split;
-    roff[D].pos_in = put(ri.pos_in.data(), ri.pos_in.size() * sizeof(int32_t));
-    roff[D].hdr = put(ri.hdr.data(), ri.hdr.size() * sizeof(int32_t));
-    roff[D].in_off = put(ri.in_off.data(), ri.in_off.size() * sizeof(int32_t));
-    roff[D].pairs = put(ri.pairs.data(), ri.pairs.size() * sizeof(int32_t));
-    roff[D].out_ranks = put(ri.out_ranks.data(), ri.out_ranks.size() * sizeof(int32_t));
+  const int sqt_dmax = bern::square_smem_degree(n);
+  struct SqOff { size_t units, pos, words, ranks; int m_pad, n_units; };
+  std::vector<SqOff> soff(sqt_dmax + 1);
+  for (int D = 0; D <= sqt_dmax; ++D) {
+    bern::SquareImage im;
+    if (!bern::build_square_table(n, D, im)) return BERN_E_UNSUPPORTED;
+    soff[D].m_pad = im.m_pad;
+    soff[D].n_units = im.n_units;
+    soff[D].units = put(im.units.data(), im.units.size() * sizeof(int32_t));
+    soff[D].pos = put(im.pos.data(), im.pos.size() * sizeof(int32_t));
+    soff[D].words = put(im.words.data(), im.words.size() * sizeof(uint32_t));
+    soff[D].ranks = put(im.ranks.data(), im.ranks.size() * sizeof(int32_t));
     if (img.size() > kNoAllocTableBytes) return BERN_E_UNSUPPORTED;
   }
   std::vector<size_t> off_ptr(dmax + 1), off_pairs(dmax + 1);
@@ -151,18 +149,13 @@ int upload_tables(DeviceSlot& s, int n, int dmax, int deg_exps, cudaStream_t str
   v.exps = (const uint8_t*)(s.tables + off_ex);
   v.mexps = bern::num_monomials(n, deg_exps);
   v.deg_of = (const uint8_t*)(s.tables + off_dof);
-  v.row_dmax = row_dmax;
-  for (int D = 0; D <= row_dmax; ++D) {
-    bern::RowTable& rt = v.row[D];
-    rt.m_in = roff[D].m_in;
-    rt.n_out_rows = roff[D].n_out_rows;
-    rt.row_split = roff[D].row_split;
-    rt.pos_in = (const int32_t*)(s.tables + roff[D].pos_in);
-    rt.hdr = (const int4*)(s.tables + roff[D].hdr);
-    rt.in_off = (const int32_t*)(s.tables + roff[D].in_off);
-    rt.pairs = (const int4*)(s.tables + roff[D].pairs);
-    rt.out_ranks = (const int32_t*)(s.tables + roff[D].out_ranks);
-  }
+  v.sqt_dmax = sqt_dmax;
+  for (int D = 0; D <= sqt_dmax; ++D)
+    v.sqt[D] = bern::SquareTable{soff[D].m_pad, soff[D].n_units,
+                                 (const int32_t*)(s.tables + soff[D].pos),
+                                 (const int4*)(s.tables + soff[D].units),
+                                 (const uint32_t*)(s.tables + soff[D].words),
+                                 (const int32_t*)(s.tables + soff[D].ranks)};
   v.rscale_max = rmax;
   for (int l = 0; l <= rmax; ++l) {
     v.rscale[l] = (const float2*)(s.tables + off_rs[l]);
@@ -182,7 +175,9 @@ int upload_tables(DeviceSlot& s, int n, int dmax, int deg_exps, cudaStream_t str
 // Bytes of the table image upload_tables would build, from the monomial
 // counts alone (every table's length is fixed by n and the degrees), so that
 // a plan whose tables cannot fit is rejected before any of them is built.
-// Returns SIZE_MAX when a count overflows.
+// The squaring entry is that of row tables, which the units that are stored
+// never exceed: plans are accepted and refused by it.  Returns SIZE_MAX when a
+// count overflows.
 size_t table_image_bytes(int n, int dmax, int deg_exps) {
   size_t total = 0;
   bool bad = false;

@@ -3,6 +3,8 @@
 // "Prod" of Sec. 4.2, here over a shared dense graded monomial set).
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <tuple>
 #include <unordered_map>
 
 #include "bern_internal.cuh"
@@ -113,6 +115,12 @@ bool build_product_table(int n, int Dq, int Ds, int64_t max_pairs, std::vector<i
   return true;
 }
 
+// Order of the tile pairs of a square: by the degrees d1 <= d2, a tile with
+// itself last.
+static int tile_pair_order(int d1, int d2, bool same) {
+  return same ? 1 << 20 : d1 * (kMaxRowDegree + 1) + d2;
+}
+
 bool build_row_table(int n, int D, RowImage& out) {
   out = RowImage{};
   if (D < 0 || D > kMaxRowDegree) return false;
@@ -166,6 +174,43 @@ bool build_row_table(int n, int D, RowImage& out) {
         k = pack_key(&pre[(size_t)i * (n - 1)], n - 1) + pack_key(&pre[(size_t)j * (n - 1)], n - 1);
       bucket[pidx.at(k)].push_back(i * np_in + j);
     }
+  // Within an output row the pairs follow the order of the squaring kernel's
+  // tiles (build_square_table): by the tiles (the exponents but the last two) of
+  // the two rows, T1 the smaller one, then by the row of T1, which is also the
+  // first row of a pair of equal lengths.
+  std::vector<int> tile(np_in, 0), tdeg(np_in, D), trow(np_in, 0);
+  if (n >= 3) {
+    std::vector<uint8_t> tp;
+    graded_monomials(n - 2, D, tp);
+    std::unordered_map<uint64_t, int32_t> tidx;
+    for (int64_t i = 0; i < num_monomials(n - 2, D); ++i)
+      tidx[pack_key(&tp[(size_t)i * (n - 2)], n - 2)] = (int32_t)i;
+    for (int i = 0; i < np_in; ++i) tile[i] = tidx.at(pack_key(&pre[(size_t)i * (n - 1)], n - 2));
+  }
+  if (n >= 2)
+    for (int i = 0; i < np_in; ++i) {
+      trow[i] = pre[(size_t)i * (n - 1) + n - 2];
+      tdeg[i] = D - (psum(i) - trow[i]);
+    }
+  // the pair (row of T1, row of T2)
+  auto oriented = [&](int code) {
+    const int i = code / np_in, j = code % np_in;
+    const bool sw = tile[i] == tile[j] ? trow[i] > trow[j]
+                    : tdeg[i] != tdeg[j] ? tdeg[i] > tdeg[j]
+                                         : tile[i] > tile[j];
+    return sw ? std::make_pair(j, i) : std::make_pair(i, j);
+  };
+  for (auto& v : bucket)
+    std::stable_sort(v.begin(), v.end(), [&](int a, int b) {
+      const auto x = oriented(a), y = oriented(b);
+      auto rank_of_pair = [&](const std::pair<int, int>& p) {
+        return std::make_tuple(
+            tile_pair_order(tdeg[p.first], tdeg[p.second], tile[p.first] == tile[p.second]),
+            std::min(tile[p.first], tile[p.second]), std::max(tile[p.first], tile[p.second]),
+            trow[p.first]);
+      };
+      return rank_of_pair(x) < rank_of_pair(y);
+    });
   out.n_out_rows = np;
   out.m_in = (int)m_in;
   for (int P = 0; P < np; ++P) {
@@ -176,7 +221,7 @@ bool build_row_table(int n, int D, RowImage& out) {
     int has_diag = 0;
     for (int pass = 0; pass < 2; ++pass)
       for (int code : bucket[P]) {
-        const int i = code / np_in, j = code % np_in;
+        const int i = oriented(code).first, j = oriented(code).second;
         if ((i == j) != (pass == 1)) continue;
         has_diag |= (i == j);
         int oi = off[i], oj = off[j], li = len[i], lj = len[j];
@@ -284,6 +329,179 @@ void build_rscale(int n, int l, std::vector<float>& out) {
     out[(size_t)r * 2] = lo;
     out[(size_t)r * 2 + 1] = hi;
   }
+}
+
+int square_padded_terms(int n, int D) {
+  if (n == 1) return (D + 2) / 2 * 2;
+  int64_t total = 0;
+  for (int s = 0; s <= D; ++s) {             // tiles of degree D - s
+    const int64_t upto = n == 2 ? 1 : num_monomials(n - 2, s);
+    const int64_t below = s == 0 ? 0 : (n == 2 ? 1 : num_monomials(n - 2, s - 1));
+    total += (upto - below) * pad_row(D - s, D - s + 1);
+  }
+  return (int)total;
+}
+
+bool build_square_table(int n, int D, SquareImage& out) {
+  out = SquareImage{};
+  if (D < 0 || D > kMaxRowDegree || n < 1) return false;
+  const int64_t m_in = num_monomials(n, D), m_full = num_monomials(n, 2 * D);
+  if (m_in < 0 || m_in > kSquareMaxTerms || m_full < 0) return false;
+  const int m = n - 2;                     // variables of a prefix (one variable: none)
+  const int inner = n == 1 ? 1 : 2;
+  std::vector<uint8_t> pre;
+  int np = 1, np_in = 1;
+  if (m >= 1) {
+    graded_monomials(m, 2 * D, pre);
+    np = (int)num_monomials(m, 2 * D);
+    np_in = (int)num_monomials(m, D);
+  }
+  std::vector<int> deg(np, 0);
+  for (int i = 0; i < np; ++i)
+    for (int k = 0; k < m; ++k) deg[i] += pre[(size_t)i * m + k];
+  // graded ranks by exponents
+  std::vector<uint8_t> ex;
+  graded_monomials(n, 2 * D, ex);
+  std::unordered_map<uint64_t, int32_t> rank;
+  rank.reserve((size_t)m_full * 2);
+  for (int64_t r = 0; r < m_full; ++r) rank[pack_key(&ex[(size_t)r * n], n)] = (int32_t)r;
+  auto rank_of = [&](int P, int r, int c) {
+    uint8_t e[kMaxVars] = {0};
+    for (int k = 0; k < m; ++k) e[k] = pre[(size_t)P * m + k];
+    if (inner == 2) e[n - 2] = (uint8_t)r;
+    e[n - 1] = (uint8_t)c;
+    return rank.at(pack_key(e, n));
+  };
+  // input positions
+  std::vector<int> off(np_in);
+  std::vector<int32_t> padding;
+  out.pos.assign((size_t)m_in, -1);
+  int at = 0;
+  for (int P = 0; P < np_in; ++P) {
+    const int d = D - deg[P];
+    off[P] = at;
+    for (int r = 0; r <= (inner == 2 ? d : 0); ++r) {
+      for (int c = 0; c <= d - r; ++c) out.pos[rank_of(P, r, c)] = at++;
+      if (at & 1) padding.push_back(at++);
+    }
+  }
+  if (at != square_padded_terms(n, D) || at / 2 > 0x1fff) return false;
+  out.pos.insert(out.pos.end(), padding.begin(), padding.end());
+  // pairs of input prefixes by output prefix
+  std::unordered_map<uint64_t, int32_t> index;
+  auto key = [&](int i) { return m >= 1 ? pack_key(&pre[(size_t)i * m], m) : (uint64_t)0; };
+  index.reserve((size_t)np * 2);
+  for (int i = 0; i < np; ++i) index[key(i)] = i;
+  // (T1, T2): T1 of the smaller degree (equal: the earlier), by the pair's
+  // degrees, a tile with itself last; every sum below follows this order, the
+  // row tables' too (build_row_table)
+  std::vector<std::vector<std::pair<int, int>>> pairs(np);
+  for (int i = 0; i < np_in; ++i)
+    for (int j = i; j < np_in; ++j) {
+      const bool sw = deg[i] < deg[j];     // a smaller exponent sum: a larger tile
+      pairs[index.at(key(i) + key(j))].push_back(sw ? std::make_pair(j, i) : std::make_pair(i, j));
+    }
+  for (auto& v : pairs)
+    std::stable_sort(v.begin(), v.end(), [&](const std::pair<int, int>& a, const std::pair<int, int>& b) {
+      return tile_pair_order(D - deg[a.first], D - deg[a.second], a.first == a.second) <
+             tile_pair_order(D - deg[b.first], D - deg[b.second], b.first == b.second);
+    });
+  struct Unit {
+    int64_t cost;
+    int Q, r;                              // r < 0: a tile
+  };
+  std::vector<Unit> list;
+  for (int Q = 0; Q < np; ++Q) {
+    const int e = 2 * D - deg[Q];
+    if (inner == 2 && e <= kTileDegree) {
+      int64_t cost = 12 * (int64_t)((e + 1) * (e + 2) / 2);
+      for (const auto& p : pairs[Q]) {
+        const int a = D - deg[p.first], b = D - deg[p.second];
+        cost += (int64_t)((a + 1) * (a + 2) / 2) * ((b + 1) * (b + 2) / 2) + 12;
+      }
+      list.push_back({cost, Q, -1});
+    } else {
+      for (int r = 0; r <= (inner == 2 ? e : 0); ++r) {
+        int64_t cost = 12 * (int64_t)(e - r + 1);
+        for (const auto& p : pairs[Q])
+          for (int a = 0; a <= r; ++a) {
+            const int l1 = D - deg[p.first] - a + 1, l2 = D - deg[p.second] - (r - a) + 1;
+            if (l1 > 0 && l2 > 0) cost += l1 * l2 + 12;
+          }
+        list.push_back({cost, Q, r});
+      }
+    }
+  }
+  // the unit of the constant first, the others by falling cost
+  std::stable_sort(list.begin() + 1, list.end(),
+                   [](const Unit& x, const Unit& y) { return x.cost > y.cost; });
+  for (const Unit& un : list) {
+    const int Q = un.Q, e = 2 * D - deg[Q];
+    std::vector<uint32_t> words;
+    uint32_t diag = 0;
+    bool has_diag = false;
+    auto word = [&](int o1, int s1, int o2, int s2, bool tile) {
+      if (s1 > s2) {
+        std::swap(o1, o2);
+        std::swap(s1, s2);
+      }
+      const int c = tile ? s1 : row_half_case((s1 + 1) / 2, (s2 + 1) / 2);
+      words.push_back((uint32_t)o1 / 2 | (uint32_t)o2 / 2 << 13 | (uint32_t)c << 26);
+    };
+    const int rank0 = (int)out.ranks.size();
+    int size, in_n = 0, in_off = 0;
+    if (un.r < 0) {
+      for (const auto& p : pairs[Q]) {
+        const int d1 = D - deg[p.first], d2 = D - deg[p.second];
+        if (p.first == p.second) {
+          has_diag = true;
+          diag = (uint32_t)off[p.first] / 2 | (uint32_t)d1 << 26;
+        } else {
+          word(off[p.first], d1, off[p.second], d2, true);
+        }
+      }
+      size = e;
+      if (Q < np_in) {
+        in_n = D - deg[Q] + 1;
+        in_off = off[Q];
+      }
+      for (int r = 0; r <= e; ++r)
+        for (int c = 0; c <= e - r; ++c) out.ranks.push_back(rank_of(Q, r, c));
+    } else {
+      for (const auto& p : pairs[Q]) {
+        const int d1 = D - deg[p.first], d2 = D - deg[p.second];
+        for (int a = 0; a <= un.r; ++a) {
+          const int b = un.r - a;
+          if (a > d1 || b > d2) continue;
+          if (p.first == p.second && a > b) continue;
+          const int o1 = off[p.first] + pad_row(d1, a), o2 = off[p.second] + pad_row(d2, b);
+          if (p.first == p.second && a == b) {
+            has_diag = true;
+            diag = (uint32_t)o1 / 2 | (uint32_t)(d1 - a + 2) / 2 << 26;
+          } else {
+            word(o1, d1 - a + 1, o2, d2 - b + 1, false);
+          }
+        }
+      }
+      size = e - un.r + 1;
+      if (Q < np_in && un.r <= D - deg[Q]) {
+        in_n = D - deg[Q] - un.r + 1;
+        in_off = off[Q] + pad_row(D - deg[Q], un.r);
+      }
+      for (int c = 0; c < size; ++c) out.ranks.push_back(rank_of(Q, un.r, c));
+    }
+    out.units.push_back((int32_t)out.words.size());
+    out.words.insert(out.words.end(), words.begin(), words.end());
+    if (has_diag) out.words.push_back(diag);
+    out.units.push_back((int32_t)out.words.size());
+    out.units.push_back(rank0);
+    out.units.push_back(size | (un.r < 0 ? 0 : 1) << 5 | (has_diag ? 1 : 0) << 6 | in_n << 8 |
+                        in_off / 2 << 16);
+  }
+  out.m_in = (int)m_in;
+  out.m_pad = at;
+  out.n_units = (int)list.size();
+  return true;
 }
 
 // Lexicographic exponents of total degree <= l in m variables.
