@@ -7,10 +7,12 @@
 // Backward:  p = softmax(z),  dz_c = w (p_c - [c = y]),
 //   dW2_cj = sum_s dz_c a_j,  db2_c = sum_s dz_c,
 //   dz1_j = [z1_j > 0] sum_c W2_cj dz_c,  dW1_jf = sum_s dz1_j xb_f,  db1_j = sum_s dz1_j,
-// all divided by n.  Per-sample terms go to scratch; a second kernel sums
-// them per parameter over fixed chunks of samples and a third adds the chunk
-// partials in chunk order, so the result does not depend on scheduling.
+// all divided by n.  A block keeps the sums of its tiles of samples in registers
+// (per-sample terms live in shared memory only); a second kernel adds the blocks'
+// sums in block order, so the result does not depend on scheduling.
 #include <math.h>
+
+#include <algorithm>
 
 #include "device_util.cuh"
 #include "enclose_impl.cuh"
@@ -21,7 +23,6 @@ namespace bern {
 namespace {
 
 constexpr int kH = kMlpHidden;
-constexpr int kChunk = 1024;   // samples per partial sum
 
 struct SmemMlp {
   float W1[kH * kMlpMaxF];     // [j][f], zero-padded to kMlpMaxF
@@ -53,14 +54,12 @@ __device__ __forceinline__ float hidden_pre(const SmemMlp& S, int j, const float
   return acc;
 }
 
-// Logits of one sample; optionally stores the bf16 activations.
-__device__ void mlp_logits(const SmemMlp& S, const float (&xb)[kMlpMaxF], float (&z)[kMlpMaxC],
-                           __nv_bfloat16* a_out) {
+// Logits of one sample.
+__device__ void mlp_logits(const SmemMlp& S, const float (&xb)[kMlpMaxF], float (&z)[kMlpMaxC]) {
 #pragma unroll
   for (int c = 0; c < kMlpMaxC; ++c) z[c] = S.b2[c];
   for (int j = 0; j < kH; ++j) {
     const float a = bf16_round(fmaxf(hidden_pre(S, j, xb), 0.0f));
-    if (a_out) a_out[j] = __float2bfloat16_rn(a);
 #pragma unroll
     for (int c = 0; c < kMlpMaxC; ++c) z[c] = fmaf(S.W2[c * kH + j], a, z[c]);
   }
@@ -106,7 +105,7 @@ k_learned_degrees(MlpView M, int64_t n_boxes, int h, int layer, const float* __r
       degree_feature_vec(l, u, pre_nterms[it], layer, f);
 #pragma unroll
       for (int k = 0; k < kMlpMaxF; ++k) xb[k] = k < kDegFeatures ? bf16_round(f[k]) : 0.0f;
-      mlp_logits(S, xb, z, nullptr);
+      mlp_logits(S, xb, z);
       int best = 0;
       float zb = z[0];
 #pragma unroll
@@ -146,127 +145,198 @@ k_mlp_forward(MlpView M, int64_t n, const float* __restrict__ x, float* __restri
        s += (int64_t)gridDim.x * blockDim.x) {
     float xb[kMlpMaxF], z[kMlpMaxC];
     load_features(x, M.F, s, xb);
-    mlp_logits(S, xb, z, nullptr);
+    mlp_logits(S, xb, z);
 #pragma unroll
     for (int c = 0; c < kMlpMaxC; ++c)
       if (c < M.C) logits[s * M.C + c] = z[c];
   }
 }
 
-struct BackScratch {
-  float* dz1;            // [n][H]
-  __nv_bfloat16* a;      // [n][H]
-  float* dz2;            // [n][C]
-  float* loss;           // [n]
-  float* partial;        // [chunks][P + 1]
-};
+// Backward: a block takes tiles of kTile samples in turn.  First four lanes share
+// a sample (lane part p has the hidden units 4 i + p) and leave the tile's
+// activations, hidden and logit gradients in shared memory, one row per unit;
+// then thread (j, p) adds the tile to its parameters: W1[j][f] of a quarter of
+// the features, W2[c][j] of c = p, p + 4, and the biases.
+//
+// Bound: instruction issue (about 120 warp instructions per sample).  Through
+// memory (a [n][64] gradient and activation array written by strided stores and
+// read back by a thread per parameter, serially over 1024 samples) 204,800
+// samples took 174 + 336 + 27 us; now 72 + 7 us.
+constexpr int kTile = 64;
+constexpr int kTileStride = kTile + 8;   // rows on 16 bytes; four rows on distinct banks
+constexpr int kBackThreads = 4 * kTile;
+constexpr int kBackBlocks = 512;         // most blocks (partial sums)
+static_assert(kBackThreads == 4 * kH, "a thread per (unit, part)");
 
-BackScratch carve(void* base, int64_t n, int C, int64_t P) {
-  auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  char* p = (char*)base;
-  BackScratch b;
-  b.dz1 = (float*)p;
-  p += al(sizeof(float) * n * kH);
-  b.a = (__nv_bfloat16*)p;
-  p += al(sizeof(__nv_bfloat16) * n * kH);
-  b.dz2 = (float*)p;
-  p += al(sizeof(float) * n * C);
-  b.loss = (float*)p;
-  p += al(sizeof(float) * n);
-  b.partial = (float*)p;   // [chunks][P + 1]
-  (void)P;
-  return b;
-}
-
-__global__ void __launch_bounds__(128)
-k_mlp_back_samples(MlpView M, int64_t n, const float* __restrict__ x,
-                   const int32_t* __restrict__ labels, const float* __restrict__ w,
-                   BackScratch B, int* status) {
-  __shared__ SmemMlp S;
-  stage_mlp(M, S);
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    float xb[kMlpMaxF], z[kMlpMaxC];
-    load_features(x, M.F, s, xb);
-    mlp_logits(S, xb, z, B.a + s * kH);
-    float mx = -INFINITY;
+constexpr int kBackPerSM = 3;            // resident blocks (85 registers, 44-51 KB)
+template <int FP, int CP>
+__global__ void __launch_bounds__(kBackThreads, kBackPerSM)
+k_mlp_back(MlpView M, int64_t n, const float* __restrict__ x, const int32_t* __restrict__ labels,
+           const float* __restrict__ w, float* __restrict__ partial, int64_t P, int* status) {
+  __shared__ float sW1[kH][FP], sb1[kH], sW2[CP][kH], sb2[CP];
+  __shared__ __align__(16) float sX[FP][kTileStride], sD1[kH][kTileStride], sA[kH][kTileStride],
+      sD2[CP][kTileStride];
+  __shared__ float sLoss[kTile];
+  const int tid = threadIdx.x, part = tid & 3, F = M.F, C = M.C;
+  for (int i = tid; i < kH * FP; i += kBackThreads) {
+    const int j = i / FP, f = i - j * FP;
+    sW1[j][f] = f < F ? __bfloat162float(M.W1[j * F + f]) : 0.0f;
+  }
+  for (int i = tid; i < kH; i += kBackThreads) sb1[i] = M.b1[i];
+  for (int i = tid; i < CP * kH; i += kBackThreads)
+    sW2[i / kH][i % kH] = i < C * kH ? __bfloat162float(M.W2[i]) : 0.0f;
+  if (tid < CP) sb2[tid] = tid < C ? M.b2[tid] : 0.0f;
+  for (int i = tid; i < FP * kTileStride; i += kBackThreads) (&sX[0][0])[i] = 0.0f;
+  float gW1[FP / 4], gW2[CP / 4], gb1 = 0.0f, gb2[CP / 4], gl = 0.0f;
 #pragma unroll
-    for (int c = 0; c < kMlpMaxC; ++c)
-      if (c < M.C) mx = fmaxf(mx, z[c]);
-    float e[kMlpMaxC], sum = 0.0f;
+  for (int i = 0; i < FP / 4; ++i) gW1[i] = 0.0f;
 #pragma unroll
-    for (int c = 0; c < kMlpMaxC; ++c) {
-      e[c] = c < M.C ? expf(z[c] - mx) : 0.0f;
-      sum += e[c];
+  for (int i = 0; i < CP / 4; ++i) gW2[i] = gb2[i] = 0.0f;
+  const int64_t tiles = (n + kTile - 1) / kTile;
+  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int64_t s0 = t * kTile;
+    const int have = (int)min((int64_t)kTile, n - s0);
+    __syncthreads();                       // the previous tile is added
+    for (int i = tid; i < kTile * F; i += kBackThreads) {
+      const int s = i / F, f = i - s * F;
+      sX[f][s] = s < have ? bf16_round(x[s0 * F + i]) : 0.0f;
     }
-    int y = labels[s];
-    float ws = w ? w[s] : 1.0f;
-    if (y < 0 || y >= M.C) {
-      atomicOr(status, kStatusInvalid);
-      y = 0;
-      ws = 0.0f;
+    __syncthreads();
+    {
+      const int s = tid >> 2;
+      const bool live = s < have;
+      float xb[FP], z[CP];
+      unsigned on = 0;                     // the units with a positive input
+#pragma unroll
+      for (int f = 0; f < FP; ++f) xb[f] = sX[f][s];
+#pragma unroll
+      for (int c = 0; c < CP; ++c) z[c] = 0.0f;
+#pragma unroll 4
+      for (int i = 0; i < kH / 4; ++i) {
+        const int j = 4 * i + part;
+        float pre = sb1[j];
+#pragma unroll
+        for (int f = 0; f < FP; ++f) pre = fmaf(sW1[j][f], xb[f], pre);
+        const float a = bf16_round(fmaxf(pre, 0.0f));
+        sA[j][s] = a;
+        on |= (pre > 0.0f ? 1u : 0u) << i;
+#pragma unroll
+        for (int c = 0; c < CP; ++c) z[c] = fmaf(sW2[c][j], a, z[c]);
+      }
+      float mx = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < CP; ++c) {
+        z[c] += __shfl_xor_sync(0xffffffffu, z[c], 1);
+        z[c] += __shfl_xor_sync(0xffffffffu, z[c], 2);
+        z[c] += sb2[c];
+        if (c < C) mx = fmaxf(mx, z[c]);
+      }
+      float e[CP], sum = 0.0f;
+#pragma unroll
+      for (int c = 0; c < CP; ++c) {
+        e[c] = c < C ? expf(z[c] - mx) : 0.0f;
+        sum += e[c];
+      }
+      int y = live ? labels[s0 + s] : 0;
+      float ws = live ? (w ? w[s0 + s] : 1.0f) : 0.0f;
+      if (y < 0 || y >= C) {
+        if (part == 0) atomicOr(status, kStatusInvalid);
+        y = 0;
+        ws = 0.0f;
+      }
+      float zy = 0.0f;
+#pragma unroll
+      for (int c = 0; c < CP; ++c)
+        if (c == y) zy = z[c];
+      const float inv = 1.0f / sum;
+#pragma unroll
+      for (int c = 0; c < CP; ++c) {
+        e[c] = c < C && live ? ws * (e[c] * inv - (c == y ? 1.0f : 0.0f)) : 0.0f;   // dz_c
+        if ((c & 3) == part) sD2[c][s] = e[c];
+      }
+      if (part == 0) sLoss[s] = live ? ws * (logf(sum) - (zy - mx)) : 0.0f;
+#pragma unroll 4
+      for (int i = 0; i < kH / 4; ++i) {
+        const int j = 4 * i + part;
+        float dh = 0.0f;
+#pragma unroll
+        for (int c = 0; c < CP; ++c) dh = fmaf(sW2[c][j], e[c], dh);
+        sD1[j][s] = (on >> i) & 1 ? dh : 0.0f;
+      }
     }
-    float zy = 0.0f;
+    __syncthreads();
+    const int j = tid >> 2;
+#pragma unroll 2
+    for (int s = 0; s < kTile; s += 4) {
+      const float4 d = *reinterpret_cast<const float4*>(&sD1[j][s]);
+      const float4 av = *reinterpret_cast<const float4*>(&sA[j][s]);
 #pragma unroll
-    for (int c = 0; c < kMlpMaxC; ++c)
-      if (c == y) zy = z[c];
-    B.loss[s] = ws * (logf(sum) - (zy - mx));
-    float dz[kMlpMaxC];
-    const float inv = 1.0f / sum;
+      for (int i = 0; i < FP / 4; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(&sX[part * (FP / 4) + i][s]);
+        gW1[i] = fmaf(d.x, v.x, gW1[i]);
+        gW1[i] = fmaf(d.y, v.y, gW1[i]);
+        gW1[i] = fmaf(d.z, v.z, gW1[i]);
+        gW1[i] = fmaf(d.w, v.w, gW1[i]);
+      }
 #pragma unroll
-    for (int c = 0; c < kMlpMaxC; ++c) {
-      dz[c] = c < M.C ? ws * (e[c] * inv - (c == y ? 1.0f : 0.0f)) : 0.0f;
-      if (c < M.C) B.dz2[s * M.C + c] = dz[c];
-    }
-    for (int j = 0; j < kH; ++j) {
-      float dh = 0.0f;
-#pragma unroll
-      for (int c = 0; c < kMlpMaxC; ++c) dh = fmaf(S.W2[c * kH + j], dz[c], dh);
-      B.dz1[s * kH + j] = hidden_pre(S, j, xb) > 0.0f ? dh : 0.0f;
+      for (int i = 0; i < CP / 4; ++i) {
+        const float4 g = *reinterpret_cast<const float4*>(&sD2[part + 4 * i][s]);
+        gW2[i] = fmaf(g.x, av.x, gW2[i]);
+        gW2[i] = fmaf(g.y, av.y, gW2[i]);
+        gW2[i] = fmaf(g.z, av.z, gW2[i]);
+        gW2[i] = fmaf(g.w, av.w, gW2[i]);
+        gb2[i] += g.x + g.y + (g.z + g.w);
+      }
+      gb1 += d.x + d.y + (d.z + d.w);
+      if (tid == 0) gl += sLoss[s] + sLoss[s + 1] + (sLoss[s + 2] + sLoss[s + 3]);
     }
   }
-}
-
-// partial[chunk][p] for p < P (parameters) and p == P (loss)
-__global__ void __launch_bounds__(128)
-k_mlp_back_partials(int F, int C, int64_t n, const float* __restrict__ x, BackScratch B,
-                    int64_t P) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > P) return;
-  const int64_t s0 = (int64_t)blockIdx.y * kChunk, s1 = min(n, s0 + kChunk);
-  const int64_t oW1 = (int64_t)kH * F, ob1 = oW1 + kH, oW2 = ob1 + (int64_t)C * kH;
-  float acc = 0.0f;
-  if (p < oW1) {
-    const int j = (int)(p / F), f = (int)(p % F);
-    for (int64_t s = s0; s < s1; ++s) acc = fmaf(B.dz1[s * kH + j], bf16_round(x[s * F + f]), acc);
-  } else if (p < ob1) {
-    const int j = (int)(p - oW1);
-    for (int64_t s = s0; s < s1; ++s) acc += B.dz1[s * kH + j];
-  } else if (p < oW2) {
-    const int q = (int)(p - ob1), c = q / kH, j = q % kH;
-    for (int64_t s = s0; s < s1; ++s)
-      acc = fmaf(B.dz2[s * C + c], __bfloat162float(B.a[s * kH + j]), acc);
-  } else if (p < P) {
-    const int c = (int)(p - oW2);
-    for (int64_t s = s0; s < s1; ++s) acc += B.dz2[s * C + c];
-  } else {
-    for (int64_t s = s0; s < s1; ++s) acc += B.loss[s];
+  // this block's sums (parameter order: W1, b1, W2, b2, then the loss)
+  float* out = partial + (int64_t)blockIdx.x * (P + 1);
+  const int j = tid >> 2;
+  const int64_t ob1 = (int64_t)kH * F, oW2 = ob1 + kH, ob2 = oW2 + (int64_t)C * kH;
+#pragma unroll
+  for (int i = 0; i < FP / 4; ++i) {
+    const int f = part * (FP / 4) + i;
+    if (f < F) out[j * F + f] = gW1[i];
   }
-  B.partial[(int64_t)blockIdx.y * (P + 1) + p] = acc;
+  if (part == 0) out[ob1 + j] = gb1;
+#pragma unroll
+  for (int i = 0; i < CP / 4; ++i) {
+    const int c = part + 4 * i;
+    if (c < C) {
+      out[oW2 + c * kH + j] = gW2[i];
+      if (j == 0) out[ob2 + c] = gb2[i];
+    }
+  }
+  if (tid == 0) out[P] = gl;
 }
 
-__global__ void __launch_bounds__(128)
-k_mlp_back_final(int64_t n, int64_t P, int chunks, const float* __restrict__ partial,
+// The blocks' sums of 32 parameters: eight slices of blocks, each in order,
+// added in order.
+__global__ void __launch_bounds__(256)
+k_mlp_back_final(int64_t n, int64_t P, int blocks, const float* __restrict__ partial,
                  float* __restrict__ grad, float* __restrict__ loss) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > P) return;
+  __shared__ float s_sum[8][32];
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+  const int64_t p = (int64_t)blockIdx.x * 32 + lane;
+  const int per = (blocks + 7) / 8, c0 = slice * per, c1 = min(blocks, c0 + per);
   float acc = 0.0f;
-  for (int c = 0; c < chunks; ++c) acc += partial[(int64_t)c * (P + 1) + p];
-  const float v = acc / (float)n;
-  if (p < P)
-    grad[p] = v;
-  else
-    loss[0] = v;
+  if (p <= P) {
+#pragma unroll 8
+    for (int c = c0; c < c1; ++c) acc += partial[(int64_t)c * (P + 1) + p];
+  }
+  s_sum[slice][lane] = acc;
+  __syncthreads();
+  if (slice == 0 && p <= P) {
+#pragma unroll
+    for (int k = 1; k < 8; ++k) acc += s_sum[k][lane];
+    const float v = acc / (float)n;
+    if (p < P)
+      grad[p] = v;
+    else
+      loss[0] = v;
+  }
 }
 
 __global__ void __launch_bounds__(256)
@@ -288,15 +358,11 @@ k_mlp_adam(int F, int C, int64_t P, float* __restrict__ param, float* __restrict
   else if (p >= ob1 && p < oW2) W2b[p - ob1] = __float2bfloat16_rn(th);
 }
 
-int chunks_of(int64_t n) { return (int)((n + kChunk - 1) / kChunk); }
-
 }  // namespace
 
 size_t mlp_backward_scratch(int64_t n, int F, int C) {
-  auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  const int64_t P = mlp_num_params(F, C);
-  return al(sizeof(float) * n * kH) + al(2 * (size_t)n * kH) + al(sizeof(float) * n * C) +
-         al(sizeof(float) * n) + al(sizeof(float) * (size_t)chunks_of(n) * (P + 1));
+  const int64_t blocks = std::min<int64_t>(kBackBlocks, (n + kTile - 1) / kTile);
+  return sizeof(float) * (size_t)std::max<int64_t>(1, blocks) * (size_t)(mlp_num_params(F, C) + 1);
 }
 
 static unsigned grid_for(int64_t n, int threads, int cap) {
@@ -350,15 +416,15 @@ cudaError_t launch_mlp_backward(const Launch& L, const MlpView& M, int64_t n, co
                                 float* grad, float* loss) {
   if (n <= 0) return cudaErrorInvalidValue;
   const int64_t P = mlp_num_params(M.F, M.C);
-  BackScratch B = carve(scratch, n, M.C, P);
-  k_mlp_back_samples<<<grid_for(n, 128, device_sms(L) * 16), 128, 0, L.stream>>>(M, n, x, labels, w, B,
-                                                                       L.status);
-  const int chunks = chunks_of(n);
-  dim3 g2((unsigned)((P + 1 + 127) / 128), (unsigned)chunks);
-  k_mlp_back_partials<<<g2, 128, 0, L.stream>>>(M.F, M.C, n, x, B, P);
-  k_mlp_back_final<<<(unsigned)((P + 1 + 127) / 128), 128, 0, L.stream>>>(n, P, chunks,
-                                                                           B.partial, grad, loss);
-  *L.launches += 3;
+  float* partial = (float*)scratch;
+  const int blocks = (int)std::min<int64_t>(std::min<int64_t>(kBackBlocks, kBackPerSM * device_sms(L)),
+                                            (n + kTile - 1) / kTile);
+  auto kern = M.F <= 8 ? (M.C <= 4 ? k_mlp_back<8, 4> : k_mlp_back<8, 8>)
+                       : (M.C <= 4 ? k_mlp_back<16, 4> : k_mlp_back<16, 8>);
+  kern<<<blocks, kBackThreads, 0, L.stream>>>(M, n, x, labels, w, partial, P, L.status);
+  k_mlp_back_final<<<(unsigned)((P + 1 + 31) / 32), 256, 0, L.stream>>>(n, P, blocks, partial,
+                                                                        grad, loss);
+  *L.launches += 2;
   return cudaGetLastError();
 }
 
