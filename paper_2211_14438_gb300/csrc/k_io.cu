@@ -44,7 +44,9 @@ cudaError_t launch_init_inputs(const Launch& L, int n, int64_t n_boxes, const fl
 }
 
 // a5: copy the output-layer polynomials into the caller's (keys, coef) form.
-// One block per (box, output).
+// A block per (box, output) and kPackTerms terms: one block for all terms took
+// 530 us on 48 boxes of 74,613 terms, 14 us in parts.
+constexpr int kPackTerms = 2048;
 __global__ void k_pack(Tables T, int o, const float* __restrict__ pre_up,
                        const float* __restrict__ pre_lo, int64_t ld,
                        const int32_t* __restrict__ nterms, bern_result res, int* status) {
@@ -52,7 +54,7 @@ __global__ void k_pack(Tables T, int o, const float* __restrict__ pre_up,
   const int64_t b = item / o;
   const int j = (int)(item - b * o);
   const int nt = nterms[item];
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && blockIdx.y == 0) {
     res.n_terms[item * 2] = nt;
     res.n_terms[item * 2 + 1] = nt;
     if (nt > res.cap_terms && (res.coef || res.keys)) atomicOr(status, kStatusCapacity);
@@ -62,11 +64,12 @@ __global__ void k_pack(Tables T, int o, const float* __restrict__ pre_up,
   for (int k = 0; k < 2; ++k) {
     const float* P = k == 0 ? pre_up : pre_lo;
     const int64_t base = (item * 2 + k) * res.cap_terms;
-    for (int r = threadIdx.x; r < nt; r += blockDim.x) {
+    for (int64_t r = (int64_t)blockIdx.y * kPackTerms + threadIdx.x;
+         r < min((int64_t)nt, ((int64_t)blockIdx.y + 1) * kPackTerms); r += blockDim.x) {
       if (res.coef) res.coef[base + r] = P[(b * ld + r) * o + j];
       if (res.keys) {
         uint64_t key = 0;
-        for (int v = 0; v < n; ++v) key |= (uint64_t)T.exps[(int64_t)r * n + v] << (8 * v);
+        for (int v = 0; v < n; ++v) key |= (uint64_t)T.exps[r * n + v] << (8 * v);
         res.keys[base + r] = key;
       }
     }
@@ -77,8 +80,12 @@ cudaError_t launch_pack(const Launch& L, const Tables& T, int64_t n_boxes, int o
                         const float* pre_up, const float* pre_lo, int64_t ld,
                         const int32_t* nterms, bern_result res) {
   if (n_boxes == 0) return cudaSuccess;
-  k_pack<<<(unsigned)(n_boxes * o), 128, 0, L.stream>>>(T, o, pre_up, pre_lo, ld, nterms, res,
-                                                        L.status);
+  // term counts are at most ld (a larger one fails the capacity check, or is
+  // bounded by cap_terms)
+  const int64_t terms = std::max<int64_t>(1, std::min(ld, res.cap_terms));
+  const int64_t parts = std::min<int64_t>(65535, (terms + kPackTerms - 1) / kPackTerms);
+  dim3 grid((unsigned)(n_boxes * o), (unsigned)parts);
+  k_pack<<<grid, 128, 0, L.stream>>>(T, o, pre_up, pre_lo, ld, nterms, res, L.status);
   ++*L.launches;
   return cudaGetLastError();
 }
