@@ -28,6 +28,7 @@
 // count are read as zero.
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "device_util.cuh"
 #include "packed.cuh"
@@ -157,24 +158,58 @@ k_affine(int h_out, int h_in, const float* __restrict__ W, const float* __restri
 
 // Persistent, register-blocked form for the wide layers: a block of four
 // warps keeps W (h_in x h_out, k-major, neurons padded to 64) in shared
-// memory for the whole launch and walks boxes; per box it stages 64-row tiles
-// of the input as (midpoint, radius) pairs, and every thread accumulates an
-// 8 (neurons) x 4 (rows) tile of the three sums per 64-neuron slice: neurons
-// 4 tm .. 4 tm + 3 and 32 + 4 tm .. 32 + 4 tm + 3, so the eight lanes of a
-// row read each half of the slice's weights as one contiguous 128-byte float4
-// load; 4 pairs are read as float2 per input j, and |w| is taken in the
-// radius FMA itself.  The staging issues kWBatch loads of each bound per
-// thread before converting any.  A warp covers 16 rows of the tile and skips
+// memory for the whole launch and walks boxes; per box it stages tiles of 16 TR
+// rows of the input as (midpoint, radius) pairs, and every thread
+// accumulates an 8 (neurons) x TR (rows) tile of the three sums per 64-neuron
+// slice: neurons 4 tm .. 4 tm + 3 and 32 + 4 tm .. 32 + 4 tm + 3, so the eight
+// lanes of a row read each half of the slice's weights as one contiguous
+// 128-byte load.  Sums of two neighbouring neurons are one packed FMA
+// (packed.cuh: the weights of a load are already pairs, the duplicated midpoint
+// and radius the other operand).  A tile holds only the inputs that have terms
+// in it: dead neurons and identity neurons of a lower degree drop out of the
+// higher rows (their products are exact zeros), about half of the inputs of the
+// benchmark network's last layers.  The next tile's list of inputs is made
+// while a tile is staged.  The staging issues kWBatch loads of each bound per
+// thread before converting any.  A warp covers 4 TR rows of the tile and skips
 // the tile when all of them are at or past the box's term count.  With a
 // ScreenOut it also screens the box's output items (R21): every thread sums
 // max(0, upper) and min(0, lower) of its output coefficients past the first
 // (rounding up, resp. down), the four lanes of a warp that share neurons
 // combine theirs, each warp adds its sum into its own shared row, and after
 // the box the rows are added to the constant coefficient in warp order.
+//
+// Bound: the FP32 pipe during the products, the staging between them.  Layer 4
+// of [3,64x4,1], 5120 boxes: 595 us with three scalar FMAs over all inputs, 404 us
+// (its 1.04e10 FMAs, zeros included, take 267 us at the measured rate).
 constexpr int kWThreads = 128;
 constexpr int kWBatch = 8;
 
-template <int TR, int MINB, bool SCREEN>
+__device__ __forceinline__ p2 fma2_rd(p2 a, p2 b, p2 c) {
+  p2 r;
+  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// The inputs with a term at row r0 or later, in order; one warp.
+__device__ __forceinline__ int live_inputs(const int* sN, int h_in, int r0, int* list) {
+  const int lane = threadIdx.x & 31;
+  int n = 0;
+  for (int j0 = 0; j0 < h_in; j0 += 32) {
+    const int j = j0 + lane;
+    const bool live = j < h_in && sN[j] > r0;
+    const unsigned m = __ballot_sync(0xffffffffu, live);
+    if (live) list[n + __popc(m & ((1u << lane) - 1u))] = j;
+    n += __popc(m);
+  }
+  return n;
+}
+
+// LIVE: tiles hold only the inputs with terms, and the FMAs are packed; not worth
+// the lists and the wider register tiles for few inputs or a single tile (28
+// rows, 33 x 47, 2000 boxes: 28.5 us without, 31 us with them).
+constexpr int kWideLiveInputs = 48, kWideLiveRows = 32;
+
+template <int TR, int MINB, bool SCREEN, bool LIVE>
 __global__ void __launch_bounds__(kWThreads, MINB)
 k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
               const float* __restrict__ bias, const float* __restrict__ in_up,
@@ -188,12 +223,12 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
   float* sW = reinterpret_cast<float*>(smem4);       // [h_in][hp]
   float2* sCR = reinterpret_cast<float2*>(sW + (size_t)h_in * hp);   // [ROWS][h_in + 1]
   int* sN = reinterpret_cast<int*>(sCR + (size_t)ROWS * (h_in + 1));   // [h_in]
+  int* sJ = sN + h_in;                               // [2][h_in]: the inputs of a tile
   // screen partials: per warp and neuron the directed sums of max(0, upper)
   // and min(0, lower) over the warp's rows past the first, and row 0 itself
-  float* sScr = reinterpret_cast<float*>(sN + h_in);   // [4][2][hp]
+  float* sScr = reinterpret_cast<float*>(sJ + 2 * h_in);   // [4][2][hp]
   float* sC0 = sScr + 8 * hp;                          // [2][hp]
-  constexpr bool screen = SCREEN;
-  __shared__ int sMax;
+  __shared__ int sMax, sLive[2];
   const int tid = threadIdx.x, warp = tid >> 5;
   for (int idx = tid; idx < h_in * hp; idx += kWThreads) {
     const int j = idx / hp, m = idx - j * hp;
@@ -201,7 +236,6 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
   }
   const int tm = tid & 7, tr = tid >> 3;             // 8 x 16 threads
   const int ldx = h_in + 1;
-  const int step_r = kWThreads / h_in, step_j = kWThreads - step_r * h_in;
   const bool vec_out =
       (h_out & 3) == 0 &&
       ((reinterpret_cast<uintptr_t>(out_up) | reinterpret_cast<uintptr_t>(out_lo)) & 15) == 0;
@@ -227,85 +261,147 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
       continue;
     }
     for (int m = tid; m < h_out; m += kWThreads) out_nterms[b * h_out + m] = M;
-    if (screen)
+    if (SCREEN)
       for (int x = tid; x < 8 * hp; x += kWThreads) sScr[x] = 0.0f;
+    if (LIVE && warp == 0) {
+      const int nl = live_inputs(sN, h_in, 0, sJ);
+      if (tid == 0) sLive[0] = nl;
+    }
     const float* gU = in_up + (b * in_ld) * h_in;
     const float* gL = in_lo + (b * in_ld) * h_in;
-    for (int r0 = 0; r0 < M; r0 += ROWS) {
+    int buf = 0;
+    for (int r0 = 0; r0 < M; r0 += ROWS, buf ^= 1) {
       __syncthreads();                               // the previous tile is consumed
-      // element idx = rr * h_in + j of the tile; (rr, j) advance by
-      // (step_r, step_j) per kWThreads elements
-      int rr = tid / h_in, j = tid - (tid / h_in) * h_in;
-      for (int idx = tid; idx < ROWS * h_in; idx += kWThreads * kWBatch) {
-        float u[kWBatch], l[kWBatch];
-        int at[kWBatch];
+      const int nl = LIVE ? sLive[buf] : h_in;
+      const int* J = sJ + buf * h_in;
+      if (!LIVE || nl > 0) {
+        // element idx = rr * nl + jj of the tile; (rr, jj) advance by
+        // (step_r, step_j) per kWThreads elements
+        const int step_r = kWThreads / nl, step_j = kWThreads - step_r * nl;
+        int rr = tid / nl, jj = tid - (tid / nl) * nl;
+        for (int idx = tid; idx < ROWS * nl; idx += kWThreads * kWBatch) {
+          float u[kWBatch], l[kWBatch];
+          int at[kWBatch];
 #pragma unroll
-        for (int q = 0; q < kWBatch; ++q) {
-          const bool in = idx + q * kWThreads < ROWS * h_in;
-          const int r = r0 + rr;
-          const bool live = in && r < sN[j];         // sN[j] <= M <= in_ld
-          u[q] = live ? gU[(int64_t)r * h_in + j] : 0.0f;
-          l[q] = live ? gL[(int64_t)r * h_in + j] : 0.0f;
-          at[q] = in ? rr * ldx + j : -1;
-          rr += step_r;
-          j += step_j;
-          if (j >= h_in) {
-            j -= h_in;
-            ++rr;
+          for (int q = 0; q < kWBatch; ++q) {
+            const bool in = idx + q * kWThreads < ROWS * nl;
+            const int r = r0 + rr, j = LIVE ? (in ? J[jj] : 0) : jj;
+            const bool live = in && r < sN[j];       // sN[j] <= M <= in_ld
+            u[q] = live ? gU[(int64_t)r * h_in + j] : 0.0f;
+            l[q] = live ? gL[(int64_t)r * h_in + j] : 0.0f;
+            at[q] = in ? rr * ldx + jj : -1;
+            rr += step_r;
+            jj += step_j;
+            if (jj >= nl) {
+              jj -= nl;
+              ++rr;
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < kWBatch; ++q) {
+            const float c = __fmaf_rn(0.5f, u[q], 0.5f * l[q]);
+            const float rd = fmaxf(__fsub_ru(u[q], c), __fsub_ru(c, l[q]));
+            if (at[q] >= 0) sCR[at[q]] = make_float2(c, rd);
           }
         }
-#pragma unroll
-        for (int q = 0; q < kWBatch; ++q) {
-          const float c = __fmaf_rn(0.5f, u[q], 0.5f * l[q]);
-          const float rd = fmaxf(__fsub_ru(u[q], c), __fsub_ru(c, l[q]));
-          if (at[q] >= 0) sCR[at[q]] = make_float2(c, rd);
-        }
+      }
+      if (LIVE && warp == 0 && r0 + ROWS < M) {
+        const int n2 = live_inputs(sN, h_in, r0 + ROWS, sJ + (buf ^ 1) * h_in);
+        if (tid == 0) sLive[buf ^ 1] = n2;
       }
       __syncthreads();
       if (r0 + warp * 4 * TR >= M) continue;         // warp-uniform; no barrier follows
       for (int m0 = 0; m0 < h_out; m0 += 64) {
-        float uc[TR][8], lc[TR][8], rad[TR][8];
+        // LIVE: pairs of neighbouring neurons, i = 0, 1 the first half, 2, 3 the
+        // second; otherwise one neuron each
+        p2 uc[TR][4], lc[TR][4], rad[TR][4];
+        float us[TR][8], ls[TR][8], rs[TR][8];
 #pragma unroll
         for (int k = 0; k < TR; ++k)
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int m = m0 + (i < 4 ? 4 * tm + i : 28 + 4 * tm + i), r = r0 + tr * TR + k;
-            const float b0 = (r == 0 && m < h_out) ? bias[m] : 0.0f;
-            uc[k][i] = b0;
-            lc[k][i] = b0;
-            rad[k][i] = 0.0f;
+          for (int i = 0; i < 4; ++i) {
+            const int m = m0 + 4 * tm + (i < 2 ? 2 * i : 28 + 2 * i), r = r0 + tr * TR + k;
+            const float b0 = r == 0 && m < h_out ? bias[m] : 0.0f;
+            const float b1 = r == 0 && m + 1 < h_out ? bias[m + 1] : 0.0f;
+            uc[k][i] = lc[k][i] = pack2(b0, b1);
+            rad[k][i] = 0ull;
+            us[k][2 * i] = ls[k][2 * i] = b0;
+            us[k][2 * i + 1] = ls[k][2 * i + 1] = b1;
+            rs[k][2 * i] = rs[k][2 * i + 1] = 0.0f;
           }
         const float* pw = sW + m0 + tm * 4;
         const float2* pcr = sCR + (tr * TR) * ldx;
+        if constexpr (LIVE) {
 #pragma unroll 2
-        for (int j = 0; j < h_in; ++j) {
-          float2 cr[TR];
+          for (int jj = 0; jj < nl; ++jj) {
+            const float* pj = pw + (size_t)J[jj] * hp;
+            p2 c[TR], rd[TR];
 #pragma unroll
-          for (int k = 0; k < TR; ++k) cr[k] = pcr[k * ldx + j];
+            for (int k = 0; k < TR; ++k) {
+              const float2 v = pcr[k * ldx + jj];
+              c[k] = pack2(v.x, v.x);
+              rd[k] = pack2(v.y, v.y);
+            }
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            const float4 w4 = *reinterpret_cast<const float4*>(pw + (size_t)j * hp + 32 * half);
-            const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+            for (int half = 0; half < 2; ++half) {
+              const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(pj + 32 * half);
+              const p2 w[2] = {w2.x, w2.y};
 #pragma unroll
-            for (int k = 0; k < TR; ++k)
+              for (int i = 0; i < 2; ++i) {
+                const p2 aw = w[i] & 0x7fffffff7fffffffull;
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int ii = 4 * half + i;
-                uc[k][ii] = __fmaf_ru(w[i], cr[k].x, uc[k][ii]);
-                lc[k][ii] = __fmaf_rd(w[i], cr[k].x, lc[k][ii]);
-                rad[k][ii] = __fmaf_ru(fabsf(w[i]), cr[k].y, rad[k][ii]);
+                for (int k = 0; k < TR; ++k) {
+                  const int ii = 2 * half + i;
+                  uc[k][ii] = fma2_ru(w[i], c[k], uc[k][ii]);
+                  lc[k][ii] = fma2_rd(w[i], c[k], lc[k][ii]);
+                  rad[k][ii] = fma2_ru(aw, rd[k], rad[k][ii]);
+                }
               }
+            }
+          }
+        } else {
+#pragma unroll 2
+          for (int j = 0; j < h_in; ++j) {
+            float2 cr[TR];
+#pragma unroll
+            for (int k = 0; k < TR; ++k) cr[k] = pcr[k * ldx + j];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              const float4 w4 = *reinterpret_cast<const float4*>(pw + (size_t)j * hp + 32 * half);
+              const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+              for (int k = 0; k < TR; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const int ii = 4 * half + i;
+                  us[k][ii] = __fmaf_ru(w[i], cr[k].x, us[k][ii]);
+                  ls[k][ii] = __fmaf_rd(w[i], cr[k].x, ls[k][ii]);
+                  rs[k][ii] = __fmaf_ru(fabsf(w[i]), cr[k].y, rs[k][ii]);
+                }
+            }
           }
         }
+        float su[8], sl[8];                          // screen: this thread's rows past the first
+#pragma unroll
+        for (int i = 0; i < 8; ++i) su[i] = sl[i] = 0.0f;
 #pragma unroll
         for (int k = 0; k < TR; ++k) {
           const int r = r0 + tr * TR + k;
           const bool valid = r < M;
           float vu[8], vl[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            vu[i] = __fadd_ru(uc[k][i], rad[k][i]);
-            vl[i] = __fsub_rd(lc[k][i], rad[k][i]);
+          for (int i = 0; i < 4; ++i) {
+            float a = us[k][2 * i], c = us[k][2 * i + 1], d = ls[k][2 * i], e = ls[k][2 * i + 1];
+            float f = rs[k][2 * i], g = rs[k][2 * i + 1];
+            if constexpr (LIVE) {
+              unpack2(uc[k][i], a, c);
+              unpack2(lc[k][i], d, e);
+              unpack2(rad[k][i], f, g);
+            }
+            vu[2 * i] = __fadd_ru(a, f);
+            vu[2 * i + 1] = __fadd_ru(c, g);
+            vl[2 * i] = __fsub_rd(d, f);
+            vl[2 * i + 1] = __fsub_rd(e, g);
           }
           if (valid) {
             const int64_t o = (b * out_ld + r) * h_out + m0;
@@ -328,7 +424,7 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
               }
             }
           }
-          if (screen) {   // warp-uniform (every lane runs every k)
+          if (SCREEN) {
             if (valid && r == 0) {
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
@@ -336,31 +432,36 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
                 sC0[m] = vu[i];
                 sC0[hp + m] = vl[i];
               }
-            }
-            // this row's one-sided parts, combined over the four lanes of the
-            // warp that share neurons (lane, lane ^ 8, ^ 16, ^ 24), then added
-            // into the warp's own shared row
-            const bool part = valid && r > 0;
+            } else if (valid) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              float cu = part ? fmaxf(vu[i], 0.0f) : 0.0f;
-              float cl = part ? fminf(vl[i], 0.0f) : 0.0f;
-              cu = __fadd_ru(cu, __shfl_xor_sync(0xffffffffu, cu, 8));
-              cl = __fadd_rd(cl, __shfl_xor_sync(0xffffffffu, cl, 8));
-              cu = __fadd_ru(cu, __shfl_xor_sync(0xffffffffu, cu, 16));
-              cl = __fadd_rd(cl, __shfl_xor_sync(0xffffffffu, cl, 16));
-              if ((tid & 31) < 8) {
-                const int m = m0 + (i < 4 ? 4 * tm + i : 28 + 4 * tm + i);
-                float* ps = sScr + (warp * 2) * hp + m;
-                ps[0] = __fadd_ru(ps[0], cu);
-                ps[hp] = __fadd_rd(ps[hp], cl);
+              for (int i = 0; i < 8; ++i) {
+                su[i] = __fadd_ru(su[i], fmaxf(vu[i], 0.0f));
+                sl[i] = __fadd_rd(sl[i], fminf(vl[i], 0.0f));
               }
+            }
+          }
+        }
+        if (SCREEN) {   // warp-uniform
+          // combined over the four lanes of the warp that share neurons (lane,
+          // lane ^ 8, ^ 16, ^ 24), then added into the warp's own shared row
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float cu = su[i], cl = sl[i];
+            cu = __fadd_ru(cu, __shfl_xor_sync(0xffffffffu, cu, 8));
+            cl = __fadd_rd(cl, __shfl_xor_sync(0xffffffffu, cl, 8));
+            cu = __fadd_ru(cu, __shfl_xor_sync(0xffffffffu, cu, 16));
+            cl = __fadd_rd(cl, __shfl_xor_sync(0xffffffffu, cl, 16));
+            if ((tid & 31) < 8) {
+              const int m = m0 + (i < 4 ? 4 * tm + i : 28 + 4 * tm + i);
+              float* ps = sScr + (warp * 2) * hp + m;
+              ps[0] = __fadd_ru(ps[0], cu);
+              ps[hp] = __fadd_rd(ps[hp], cl);
             }
           }
         }
       }
     }
-    if (screen) {
+    if (SCREEN) {
       // the box's items: row 0 plus the warps' partials in warp order; the
       // stable ones get their case and interval, the others join the list
       __syncthreads();
@@ -555,7 +656,7 @@ static size_t short_smem(int h_out, int h_in) {
 static size_t wide_smem(int h_out, int h_in, int rows) {
   const size_t hp = (size_t)((h_out + 63) & ~63);
   return hp * h_in * sizeof(float) + (size_t)rows * (h_in + 1) * sizeof(float2) +
-         (size_t)h_in * sizeof(int) + 10 * hp * sizeof(float);   // + the screen partials
+         3 * (size_t)h_in * sizeof(int) + 10 * hp * sizeof(float);   // + the screen partials
 }
 
 // Narrow output layers (h_out <= 4, e.g. a network's output): one thread per
@@ -921,31 +1022,43 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
   const bool few_rows = std::min(in_ld, out_ld) <= 16;     // short polynomials: short tiles
   if (h_out >= 32) {
     // wide layers: autotuned among the persistent register-blocked kernel with
-    // 4-row (0), 2-row (2, the default for longer polynomials) or 1-row (3)
-    // thread tiles, when its weights fit shared memory, block tiles (1), and
+    // 4-row (0), 2-row (2, the default) or 1-row (3, up to 64 rows) thread tiles, when its weights fit shared memory, block tiles (1), and
     // for short polynomials a warp per box (4, their default)
     const std::string key = "affine/" + std::to_string(h_out) + "/" + std::to_string(h_in) +
                             "/" + std::to_string(in_ld) + "/" + std::to_string(n_boxes);
-    const bool wide_ok = wide_smem(h_out, h_in, 64) <= 200 * 1024;
+    // 4-row thread tiles (64-row tiles) take the 2-row form where they do not fit
+    const bool wide_ok = wide_smem(h_out, h_in, 32) <= 200 * 1024;
+    const bool wide4_ok = wide_smem(h_out, h_in, 64) <= 200 * 1024;
     const size_t ssmem = short_smem(h_out, h_in);
     const bool short_ok = few_rows && ssmem <= 200 * 1024;
-    int v = tune_variant(L, "affine", key, short_ok ? 4 : (wide_ok ? 2 : 1));
+    // 1-row thread tiles from 33 to 64 rows (with lists): a 32-row tile is half empty at 35 rows,
+    // and six blocks fit an SM instead of four (35 rows, 64 x 64, 5120 boxes: 132
+    // against 150 us; 165 rows: 610 against 495 us)
+    const int64_t rows_in = std::min(in_ld, out_ld);
+    const bool live = h_in >= kWideLiveInputs && rows_in > kWideLiveRows;
+    const int rows_dflt = live && rows_in <= 64 ? 3 : 2;
+    int v = tune_variant(L, "affine", key, short_ok ? 4 : (wide_ok ? rows_dflt : 1));
     if (v == 4 && !short_ok) v = wide_ok ? 2 : 1;
     if (v != 1 && v != 4 && !wide_ok) v = short_ok ? 4 : 1;
+    if (v == 0 && !wide4_ok) v = 2;
     TuneTimer tt;
     tune_begin(L, "affine", tt);
     cudaError_t e;
     if (v == 0 || v == 2 || v == 3) {
       const int rows = v == 0 ? 64 : (v == 2 ? 32 : 16);
       const size_t wsmem = wide_smem(h_out, h_in, rows);
-      auto kern = screen ? (v == 0 ? k_affine_wide<4, 4, true>
-                                   : (v == 2 ? k_affine_wide<2, 6, true> : k_affine_wide<1, 8, true>))
-                         : (v == 0 ? k_affine_wide<4, 4, false>
-                                   : (v == 2 ? k_affine_wide<2, 6, false>
-                                             : k_affine_wide<1, 8, false>));
+      auto pick = [&](auto sc, auto lv) {
+        constexpr bool SC = decltype(sc)::value, LV = decltype(lv)::value;
+        return v == 0 ? k_affine_wide<4, LV ? 3 : 4, SC, LV>
+                      : (v == 2 ? k_affine_wide<2, LV ? 5 : 6, SC, LV> : k_affine_wide<1, 8, SC, LV>);
+      };
+      using Yes = std::true_type;
+      using No = std::false_type;
+      auto kern = screen ? (live ? pick(Yes{}, Yes{}) : pick(Yes{}, No{}))
+                         : (live ? pick(No{}, Yes{}) : pick(No{}, No{}));
       e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
       if (e != cudaSuccess) return e;
-      const int max_sm = v == 0 ? 4 : (v == 2 ? 6 : 8);
+      const int max_sm = v == 0 ? (live ? 3 : 4) : (v == 2 ? (live ? 5 : 6) : 8);
       int per_sm = (int)std::min<size_t>(max_sm, (220 * 1024) / (wsmem + 1024));
       if (per_sm < 1) per_sm = 1;
       const int64_t blocks = std::min<int64_t>(n_boxes, device_sms(L) * per_sm);
