@@ -1010,6 +1010,23 @@ static cudaError_t launch_cfg(const Launch& L, int64_t n_boxes, int h_out, int h
   return cudaGetLastError();
 }
 
+static cudaError_t launch_short(const Launch& L, int64_t n_boxes, int h_out, int h_in,
+                                const float* W, const float* b, const float* in_up,
+                                const float* in_lo, int64_t in_ld, const int32_t* in_nterms,
+                                float* out_up, float* out_lo, int64_t out_ld,
+                                int32_t* out_nterms, size_t ssmem) {
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_affine_short, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem);
+  if (e != cudaSuccess) return e;
+  const int per_sm = ssmem <= 54 * 1024 ? 4 : (ssmem <= 72 * 1024 ? 3 : (ssmem <= 110 * 1024 ? 2 : 1));
+  const int64_t blocks = std::min<int64_t>((n_boxes + 3) / 4, device_sms(L) * per_sm);
+  k_affine_short<<<(unsigned)blocks, kWThreads, ssmem, L.stream>>>(
+      n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld, in_nterms, out_up, out_lo, out_ld,
+      out_nterms, L.status);
+  ++*L.launches;
+  return cudaGetLastError();
+}
+
 cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
                           const float* W, const float* b, const float* in_up,
                           const float* in_lo, int64_t in_ld, const int32_t* in_nterms,
@@ -1069,16 +1086,8 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
       e = cudaGetLastError();
       if (screen && screened) *screened = true;
     } else if (v == 4) {
-      e = cudaFuncSetAttribute(k_affine_short, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)ssmem);
-      if (e != cudaSuccess) return e;
-      const int per_sm = ssmem <= 54 * 1024 ? 4 : (ssmem <= 72 * 1024 ? 3 : (ssmem <= 110 * 1024 ? 2 : 1));
-      const int64_t blocks = std::min<int64_t>((n_boxes + 3) / 4, device_sms(L) * per_sm);
-      k_affine_short<<<(unsigned)blocks, kWThreads, ssmem, L.stream>>>(
-          n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld, in_nterms, out_up, out_lo, out_ld,
-          out_nterms, L.status);
-      ++*L.launches;
-      e = cudaGetLastError();
+      e = launch_short(L, n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld, in_nterms, out_up,
+                       out_lo, out_ld, out_nterms, ssmem);
     } else if (few_rows) {
       e = launch_cfg<64, 16, 4, 1, 32>(L, n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld,
                                        in_nterms, out_up, out_lo, out_ld, out_nterms);
@@ -1089,6 +1098,14 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
     tune_end(L, "affine", key, tt);
     return e;
   }
+  // Short polynomials into 17..31 neurons: a warp per box too, once every
+  // resident warp has one (6 rows, 4096 boxes, before and after: 20 -> 20 neurons
+  // 31 and 22 us, 2 -> 20 31 and 11 us, 60 -> 30 56 and 48 us).  Fewer boxes
+  // leave its warps alone with their load latency (300 boxes, 20 -> 20: 6.9 and
+  // 8.8 us), and up to 16 neurons are one block tile (20 -> 9: 18 and 22 us).
+  if (h_out > 16 && few_rows && h_in <= 64 && n_boxes >= 16 * (int64_t)device_sms(L))
+    return launch_short(L, n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld, in_nterms, out_up,
+                        out_lo, out_ld, out_nterms, short_smem(h_out, h_in));
   if (h_out > 8 && few_rows)
     return launch_cfg<16, 16, 2, 1, 32>(L, n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld,
                                         in_nterms, out_up, out_lo, out_ld, out_nterms);

@@ -186,3 +186,48 @@ def test_linearize_step_matches_oracle(ctx):
                     assert np.all(lv >= pv - e)
                 else:
                     assert np.all(lv <= pv + e)
+
+
+@pytest.mark.parametrize("n,D,order", [(1, 1, 1), (1, 12, 4), (2, 1, 2), (2, 14, 3), (2, 15, 3),
+                                       (3, 7, 3), (3, 8, 3), (4, 4, 4), (4, 5, 4), (5, 2, 5)])
+def test_linearize_up_to_and_past_128_terms(ctx, n, D, order):
+    """The fit in a thread per neuron (up to four variables and 128 terms) and in
+    a warp per neuron past that, on ragged prefixes, against the sums in float64."""
+    ld, lin_ld = bern.num_monomials(n, D), bern.num_monomials(n, min(n, order))
+    h, B = 5, 3
+    rng = np.random.default_rng(100 * n + D)
+    up = rng.normal(0, 1, (B, ld, h)).astype(np.float32)
+    lo = up - rng.random((B, ld, h)).astype(np.float32)
+    nt = rng.integers(1, ld + 1, (B, h)).astype(np.int32)
+    nt[0, 0], nt[0, 1], nt[1, 0] = ld, 0, 1
+    t = [torch.from_numpy(x).cuda() for x in (up, lo, nt)]
+    l_up = torch.zeros(B, lin_ld, h, device="cuda")
+    l_lo = torch.zeros_like(l_up)
+    l_nt = torch.zeros(B, h, dtype=torch.int32, device="cuda")
+    r = torch.zeros(2, B, h, device="cuda")
+    ctx.linearize(n, B, h, order, 0, t[0], t[1], ld, t[2], l_up, l_lo, lin_ld, l_nt, r[0], r[1])
+    ctx.check("bern_linearize")
+    ex = graded(n, D)[0].astype(np.float64)
+    sets = np.array([[(S >> k) & 1 for k in range(n)] for S in range(1 << n)], np.float64)
+    w = np.prod(np.where(sets[:, None] > 0, 3 * ex / ((ex + 1) * (ex + 2)), 1 / (ex + 1)), axis=2)
+    # a_T from c_S, S containing T
+    lift = np.array([[2.0 ** T.sum() * (-1.0) ** (S - T).sum() if np.all(S >= T) else 0.0
+                      for S in sets] for T in sets])
+    for src, lin in ((up, l_up.cpu().numpy()), (lo, l_lo.cpu().numpy())):
+        for b in range(B):
+            for m in range(h):
+                k = int(nt[b, m])
+                kl = min(k, lin_ld)
+                assert int(l_nt[b, m]) == kl
+                p = src[b, :k, m].astype(np.float64)
+                a = lift @ (w[:, :k] @ p)
+                # each product, weight and sum rounds once: under ld + 4n + 2^n
+                # roundings of 2^-24 of the sum of absolute values
+                mag = np.abs(lift) @ (w[:, :k] @ np.abs(p))
+                tol = 2.0 ** -24 * (ld + 4 * n + (1 << n) + 4) * mag
+                for q in range(1, kl):
+                    if ex[q].max() > 1:
+                        assert lin[b, q, m] == 0.0
+                        continue
+                    i = int((ex[q].astype(int) << np.arange(n)).sum())
+                    assert abs(lin[b, q, m] - a[i]) <= tol[i], (b, m, q)
