@@ -74,6 +74,6 @@ size_t horner_global_floats(const Tables& T, int Dmax, int cap, int d, int64_t s
 // Launches the float32 kernel when its queue can be non-empty and the
 // float64 one when A.global_d >= kHornerF64Order.
 cudaError_t launch_compose_horner(const Launch& L, const Tables& T, const ComposeScratch& S,
-                                  const ComposeArgs& A, int Dmax);
+                                  const ComposeArgs& A, int64_t n_items, int Dmax);
 
 }  // namespace bern

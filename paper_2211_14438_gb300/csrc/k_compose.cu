@@ -363,7 +363,7 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
   }
   // Horner kernels for orders >= 3, and for every order when pruning
   if (tau > 0.0f || global_d >= 3) {
-    e = launch_compose_horner(L, T, S, A, Dmax);
+    e = launch_compose_horner(L, T, S, A, n_items, Dmax);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();

@@ -37,6 +37,7 @@
 // Work layout.  One block of 256 threads per (item, bound): s~ and the two
 // ends of q (current and next) sit in shared memory; threads take output
 // monomials K of a product and walk the host-built pair list of K (I + J = K).
+// Many small float32 items take k_horner_group instead, several to a warp.
 // Polynomials too large for shared memory keep the same buffers in a slice
 // of a global workspace per block (same arithmetic, same order).
 #include <stdint.h>
@@ -45,6 +46,7 @@
 #include <type_traits>
 
 #include "compose_common.cuh"
+#include "packed.cuh"
 #include "relu_form.cuh"
 
 namespace bern {
@@ -304,6 +306,219 @@ k_compose_horner(Tables T, ComposeArgs A, ComposeScratch S, int ms_cap, int mq_c
   }
 }
 
+// float32 items by groups: a warp takes G items of one bound, lane kl*G + i
+// works on item i and on every KL-th output monomial (KL = 32/G).  s~ and the
+// two ends of q lie in shared memory with the item fastest, the ends as
+// (negated lower, upper) for the packed directed FMA.  A product overwrites q
+// from its last monomial down: monomial K reads q only at ranks <= K, so the
+// KL monomials of a step are read, then (one warp barrier) written.  Same
+// products in the same order as the block form above; only the sums over
+// dropped terms and ||s~||_1 run in another order.  Loop bounds are the warp's
+// maxima, so items of other degrees or orders only idle.
+//
+// Bound: the issue slots of the pair walk (a pair's table entry, two shared
+// loads, a packed FMA).  The block form's 256 threads stood idle on the few
+// monomials of a small polynomial and met at four barriers a product.
+// 4096 boxes of [2,20,20,1] at order 4, layers of 15 and of 153 monomials: 281
+// and 282 us before, 16 and 153 us now.
+constexpr int kGroupWarps = 4;
+
+template <int G>
+__device__ __forceinline__ void horner_group(const Tables& T, const ComposeArgs& A,
+                                             const ComposeScratch& S, int count, int ms_cap,
+                                             int mq_cap, int* status) {
+  using O = Dir<float>;
+  constexpr int KL = 32 / G;
+  constexpr unsigned kAll = 0xffffffffu;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int it = lane % G, kl = lane / G;
+  p2* q = reinterpret_cast<p2*>(smem_raw) + (size_t)warp * mq_cap * G + it;
+  float* s = reinterpret_cast<float*>(reinterpret_cast<p2*>(smem_raw) +
+                                      (size_t)kGroupWarps * mq_cap * G) +
+             (size_t)warp * ms_cap * G + it;
+  auto sum_ru = [&](float v) {
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) v = __fadd_ru(v, __shfl_xor_sync(kAll, v, o));
+    return v;
+  };
+  auto sum_rd = [&](float v) {
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) v = __fadd_rd(v, __shfl_xor_sync(kAll, v, o));
+    return v;
+  };
+  const int h = A.h;
+  const int groups = (count + G - 1) / G;
+  for (int task = blockIdx.x * kGroupWarps + warp; task < 2 * groups;
+       task += gridDim.x * kGroupWarps) {
+    const bool up = task & 1;
+    const int idx = (task >> 1) * G + it;
+    bool ok = idx < count;
+    const int64_t item = S.queue[(int64_t)kQHorner * S.qcap + (ok ? idx : count - 1)];
+    const int Mpre = A.pre_nterms[item];
+    const int D = degree_of(T, Mpre);
+    const int Ms = T.mcount[D];
+    int d = A.degrees ? (int)A.degrees[item] : A.global_d;
+    // shapes the launcher sized the buffers for (checked again here)
+    if (Ms > ms_cap || d < 1 || d > kMaxOrder || T.mcount[min(d * D, A.cap)] > mq_cap) {
+      if (ok && kl == 0) atomicOr(status, kStatusUnsupported);
+      ok = false;
+    }
+    if (!ok) d = 0;
+    const float Lo = A.lo[item];
+    const float inv = 1.0f / (A.hi[item] - Lo);
+    const float* P = (up ? A.pre_up : A.pre_lo) + A.base(item, A.pre_ld);
+    const float* a = A.coef + item * kCoefStride;
+    float l1 = 0.0f;
+    for (int r = kl; r < (ok ? Ms : 0); r += KL) {
+      float v = r < Mpre ? P[(int64_t)r * h] : 0.0f;
+      if (r == 0) v = __fsub_rn(v, Lo);
+      v = __fmul_rn(v, inv);
+      s[r * G] = v;
+      l1 = __fadd_ru(l1, fabsf(v));
+    }
+    l1 = sum_ru(l1);
+    const float eta = __fmul_ru(5.0f * O::u, l1);
+    const float g = __fadd_ru(1.0f, eta);
+    if (ok && kl == 0) q[0] = pack2(-a[d], a[d]);
+    __syncwarp();
+    int Dq = 0;
+    float Rup = 0.0f, Rlo = 0.0f;   // identical in the lanes of an item
+    const int dmax = __reduce_max_sync(kAll, d);
+    for (int t = 0; t < dmax; ++t) {
+      const int j = d - 1 - t;
+      bool act = ok && j >= 0;
+      const int Dp = act ? Dq + D : 0, Dk = min(Dp, A.cap);
+      const int32_t* ptr = nullptr;
+      const int2* pairs = nullptr;
+      int Mp = 0, Mk = 0;
+      float aj = 0.0f;
+      if (act) {
+        const ProdTable pt = T.prod[Dq * kProdStride + D];
+        if (Dp > kMaxTableDegree || pt.ptr == nullptr) {
+          if (kl == 0) atomicOr(status, kStatusUnsupported);
+          ok = act = false;
+        } else {
+          ptr = pt.ptr;
+          pairs = pt.pairs;
+          Mp = T.mcount[Dp];
+          Mk = T.mcount[Dk];
+          aj = a[j];
+        }
+      }
+      // carried remainder rho * s~ (R_lo <= 0 <= R_up)
+      const float cRup = O::fma_ru(-Rlo, eta, O::mul_ru(Rup, g));
+      const float cRlo = O::fma_rd(-Rup, eta, O::mul_rd(Rlo, g));
+      float dru = 0.0f, drl = 0.0f;
+      const int Mw = __reduce_max_sync(kAll, Mp);
+      for (int top = Mw - 1; top >= 0; top -= KL) {
+        const int K = top - kl;
+        const bool on = K >= 0 && K < Mp;
+        p2 acc = 0;
+        if (on) {
+          if (K == 0) acc = pack2(-aj, aj);
+          const int p1 = __ldg(ptr + K + 1);
+#pragma unroll 4
+          for (int p = __ldg(ptr + K); p < p1; ++p) {
+            const int2 pr = __ldg(pairs + p);
+            const float sv = s[pr.y * G];
+            float nlo, hi;
+            unpack2(q[pr.x * G], nlo, hi);
+            // a negative factor swaps the ends: up by (-lo)|s~|, -lo by up|s~|
+            const bool pos = sv >= 0.0f;
+            const float av = fabsf(sv);
+            acc = fma2_ru(pack2(pos ? nlo : hi, pos ? hi : nlo), pack2(av, av), acc);
+          }
+        }
+        if (KL > 1) __syncwarp();
+        if (on) {
+          if (K < Mk) {
+            q[K * G] = acc;
+          } else {
+            float nlo, hi;
+            unpack2(acc, nlo, hi);
+            dru = __fadd_ru(dru, fmaxf(hi, 0.0f));
+            drl = __fadd_rd(drl, fminf(-nlo, 0.0f));
+          }
+        }
+      }
+      __syncwarp();
+      dru = sum_ru(dru);
+      drl = sum_rd(drl);
+      float pru = 0.0f, prl = 0.0f;
+      if (A.tau > 0.0f) {
+        // pruning (relative to the L1 norm of this bound's end of q)
+        auto end = [&](int K) {
+          float nlo, hi;
+          unpack2(q[K * G], nlo, hi);
+          return fabsf(up ? hi : nlo);
+        };
+        float nrm = 0.0f;
+        for (int K = kl; K < Mk; K += KL) nrm = __fadd_ru(nrm, end(K));
+        nrm = sum_ru(nrm);
+        const float thr = A.tau * nrm;
+        for (int K = 1 + kl; K < Mk; K += KL) {
+          if (end(K) < thr) {
+            float nlo, hi;
+            unpack2(q[K * G], nlo, hi);
+            pru = __fadd_ru(pru, fmaxf(hi, 0.0f));
+            prl = __fadd_rd(prl, fminf(-nlo, 0.0f));
+            q[K * G] = 0;
+          }
+        }
+        pru = sum_ru(pru);
+        prl = sum_rd(prl);
+        __syncwarp();
+      }
+      if (act) {
+        Rup = __fadd_ru(__fadd_ru(cRup, dru), pru);
+        Rlo = __fadd_rd(__fadd_rd(cRlo, drl), prl);
+        Dq = Dk;
+      }
+    }
+    const int Mout = ok ? T.mcount[Dq] : 0;
+    float* Q = (up ? A.post_up : A.post_lo) + A.base(item, A.post_ld);
+    int nz = 1;
+    for (int K = 1 + kl; K < Mout; K += KL) {
+      float nlo, hi;
+      unpack2(q[K * G], nlo, hi);
+      const float v = up ? hi : -nlo;
+      Q[(int64_t)K * h] = v;
+      if (v != 0.0f) nz = K + 1;
+    }
+    if (A.tau > 0.0f) {
+#pragma unroll
+      for (int o = G; o < 32; o <<= 1) nz = max(nz, __shfl_xor_sync(kAll, nz, o));
+    }
+    if (ok && kl == 0) {
+      const float le = __fmul_ru(horner_lip(a, d, eta), eta);
+      float nlo, hi;
+      unpack2(q[0], nlo, hi);
+      const float v = up ? __fadd_ru(__fadd_ru(hi, Rup), le)
+                         : __fsub_rd(__fsub_rd(__fadd_rd(-nlo, Rlo), le), A.eps[item]);
+      Q[0] = v;
+      if (!isfinite(v)) atomicOr(status, kStatusNonFinite);
+      // with pruning, the term count is the graded prefix up to the highest
+      // degree with a kept term (both bounds share it)
+      if (A.tau > 0.0f) atomicMax(&A.post_nterms[item], T.mcount[degree_of(T, nz)]);
+    }
+    __syncwarp();
+  }
+}
+
+// Up to `few` queued items (the host knows only the neurons of the call) take a
+// warp each: there G items in a warp leave schedulers idle.
+template <int G>
+__global__ void __launch_bounds__(32 * kGroupWarps)
+k_horner_group(Tables T, ComposeArgs A, ComposeScratch S, int ms_cap, int mq_cap, int few,
+               int* status) {
+  const int count = S.qcount[kQHorner];
+  if (G == 1 || count < few)
+    horner_group<1>(T, A, S, count, ms_cap, mq_cap, status);
+  else
+    horner_group<G>(T, A, S, count, ms_cap, mq_cap, status);
+}
+
 }  // namespace
 
 namespace {
@@ -328,9 +543,28 @@ bool in_global(size_t floats, int64_t smem_limit) {
   return (int64_t)(floats * sizeof(float)) > std::min<int64_t>(smem_limit, 200 * 1024);
 }
 
+size_t group_smem(int G, int ms, int mq) {
+  return (size_t)kGroupWarps * G * ((size_t)ms * sizeof(float) + (size_t)mq * sizeof(p2));
+}
+
+// Items per warp of k_horner_group, 0 for a block per item.  By the buffers of a
+// block of four warps: eight or four items up to 20 KB, two or one up to 32 KB
+// (passes over 2000 boxes with 8 / 4 / 2 / 1 items a warp and a block per item,
+// us: [3,64,1] order 3, 20 monomials 78 / 81 / 90 / 112 / 364; [2,20,20,1] order
+// 4, 153 monomials 224 / 198 / 186 / 204 / 383; [4,20,20,1] order 3, 715
+// monomials - / - / 632 / 572 / 816).  Under 16 neurons per multiprocessor a
+// block per item ends sooner: all of its warps work on the one product
+// ([3,32,32,1], orders 3 and 4, 8 boxes: 111 against 134 us).
+int group_items(const Launch& L, int64_t n_items, int ms, int mq) {
+  if (n_items < 16 * (int64_t)device_sms(L)) return 0;
+  for (int G : {8, 4, 2, 1})
+    if (group_smem(G, ms, mq) <= (G > 2 ? 20 : 32) * 1024) return G;
+  return 0;
+}
+
 template <typename R>
 cudaError_t launch_variant(const Launch& L, const Tables& T, const ComposeScratch& S,
-                           const ComposeArgs& A, int Dmax, int Dout) {
+                           const ComposeArgs& A, int64_t n_items, int Dmax, int Dout) {
   constexpr bool kF64 = std::is_same<R, double>::value;
   const size_t floats = variant_floats(T, Dmax, Dout, kF64);
   if (floats == SIZE_MAX) return cudaErrorInvalidValue;
@@ -342,6 +576,21 @@ cudaError_t launch_variant(const Launch& L, const Tables& T, const ComposeScratc
         T, A, S, ms_cap, mq_cap, S.hws, (int64_t)floats, L.status);
     ++*L.launches;
     return cudaGetLastError();
+  }
+  if constexpr (!kF64) {
+    const int G = group_items(L, n_items, ms_cap, mq_cap);
+    if (G) {
+      auto kern = G == 8   ? k_horner_group<8>
+                  : G == 4 ? k_horner_group<4>
+                  : G == 2 ? k_horner_group<2>
+                           : k_horner_group<1>;
+      const size_t gsmem = group_smem(G, ms_cap, mq_cap);
+      const int per_sm = std::max(1, std::min(10, (int)((224 * 1024) / (gsmem + 1024))));
+      kern<<<device_sms(L) * per_sm, 32 * kGroupWarps, gsmem, L.stream>>>(
+          T, A, S, ms_cap, mq_cap, 64 * device_sms(L), L.status);
+      ++*L.launches;
+      return cudaGetLastError();
+    }
   }
   const size_t smem = floats * sizeof(float);
   if (smem > 48 * 1024) {
@@ -380,15 +629,15 @@ size_t horner_global_floats(const Tables& T, int Dmax, int cap, int d, int64_t s
 }
 
 cudaError_t launch_compose_horner(const Launch& L, const Tables& T, const ComposeScratch& S,
-                                  const ComposeArgs& A, int Dmax) {
+                                  const ComposeArgs& A, int64_t n_items, int Dmax) {
   const int d = std::max(1, A.global_d);
   const bool f64 = d >= kHornerF64Order;
   // float32 items exist unless every item has order d >= kHornerF64Order
   if ((A.tau > 0.0f || d >= 3) && (A.degrees != nullptr || !f64)) {
-    cudaError_t e = launch_variant<float>(L, T, S, A, Dmax, dout_f32(Dmax, A.cap, d));
+    cudaError_t e = launch_variant<float>(L, T, S, A, n_items, Dmax, dout_f32(Dmax, A.cap, d));
     if (e != cudaSuccess) return e;
   }
-  if (f64) return launch_variant<double>(L, T, S, A, Dmax, dout_f64(Dmax, A.cap, d));
+  if (f64) return launch_variant<double>(L, T, S, A, n_items, Dmax, dout_f64(Dmax, A.cap, d));
   return cudaSuccess;
 }
 

@@ -300,3 +300,48 @@ def test_six_inputs_cap16_pruned(ctx):
     assert np.all(np.abs(g1["lo"] - g0["lo"]) <= 1e-3 * scale)
     for bi in range(len(boxes)):
         assert mc_check(g1, bi, w.net, boxes[bi], 5_000, rng) == 0
+
+
+@pytest.mark.parametrize("n,D,d,cap,tau", [
+    (2, 1, 3, 16, 0.0), (2, 4, 4, 16, 0.0), (2, 4, 4, 9, 0.0), (3, 2, 3, 16, 0.0),
+    (3, 5, 3, 16, 0.0), (4, 1, 2, 16, 0.0625), (2, 4, 3, 8, 0.0625), (1, 2, 4, 5, 0.03125),
+    (6, 1, 1, 16, 0.125)])
+def test_several_items_a_warp_equal_a_block_per_item(ctx, n, D, d, cap, tau):
+    """Many neurons in one call (several to a warp, one to a warp when few of
+    them compose) against the same neurons in slices that take a block each.
+    Coefficients are small dyadic numbers, so every sum is exact whatever its
+    order and the results agree bit for bit, pruning included."""
+    B, h = 300, 41                                   # 12,300 neurons
+    M = bern.num_monomials(n, D)
+    keep = bern.num_monomials(n, min(max(d, 1) * D, cap))
+    rng = np.random.default_rng(1000 * n + 100 * D + 10 * d + cap)
+    up = (rng.integers(-4, 5, (B, M, h)) / 4 * (rng.random((B, M, h)) < 0.5)).astype(np.float32)
+    lo = (up - rng.integers(0, 3, (B, M, h)) / 4).astype(np.float32)
+    nt = rng.choice([M, M, max(1, M - 1), n + 1, 1], (B, h)).astype(np.int32)
+    L = np.full((B, h), -1.0, np.float32)
+    H = np.full((B, h), 1.0, np.float32)
+    coef = np.zeros((B, h, bern.COEF_STRIDE), np.float32)
+    coef[..., :d + 1] = rng.integers(0, 5, (B, h, d + 1)) / 8
+    eps = (rng.integers(0, 5, (B, h)) / 64).astype(np.float32)
+    dg = rng.integers(max(1, d - 1), d + 1, (B, h)).astype(np.uint8)
+    few = rng.random((B, h)) < 0.05                  # the second call: most are copied or dead
+    for kind in (np.full((B, h), 2, np.int8), np.where(few, 2, rng.integers(0, 2, (B, h)))):
+        kind = kind.astype(np.int8)
+        for degrees in (None, dg):
+            def run(sl):
+                t = {k: torch.from_numpy(np.ascontiguousarray(v[sl])).cuda() for k, v in
+                     dict(up=up, lo=lo, nt=nt, L=L, H=H, coef=coef, eps=eps, kind=kind,
+                          dg=dg).items()}
+                nb = len(t["nt"])
+                pu = torch.full((nb, max(keep, M), h), 7.0, device="cuda")
+                pl = torch.full_like(pu, 7.0)
+                pn = torch.zeros(nb, h, dtype=torch.int32, device="cuda")
+                ctx.compose(n, nb, h, cap, tau, t["kind"], t["coef"], t["eps"],
+                            None if degrees is None else t["dg"], d, t["L"], t["H"], t["up"],
+                            t["lo"], M, t["nt"], pu, pl, pu.shape[1], pn)
+                ctx.check("compose")
+                return [x.cpu().numpy() for x in (pu, pl, pn)]
+            whole = run(slice(0, B))
+            for s in range(0, B, 50):                # 2050 neurons
+                for a, b in zip(run(slice(s, s + 50)), whole):
+                    assert np.array_equal(a, b[s:s + 50])
