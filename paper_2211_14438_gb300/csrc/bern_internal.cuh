@@ -313,6 +313,7 @@ cudaError_t launch_pack(const Launch& L, const Tables& T, int64_t n_boxes, int o
 constexpr int kComposeQueues = kMaxRowDegree + 6;
 // Lists for the per-box Bernstein orders of learned plans (one per order value).
 constexpr int kOrderQueues = 32;
+constexpr int kQueueThreads = 512;   // items per block of the queueing kernels
 constexpr int kQueueLists = kComposeQueues > kOrderQueues ? kComposeQueues : kOrderQueues;
 struct ComposeScratch {
   int* qcount;       // kComposeQueues counters (zeroed by the launcher)

@@ -57,6 +57,38 @@ __device__ float block_dsum(float v, float* scratch) {
   return r;
 }
 
+// Appends the block's items to NQ work lists in item order (q: the thread's list,
+// -1 none): the rank of equal lists within a warp, a scan over the warps by one
+// warp per list, one atomic per list and block.  Called by every thread of a block
+// of whole warps.
+template <int NQ>
+__device__ __forceinline__ void append_to_lists(int q, int item, int* qcount, int32_t* queue,
+                                                int64_t qcap) {
+  constexpr int S = NQ | 1;                  // odd stride: a list's column without conflicts
+  __shared__ int s_at[32 * S];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int i = threadIdx.x; i < 32 * S; i += blockDim.x) s_at[i] = 0;
+  __syncthreads();
+  const unsigned same = __match_any_sync(0xffffffffu, q);
+  const int rank = __popc(same & ((1u << lane) - 1u));
+  if (q >= 0 && rank == 0) s_at[warp * S + q] = __popc(same);
+  __syncthreads();
+  for (int l = warp; l < NQ; l += nw) {
+    const int c = s_at[lane * S + l];
+    int run = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += v;
+    }
+    int base = 0;
+    if (lane == 31 && run) base = atomicAdd(&qcount[l], run);
+    s_at[lane * S + l] = __shfl_sync(0xffffffffu, base, 31) + run - c;
+  }
+  __syncthreads();
+  if (q >= 0) queue[(int64_t)q * qcap + s_at[warp * S + q] + rank] = item;
+}
+
 // Exact binomials C(l,k), l,k <= 24 (all < 2^24, so exact in float32).
 struct BinomTable {
   float v[kMaxEncloseOrder + 1][kMaxEncloseOrder + 1];

@@ -30,17 +30,13 @@
 namespace bern {
 
 // ------------------------------------------------------------ classification
-// Each block classifies 1024 consecutive items and appends them to the
-// queues in item order (ballot/popc within a warp, a scan over the warps),
-// reserving its range of every queue with one atomic; so a queue is a list
-// of sorted runs, and a warp's 32 consecutive entries are mostly neighbouring
-// neurons of one box.
-__global__ void __launch_bounds__(1024)
+// Each block classifies kQueueThreads consecutive items and appends them to the
+// queues in item order, reserving its range of every queue with one atomic; so a
+// queue is a list of sorted runs, and a warp's 32 consecutive entries are mostly
+// neighbouring neurons of one box.
+__global__ void __launch_bounds__(kQueueThreads)
 k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int sq_dmax, ComposeScratch S,
                 int* status) {
-  __shared__ int s_wcnt[32][kComposeQueues];
-  __shared__ int s_base[kComposeQueues];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int q = -1;
   if (item < n_items) {
@@ -84,25 +80,7 @@ k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int sq_dmax, ComposeSc
     }
     A.post_nterms[item] = nt;
   }
-  int rank_in_warp = 0;
-  for (int qq = 0; qq < kComposeQueues; ++qq) {
-    const unsigned m = __ballot_sync(0xffffffffu, q == qq);
-    if (q == qq) rank_in_warp = __popc(m & ((1u << lane) - 1u));
-    if (lane == 0) s_wcnt[warp][qq] = __popc(m);
-  }
-  __syncthreads();
-  if (threadIdx.x < kComposeQueues) {
-    const int qq = threadIdx.x;
-    int run = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {   // exclusive scan over warps
-      const int c = s_wcnt[w][qq];
-      s_wcnt[w][qq] = run;
-      run += c;
-    }
-    s_base[qq] = run ? atomicAdd(&S.qcount[qq], run) : 0;
-  }
-  __syncthreads();
-  if (q >= 0) S.queue[(int64_t)q * S.qcap + s_base[q] + s_wcnt[warp][q] + rank_in_warp] = (int)item;
+  append_to_lists<kComposeQueues>(q, (int)item, S.qcount, S.queue, S.qcap);
 }
 
 // ------------------------------------------------------------ elementwise items
@@ -145,29 +123,34 @@ k_compose_copy(ComposeArgs A, ComposeScratch S) {
   }
 }
 
-// Order-1 items: a0 + a1*s~ for both bounds, one warp per item.
-__global__ void __launch_bounds__(256)
-k_compose_linear(ComposeArgs A, ComposeScratch S, int* status) {
+// Order-1 items: a_0 + a_1 s~ for both bounds.  A warp takes G entries of the
+// queue, lane kl*G + i row kl, kl + 32/G, ... of entry i: eight entries are
+// mostly neighbouring neurons, whose rows then come and go in whole sectors.
+template <int G>
+__device__ __forceinline__ void compose_linear(const ComposeArgs& A, const ComposeScratch& S,
+                                               int n_lin, int* status) {
+  constexpr int KL = 32 / G;
   const int lane = threadIdx.x & 31;
+  const int i = lane % G, kl = lane / G;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int n_lin = S.qcount[kQLinear];
-  const int h = A.h;
-  for (int t = gw; t < n_lin; t += nw) {
-    const int64_t item = S.queue[(int64_t)kQLinear * S.qcap + t];
+  const int64_t h = A.h;
+  for (int64_t t = (int64_t)gw * G; t < n_lin; t += (int64_t)nw * G) {
+    const bool on = t + i < n_lin;
+    const int64_t item = S.queue[(int64_t)kQLinear * S.qcap + (on ? t + i : t)];
     const int Mpre = A.pre_nterms[item];
-    const float* Pu = A.pre_up + A.base(item, A.pre_ld);
-    const float* Pl = A.pre_lo + A.base(item, A.pre_ld);
-    float* Qu = A.post_up + A.base(item, A.post_ld);
-    float* Ql = A.post_lo + A.base(item, A.post_ld);
+    const int64_t src = A.base(item, A.pre_ld), dst = A.base(item, A.post_ld);
+    const float* Pu = A.pre_up + src;
+    const float* Pl = A.pre_lo + src;
+    float* Qu = A.post_up + dst;
+    float* Ql = A.post_lo + dst;
     const float Lo = A.lo[item], Hi = A.hi[item];
     const float inv = 1.0f / (Hi - Lo);
     const float* cf = A.coef + item * kCoefStride;
     const float a0 = cf[0], a1 = cf[1];
-    const int Mout = A.post_nterms[item];     // the graded prefix of Mpre's degree
+    const int Mout = on ? A.post_nterms[item] : 0;   // the graded prefix of Mpre's degree
     float lu = 0.0f, ll = 0.0f, cu0 = 0.0f, cl0 = 0.0f;
-    for (int r = lane; r < Mout; r += 32) {
-      float vu = r < Mpre ? Pu[(int64_t)r * h] : 0.0f, vl = r < Mpre ? Pl[(int64_t)r * h] : 0.0f;
+    auto row = [&](int r, float vu, float vl) {
       if (r == 0) {
         vu = __fsub_rn(vu, Lo);
         vl = __fsub_rn(vl, Lo);
@@ -182,13 +165,31 @@ k_compose_linear(ComposeArgs A, ComposeScratch S, int* status) {
         cu0 = cu;
         cl0 = cl;
       } else {
-        Qu[(int64_t)r * h] = cu;
-        Ql[(int64_t)r * h] = cl;
+        Qu[r * h] = cu;
+        Ql[r * h] = cl;
       }
+    };
+    int r = kl;
+    for (; r + 3 * KL < Mout; r += 4 * KL) {   // four rows of both bounds in flight
+      float vu[4], vl[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int rr = r + q * KL;
+        vu[q] = rr < Mpre ? Pu[rr * h] : 0.0f;
+        vl[q] = rr < Mpre ? Pl[rr * h] : 0.0f;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) row(r + q * KL, vu[q], vl[q]);
     }
-    lu = warp_dsum<true>(lu);
-    ll = warp_dsum<true>(ll);
-    if (lane == 0) {
+    for (; r < Mout; r += KL)
+      row(r, r < Mpre ? Pu[r * h] : 0.0f, r < Mpre ? Pl[r * h] : 0.0f);
+    __syncwarp();
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) {
+      lu = __fadd_ru(lu, __shfl_xor_sync(0xffffffffu, lu, o));
+      ll = __fadd_ru(ll, __shfl_xor_sync(0xffffffffu, ll, o));
+    }
+    if (on && kl == 0) {
       const float lip = fabsf(a1);
       const float eu = __fmul_ru(5.0f * kU, lu), el = __fmul_ru(5.0f * kU, ll);
       const float vu = __fadd_ru(cu0, __fmul_ru(lip, eu));
@@ -198,6 +199,18 @@ k_compose_linear(ComposeArgs A, ComposeScratch S, int* status) {
       if (!isfinite(vu) || !isfinite(vl)) atomicOr(status, kStatusNonFinite);
     }
   }
+}
+
+// Eight entries a warp once that leaves each scheduler one or more warps (5120
+// boxes of [3,64x4,1] with learned orders, the four layers: 23, 29, 49 and 88 us
+// at an entry a warp, now 9, 11, 14 and 19 us), one below.
+__global__ void __launch_bounds__(256)
+k_compose_linear(ComposeArgs A, ComposeScratch S, int few, int* status) {
+  const int n_lin = S.qcount[kQLinear];
+  if (n_lin < few)
+    compose_linear<1>(A, S, n_lin, status);
+  else
+    compose_linear<8>(A, S, n_lin, status);
 }
 
 // ------------------------------------------------------------ pair-list squaring
@@ -326,7 +339,8 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
                                S.tws ? square_max_degree(T.n) : square_smem_degree(T.n));
   cudaError_t e = cudaMemsetAsync(S.qcount, 0, kComposeQueues * sizeof(int), L.stream);
   if (e != cudaSuccess) return e;
-  k_compose_queue<<<(unsigned)((n_items + 1023) / 1024), 1024, 0, L.stream>>>(
+  k_compose_queue<<<(unsigned)((n_items + kQueueThreads - 1) / kQueueThreads), kQueueThreads, 0,
+                    L.stream>>>(
       T, A, n_items, sq_dmax, S, L.status);
   ++*L.launches;
   // order-2 items exist only with order 2 somewhere in the plan (with pruning
@@ -345,7 +359,7 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
   // they go to the Horner kernel)
   if (tau == 0.0f && (degrees != nullptr || global_d == 1)) {
     k_compose_linear<<<(unsigned)std::min<int64_t>((n_items + 7) / 8, device_sms(L) * 16), 256,
-                       0, L.stream>>>(A, S, L.status);
+                       0, L.stream>>>(A, S, 32 * device_sms(L), L.status);
     ++*L.launches;
   }
   // pair-list kernel for order-2 items beyond the squaring kernels

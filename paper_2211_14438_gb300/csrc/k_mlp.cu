@@ -82,7 +82,16 @@ k_degree_features(int64_t n, const float* __restrict__ lo, const float* __restri
   }
 }
 
-// One block per box; threads over the box's neurons.
+// The proposals of a box by a warp, two neurons per lane at a time.  Weights in
+// shared memory at the proposals' own sizes (8 features, 4 classes), four values
+// per load, each load for both neurons; the products and their order are those
+// of mlp_logits, whose padding only adds zeros.
+//
+// Bound: FMA issue and the shared loads that feed it (half each).  A block of 128
+// threads per box at the padded sizes took 39 us for 5120 boxes of 64 neurons,
+// this 25 us.
+static_assert(kDegFeatures <= 8 && kDegClasses <= 4, "proposal weights are two and one float4");
+
 __global__ void __launch_bounds__(128)
 k_learned_degrees(MlpView M, int64_t n_boxes, int h, int layer, const float* __restrict__ lo,
                   const float* __restrict__ hi, const int32_t* __restrict__ pre_nterms,
@@ -91,43 +100,79 @@ k_learned_degrees(MlpView M, int64_t n_boxes, int h, int layer, const float* __r
                   int32_t* __restrict__ order_out, uint8_t* __restrict__ degrees,
                   int8_t* __restrict__ kind, float* __restrict__ coef, float* __restrict__ eps,
                   int* status) {
-  __shared__ SmemMlp S;
-  __shared__ int s_max;
-  stage_mlp(M, S);
-  for (int64_t b = blockIdx.x; b < n_boxes; b += gridDim.x) {
-    if (threadIdx.x == 0) s_max = 1;
-    __syncthreads();
+  __shared__ float4 s_w1[kH][2], s_w2[kH];
+  __shared__ float s_b1[kH], s_b2[4];
+  for (int i = threadIdx.x; i < kH * 8; i += blockDim.x) {
+    const int j = i >> 3, f = i & 7;
+    reinterpret_cast<float*>(s_w1)[i] =
+        f < kDegFeatures ? __bfloat162float(M.W1[j * kDegFeatures + f]) : 0.0f;
+  }
+  for (int i = threadIdx.x; i < kH * 4; i += blockDim.x) {
+    const int j = i >> 2, c = i & 3;
+    reinterpret_cast<float*>(s_w2)[i] = c < kDegClasses ? __bfloat162float(M.W2[c * kH + j]) : 0.0f;
+  }
+  for (int i = threadIdx.x; i < kH; i += blockDim.x) s_b1[i] = M.b1[i];
+  if (threadIdx.x < 4) s_b2[threadIdx.x] = threadIdx.x < kDegClasses ? M.b2[threadIdx.x] : 0.0f;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  for (int64_t b = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5); b < n_boxes;
+       b += (int64_t)gridDim.x * warps) {
     int dmax = 1;
-    for (int m = threadIdx.x; m < h; m += blockDim.x) {
-      const int64_t it = b * h + m;
-      const float l = lo[it], u = hi[it];
-      float f[kDegFeatures], xb[kMlpMaxF], z[kMlpMaxC];
-      degree_feature_vec(l, u, pre_nterms[it], layer, f);
+    for (int m = lane; m < h; m += 64) {
+      float l[2], u[2], xb[2][8], z[2][4];
 #pragma unroll
-      for (int k = 0; k < kMlpMaxF; ++k) xb[k] = k < kDegFeatures ? bf16_round(f[k]) : 0.0f;
-      mlp_logits(S, xb, z);
-      int best = 0;
-      float zb = z[0];
+      for (int q = 0; q < 2; ++q) {
+        const int64_t it = b * h + min(m + 32 * q, h - 1);
+        l[q] = lo[it];
+        u[q] = hi[it];
+        float f[kDegFeatures];
+        degree_feature_vec(l[q], u[q], pre_nterms[it], layer, f);
 #pragma unroll
-      for (int c = 1; c < kDegClasses; ++c)
-        if (z[c] > zb) {   // first maximum wins ties
-          zb = z[c];
-          best = c;
+        for (int k = 0; k < 8; ++k) xb[q][k] = k < kDegFeatures ? bf16_round(f[k]) : 0.0f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) z[q][c] = s_b2[c];
+      }
+#pragma unroll 4
+      for (int j = 0; j < kH; ++j) {
+        const float4 wa = s_w1[j][0], wb = s_w1[j][1], v = s_w2[j];
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+        const float v4[4] = {v.x, v.y, v.z, v.w};
+        const float b1 = s_b1[j];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          float acc = b1;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) acc = fmaf(w[k], xb[q][k], acc);
+          const float a = bf16_round(fmaxf(acc, 0.0f));
+#pragma unroll
+          for (int c = 0; c < 4; ++c) z[q][c] = fmaf(v4[c], a, z[q][c]);
         }
-      float sum = 0.0f;
+      }
 #pragma unroll
-      for (int c = 0; c < kDegClasses; ++c) sum += expf(z[c] - zb);
-      const float conf = 1.0f / sum;   // the largest softmax probability
-      const int d = min(conf >= min_conf ? best + 1 : fallback_d, max_d);
-      degrees[it] = (uint8_t)d;
-      kind[it] = (int8_t)relu_item(l, u, d, coef + it * kCoefStride, eps + it, status);
-      dmax = max(dmax, d);
+      for (int q = 0; q < 2; ++q) {
+        if (m + 32 * q >= h) continue;
+        const int64_t it = b * h + m + 32 * q;
+        int best = 0;
+        float zb = z[q][0];
+#pragma unroll
+        for (int c = 1; c < kDegClasses; ++c)
+          if (z[q][c] > zb) {   // first maximum wins ties
+            zb = z[q][c];
+            best = c;
+          }
+        float sum = 0.0f;
+#pragma unroll
+        for (int c = 0; c < kDegClasses; ++c) sum += expf(z[q][c] - zb);
+        const float conf = 1.0f / sum;   // the largest softmax probability
+        const int d = min(conf >= min_conf ? best + 1 : fallback_d, max_d);
+        degrees[it] = (uint8_t)d;
+        kind[it] = (int8_t)relu_item(l[q], u[q], d, coef + it * kCoefStride, eps + it, status);
+        dmax = max(dmax, d);
+      }
     }
+    __syncwarp();
     dmax = warp_imax(dmax);
-    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, dmax);
-    __syncthreads();
-    if (threadIdx.x == 0) order_out[b] = min(cap, order_in[b] * s_max);
-    __syncthreads();
+    if (lane == 0) order_out[b] = min(cap, order_in[b] * dmax);
   }
 }
 
@@ -388,7 +433,7 @@ cudaError_t launch_learned_degrees(const Launch& L, const MlpView& M, int64_t n_
                                    float* coef, float* eps) {
   if (n_boxes == 0) return cudaSuccess;
   if (M.F != kDegFeatures || M.C != kDegClasses) return cudaErrorInvalidValue;
-  k_learned_degrees<<<grid_for(n_boxes, 1, device_sms(L) * 16), 128, 0, L.stream>>>(
+  k_learned_degrees<<<grid_for(n_boxes, 4, device_sms(L) * 16), 128, 0, L.stream>>>(
       M, n_boxes, h, layer, lo, hi, pre_nterms, min_conf, fallback_d, max_d, cap, order_in,
       order_out,
       degrees, kind, coef, eps, L.status);
