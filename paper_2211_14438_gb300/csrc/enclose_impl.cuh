@@ -298,11 +298,13 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
   tune_begin(L, "enclose", tt);
   const size_t smem = (size_t)2 * items * G * sizeof(float);
   // the in-simplex prefix loop for four or more variables (their grids of
-  // l >= 12, 13^4 cells and more, exceed kEncloseGridMax and run elsewhere)
-  auto kern = k_enclose<LB, false, 0>;
-  if constexpr (LB >= 4)   // three-variable grids of l <= 3 take the small-grid kernel
+  // l >= 12, 13^4 cells and more, exceed kEncloseGridMax and run elsewhere);
+  // fewer variables come here from order 8 on (one) and 9 on (two and three),
+  // their lower orders run in k_enclose_small and k_enclose_tail.cu
+  auto kern = k_enclose<LB, (LB < 8), 0>;
+  if constexpr (LB > 8)
     if (T.n == 3) kern = k_enclose<LB, false, 3>;
-  if constexpr (LB <= 11)
+  if constexpr (LB >= 8 && LB <= 11)
     if (T.n >= 4) kern = k_enclose<LB, true, 0>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -318,7 +320,7 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
   return e;
 }
 
-// Tiny grids ((l+1)^n <= 64): one lane per polynomial, the lane's grid
+// Tiny grids ((l+1)^n <= 64: order 0, and one variable up to order 7): one lane per polynomial, the lane's grid
 // interleaved with its warp's (element g of lane L at grid[g*32 + L]); a warp
 // takes 32 items of one bound, a block 4 groups of 32 items (both bounds).
 constexpr int kSmallGrid = 64;
@@ -347,8 +349,7 @@ __device__ float enclose_lane(const float* __restrict__ P, int ps, int nt, int n
   const int nlines = ipow(R, n - 1);
   for (int k = n - 1; k >= 0; --k) {
     const int sk = ipow(R, n - 1 - k);
-    const int nl = n >= 4 ? simplex_lines(LB, k, sk) : nlines;
-    for (int Ln = 0; Ln < nl; ++Ln) {
+    for (int Ln = 0; Ln < nlines; ++Ln) {
       const int2 ln = __ldg(lines + (int64_t)k * nlines + Ln);
       const int base = ln.x, psum = ln.y;
       if (psum > Deff) continue;

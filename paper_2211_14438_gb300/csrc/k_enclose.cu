@@ -168,8 +168,8 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
 #define BERN_SMALL_CASE(X) \
   case X: return launch_small<X>(L, T, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
     switch (lb) {
-      BERN_SMALL_CASE(0) BERN_SMALL_CASE(1) BERN_SMALL_CASE(2) BERN_SMALL_CASE(3)
-      BERN_SMALL_CASE(4) BERN_SMALL_CASE(5) BERN_SMALL_CASE(6) BERN_SMALL_CASE(7)
+      BERN_SMALL_CASE(0) BERN_SMALL_CASE(2) BERN_SMALL_CASE(3) BERN_SMALL_CASE(4)
+      BERN_SMALL_CASE(5) BERN_SMALL_CASE(6) BERN_SMALL_CASE(7)
       default: break;
     }
 #undef BERN_SMALL_CASE
@@ -177,7 +177,7 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
 #define BERN_ENC_CASE(X) \
   case X: return launch_lb<X>(L, T, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
   switch (lb) {
-    BERN_ENC_CASE(0) BERN_ENC_CASE(1) BERN_ENC_CASE(2) BERN_ENC_CASE(3) BERN_ENC_CASE(4)
+    BERN_ENC_CASE(2) BERN_ENC_CASE(3) BERN_ENC_CASE(4)
     BERN_ENC_CASE(5) BERN_ENC_CASE(6) BERN_ENC_CASE(7) BERN_ENC_CASE(8) BERN_ENC_CASE(9)
     BERN_ENC_CASE(10) BERN_ENC_CASE(11) BERN_ENC_CASE(12) BERN_ENC_CASE(13) BERN_ENC_CASE(14)
     BERN_ENC_CASE(15) BERN_ENC_CASE(16)

@@ -1,7 +1,8 @@
 // a2 for Bernstein grids larger than shared memory (Sec. 5.1 Step 1 with
 // Def. 2, the full tensor-product grid of order l in every variable):
-// (l+1)^n cells up to the caller's budget, e.g. 9^6 = 531,441 cells for six
-// inputs at order 8.  One block per polynomial works on its own slice of a
+// (l+1)^n cells up to the caller's budget, e.g. 13^5 = 371,293 cells for five
+// inputs at order 12; orders up to 10 of four and more variables run in
+// k_enclose_slab.cu, order 10 of six here.  One block per polynomial works on its own slice of a
 // global workspace (resident in L2 while the block runs): the scaled
 // coefficients are scattered to their grid cells, then the per-variable
 // triangular transforms run from the last variable to the first, the threads
@@ -260,12 +261,12 @@ cudaError_t launch_enclose_big(const Launch& L, const Tables& T, int lb, int G, 
                                const int32_t* nterms, float* lo, float* hi, const int* list,
                                const int* count) {
   if (!L.ews || lb > T.rscale_max || !T.rscale[lb] || !T.gidx[lb]) return cudaErrorInvalidValue;
+  // lower orders fit the slab kernels with any number of variables
 #define BERN_BIG_CASE(X) \
   case X: return launch_big_lb<X>(L, T, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, list, count);
   switch (lb) {
-    BERN_BIG_CASE(2) BERN_BIG_CASE(3) BERN_BIG_CASE(4) BERN_BIG_CASE(5) BERN_BIG_CASE(6)
-    BERN_BIG_CASE(7) BERN_BIG_CASE(8) BERN_BIG_CASE(9) BERN_BIG_CASE(10) BERN_BIG_CASE(11)
-    BERN_BIG_CASE(12) BERN_BIG_CASE(13) BERN_BIG_CASE(14) BERN_BIG_CASE(15) BERN_BIG_CASE(16)
+    BERN_BIG_CASE(10) BERN_BIG_CASE(11) BERN_BIG_CASE(12) BERN_BIG_CASE(13) BERN_BIG_CASE(14)
+    BERN_BIG_CASE(15) BERN_BIG_CASE(16)
     default: return cudaErrorInvalidValue;
   }
 #undef BERN_BIG_CASE
