@@ -32,7 +32,7 @@
 // bandwidth.  Against 1-D rows with a launch per bound: layer 3 of [6,100x3,2],
 // 2048 boxes, 7.31 -> 2.66 ms; layer 4 of [3,64x4,1], 5120 boxes, 1.28 -> 1.16
 // ms.  Against a block per item over pair lists (each thread gathering its own
-// list): layer 4 of [6,64x4,1], degree 8, 48 boxes, 51.4 -> 7.1 ms.
+// list): layer 4 of [6,64x4,1], degree 8, 48 boxes, 51.4 -> 6.4 ms.
 #include <algorithm>
 
 #include "compose_common.cuh"
@@ -547,9 +547,15 @@ k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstrid
 // the constant terms from the parts' remainders in order.
 //   scratch of a group: padded pairs x 32 lanes of s, then per warp of the parts a
 //   remainder (32 pairs), the constant and sum|s| (32 pairs each).
+// The units kernel waits for its loads of s (14 resident warps, a third of them from
+// the L1): one block of 16 warps on neighbouring units per multiprocessor instead
+// of two of 8 shares more of the L1, and 16 tasks per group of its size end closer
+// together (100 groups, n = 6, D = 8: 7.1 ms, 6.9 with 8 tasks, 6.4 with 16 and
+// 6.3 with 32, whose remainders cost that again).
 constexpr int kSquareWarpTerms = 32;         // padded terms of a warp per group
 constexpr int kSquareChunks = 16;
-constexpr int kSquareParts = kSquareChunks * kSquareWarps;
+constexpr int kUnitWarps = 16;                // one block per multiprocessor
+constexpr int kSquareParts = kSquareChunks * kUnitWarps;
 
 __global__ void __launch_bounds__(256)
 k_square_scale(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int first, int groups,
@@ -577,12 +583,12 @@ k_square_scale(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int 
   }
 }
 
-__global__ void __launch_bounds__(32 * kSquareWarps, kSquareBlocks)
+__global__ void __launch_bounds__(32 * kUnitWarps, 1)
 k_square_units(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int first, int groups,
                int64_t gstride, int* status) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int task = blockIdx.x; task < groups * kSquareChunks; task += gridDim.x) {
-    const int g = task / kSquareChunks, part = (task - g * kSquareChunks) * kSquareWarps + warp;
+    const int g = task / kSquareChunks, part = (task - g * kSquareChunks) * kUnitWarps + warp;
     int group = first + g;
     const int D = find_group(S, dlo, dhi, group);
     if (D < 0) break;
@@ -685,8 +691,8 @@ cudaError_t launch_compose_square(const Launch& L, const Tables& T, const Compos
       k_square_scale<<<(unsigned)std::min<int64_t>(groups, device_sms(L) * 8), 256, 0, L.stream>>>(
           T, A, S, dsm + 1, dmx, (int)first, groups, gstride, L.status);
       k_square_units<<<(unsigned)std::min<int64_t>((int64_t)groups * kSquareChunks,
-                                                   device_sms(L) * kSquareBlocks * 8),
-                       32 * kSquareWarps, 0, L.stream>>>(T, A, S, dsm + 1, dmx, (int)first,
+                                                   device_sms(L) * 8),
+                       32 * kUnitWarps, 0, L.stream>>>(T, A, S, dsm + 1, dmx, (int)first,
                                                          groups, gstride, L.status);
       k_square_constant<<<(unsigned)std::min<int64_t>(groups, device_sms(L) * 16), 32, 0,
                           L.stream>>>(T, A, S, dsm + 1, dmx, (int)first, groups, gstride,
