@@ -351,8 +351,8 @@ def source_sha(path):
         return hashlib.sha256(f.read()).hexdigest()[:16]
 
 
-KERNEL_SOURCES = {"affine": "k_affine.cu", "enclose": "k_enclose.cu", "compose": "k_compose.cu",
-                  "relu": "k_enclose.cu", "init": "k_io.cu", "layer": "k_layer.cu"}
+KERNEL_SOURCES = {"affine": "k_affine.cu", "enclose": "k_enclose.cu",
+                  "compose": "k_compose_square.cu", "relu": "k_enclose.cu", "init": "k_io.cu", "layer": "k_layer.cu"}
 
 
 def ncu_traffic(kernel_key):

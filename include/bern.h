@@ -178,8 +178,8 @@ int bern_set_pointer_mode(bern_ctx* ctx, int mode);
  * (network widths, plan, batch size) times every variant of the tunable
  * kernels (the wide-layer affine kernel: persistent register-blocked with
  * 4-, 2- or 1-row thread tiles, or 64x32 block tiles; the Bernstein
- * enclosure: 8, 4 or 2 items per block) on its first
- * chunk and keeps the fastest per shape.  All variants compute identical
+ * enclosure where it runs on grids: 8, 4 or 2 items per block) on its first
+ * chunk, twice each, and keeps the fastest per shape.  All variants compute identical
  * results.  enable = 0 uses the built-in defaults. */
 int bern_set_autotune(bern_ctx* ctx, int enable);
 
@@ -192,7 +192,9 @@ int bern_set_autotune(bern_ctx* ctx, int enable);
  * 2 for longer polynomials) or "enclose"
  * (variants 0-2: 8, 4 or 2 items per block with a warp per polynomial; 3, 4:
  * a block of 128 or 320 threads per polynomial for shared-memory grids of
- * 256 cells or more at orders 3-16, else as 2).  variant = -1 clears the
+ * 256 cells or more at orders 3-16, else as 2; without effect on the
+ * enclosures that use no grid: order 1, two and three variables up to order
+ * 8, four and more up to order 10).  variant = -1 clears the
  * force.
  * Drops captured graphs.  Returns BERN_E_INVALID for an unknown kind or a
  * variant out of range. */
@@ -272,7 +274,7 @@ int bern_enclose_scales(int n, int l, float* out, int64_t cap);
 /* The composition's row tables for input degree D (Sec. 5.1 Step 3 at ReLU
  * order 2: s^2 is formed as sums of 1-D convolutions of the rows of s, a row
  * being the monomials that share the exponents of t_1..t_{n-1}, laid out with
- * the last exponent running), as the row-convolution kernel reads them.
+ * the last exponent running), as the fused layer kernel (bern_layer) reads them.
  *   sizes[5] receives m_in = M(n, D), the output rows, the row where the
  *   second half of the work starts, the pairs and the output ranks.
  *   out (NULL: sizes only) receives, concatenated, int32:
@@ -287,7 +289,8 @@ int bern_enclose_scales(int n, int l, float* out, int64_t cap);
  *     out_ranks[...]   graded rank (degree <= 2D) of each output row element.
  * Host only; no GPU needed.  Returns BERN_OK; BERN_E_INVALID (sizes NULL, n
  * outside [1, 8], D outside [0, 8], or cap too small); BERN_E_UNSUPPORTED
- * when the input has more than 750 terms (those use the pair-list kernel). */
+ * when the input has more than 750 terms (the fused kernel does not take
+ * those). */
 int bern_compose_rows(int n, int D, int32_t* out, int64_t cap, int64_t* sizes);
 
 /* The output-stationary pair lists of the other composition kernels (Sec.
