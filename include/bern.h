@@ -206,6 +206,14 @@ int bern_force_variant(bern_ctx* ctx, const char* kind, int variant);
  * the same values in the same order (a setting for tests and tuning). */
 int bern_set_horner_smem_limit(bern_ctx* ctx, int64_t bytes);
 
+/* Largest device scratch (bytes, at most and by default 512 MB) the order-2
+ * compositions may keep their inputs past shared memory in.  Squares whose
+ * groups of 32 neurons exceed it run in several passes, with the same values in
+ * the same order; where not one group fits, or the device cannot give the
+ * memory, they take the pair-list kernel, whose sums run in another order (a
+ * setting for tests and tuning). */
+int bern_set_square_scratch_limit(bern_ctx* ctx, int64_t bytes);
+
 /* Use CUDA-graph replay for bern_propagate (default 1).  With graphs on, the
  * launch sequence of one (network shape, batch size, plan, buffers) tuple is
  * captured once and replayed. */

@@ -54,7 +54,8 @@ EXPORTS = [
     "bern_enclose", "bern_relu_coeffs", "bern_compose", "bern_propagate_noalloc",
     "bern_mlp_num_params", "bern_degree_features", "bern_mlp_forward", "bern_mlp_backward",
     "bern_mlp_adam", "bern_propagate_traced", "bern_split_features",
-    "bern_set_horner_smem_limit", "bern_set_autotune", "bern_force_variant",
+    "bern_set_horner_smem_limit", "bern_set_square_scratch_limit", "bern_set_autotune",
+    "bern_force_variant",
     "bern_poly_to_x", "bern_linearize", "bern_fma_throughput", "bern_layer", "bern_set_fused",
     "bern_bernstein_square",
     "bern_bernstein_elevate",
@@ -128,6 +129,7 @@ def load(build_if_missing: bool = True):
         "bern_set_pointer_mode": (I, [V, I]),
         "bern_set_graphs": (I, [V, I]),
         "bern_set_horner_smem_limit": (I, [V, I64]),
+        "bern_set_square_scratch_limit": (I, [V, I64]),
         "bern_set_autotune": (I, [V, I]),
         "bern_force_variant": (I, [V, ctypes.c_char_p, I]),
         "bern_poly_to_x": (I, [V, I, I64, I, V, V, V, I64, V]),
@@ -345,6 +347,10 @@ class Context:
     def set_horner_smem_limit(self, nbytes: int):
         _check(self.lib.bern_set_horner_smem_limit(self.h, int(nbytes)),
                "bern_set_horner_smem_limit")
+
+    def set_square_scratch_limit(self, nbytes: int):
+        _check(self.lib.bern_set_square_scratch_limit(self.h, int(nbytes)),
+               "bern_set_square_scratch_limit")
 
     def set_pointer_mode(self, mode: int):
         _check(self.lib.bern_set_pointer_mode(self.h, mode), "bern_set_pointer_mode")

@@ -82,6 +82,8 @@ struct bern_ctx {
   DevBuf ctr;                       // box counters of the fused layer kernels
   DevBuf ebuf;                      // grids of enclosures above shared memory
   DevBuf sqbuf;                     // scaled inputs of the long squares
+  size_t sq_asked = 0;              // the most that was asked for it
+  int64_t square_scratch_limit = kSquareScratchBytes;
   DevBuf btnt;                      // term counts of the Bernstein-basis layer sum
   int fused = 0;                    // fused layer kernels where a plan allows them
   std::vector<GraphEntry> graphs;
@@ -372,9 +374,28 @@ int ensure_prod_tables(bern_ctx* c, int n, int Dmax, int dmax, int cap) {
   return finish(BERN_OK);
 }
 
+// The scratch of the long squares: `bytes`, or what the device has of it down to
+// one group (`group` bytes, the squares then take passes of what fits).  Less
+// leaves the context's buffer empty and the items to the pair lists; it is asked
+// for again by the next call, a part of it only when a call wants more.
+cudaError_t ensure_square_scratch(bern_ctx* c, size_t bytes, size_t group) {
+  DevBuf& b = c->sqbuf;
+  if (b.bytes >= bytes || (b.bytes >= group && c->sq_asked >= bytes)) return cudaSuccess;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    return cudaSuccess;             // no allocation in the caller's capture
+  c->sq_asked = bytes;
+  for (size_t want = bytes;; want = std::max(group, want / 2)) {
+    const cudaError_t e = b.reserve(want);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();             // not this call's error
+    if (want == group) return cudaSuccess;
+  }
+}
+
 // Composition work queues for up to `items` items.
 int ensure_queues(bern_ctx* c, int64_t items, ComposeScratch* out, size_t horner_floats = 0,
-                  size_t square_bytes = 0) {
+                  size_t square_bytes = 0, size_t square_group = 0) {
   // *out is part of the graph key byte for byte: zero its padding too
   std::memset(out, 0, sizeof *out);
   const size_t bytes = 256 + (size_t)kQueueLists * items * sizeof(int);
@@ -395,9 +416,13 @@ int ensure_queues(bern_ctx* c, int64_t items, ComposeScratch* out, size_t horner
   out->tws = nullptr;
   out->tws_bytes = 0;
   if (square_bytes) {
-    if ((e = c->sqbuf.reserve(square_bytes)) != cudaSuccess) return map_cuda(e);
-    out->tws = c->sqbuf.p;
-    out->tws_bytes = (int64_t)c->sqbuf.bytes;
+    if ((e = ensure_square_scratch(c, square_bytes, square_group)) != cudaSuccess)
+      return map_cuda(e);
+    const int64_t got = std::min((int64_t)c->sqbuf.bytes, c->square_scratch_limit);
+    if (got >= (int64_t)square_group) {
+      out->tws = c->sqbuf.p;
+      out->tws_bytes = got;
+    }
   }
   return BERN_OK;
 }
@@ -913,6 +938,12 @@ int bern_set_horner_smem_limit(bern_ctx* c, int64_t bytes) {
   return BERN_OK;
 }
 
+int bern_set_square_scratch_limit(bern_ctx* c, int64_t bytes) {
+  if (!c || bytes < 0) return BERN_E_INVALID;
+  c->square_scratch_limit = std::min(bytes, kSquareScratchBytes);
+  return BERN_OK;
+}
+
 int bern_set_graphs(bern_ctx* c, int enable) {
   if (!c) return BERN_E_INVALID;
   c->use_graphs = enable ? 1 : 0;
@@ -1196,9 +1227,11 @@ int bern_compose(bern_ctx* c, int n, int64_t n_boxes, int h, int degree_cap, flo
   }
   ComposeScratch CS;
   const size_t square_bytes =
-      prune_tau == 0.0f && global_d >= 2 ? square_scratch_bytes(n, Dmax, n_boxes * h) : 0;
+      prune_tau == 0.0f && global_d >= 2
+          ? square_scratch_bytes(n, Dmax, n_boxes * h, c->square_scratch_limit)
+          : 0;
   if ((rc = ensure_queues(c, std::max<int64_t>(1, n_boxes * h), &CS, horner_floats,
-                          square_bytes)))
+                          square_bytes, square_group_bytes(n, Dmax))))
     return rc;
   return map_cuda(launch_compose(c->launch(), *T, CS, n_boxes, h, degree_cap, prune_tau, kind,
                                  coef, eps, degrees, global_d, lo, hi, pre_up, pre_lo, pre_ld,
@@ -1315,11 +1348,15 @@ int bern_propagate_traced(bern_ctx* c, const bern_net* net, const float* boxes,
   int hmax = 1;
   for (const auto& l : P.L) hmax = std::max(hmax, l.h_out);
   ComposeScratch CS;
-  size_t square_bytes = 0;
+  size_t square_bytes = 0, square_group = 0;
   for (const auto& l : P.L)
-    if (l.hidden && P.tau == 0.0f && l.d >= 2 && !l.fused)
-      square_bytes = std::max(square_bytes, square_scratch_bytes(P.n, l.D_pre, chunk * l.h_out));
-  if ((rc = ensure_queues(c, chunk * hmax, &CS, horner_floats, square_bytes))) return rc;
+    if (l.hidden && P.tau == 0.0f && l.d >= 2 && !l.fused) {
+      square_bytes = std::max(square_bytes, square_scratch_bytes(P.n, l.D_pre, chunk * l.h_out,
+                                                                 c->square_scratch_limit));
+      square_group = std::max(square_group, square_group_bytes(P.n, l.D_pre));
+    }
+  if ((rc = ensure_queues(c, chunk * hmax, &CS, horner_floats, square_bytes, square_group)))
+    return rc;
 
   // autotune once per plan shape: probe every variant of every tunable kind
   // on the first chunk (plain launches, timed per launch), keep the fastest

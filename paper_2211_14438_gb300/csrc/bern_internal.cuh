@@ -108,8 +108,10 @@ int square_padded_terms(int n, int D);
 // Largest degree whose inputs fit the shared-memory / the scratch kernels.
 int square_smem_degree(int n);
 int square_max_degree(int n);
-// Scratch of the long inputs for items of degree <= Dmax (0: none needed).
-size_t square_scratch_bytes(int n, int Dmax, int64_t n_items);
+// Scratch of the long inputs for items of degree <= Dmax, at most `limit` bytes
+// of it (0: none needed, or not a group within the limit), and that of one group.
+size_t square_scratch_bytes(int n, int Dmax, int64_t n_items, int64_t limit);
+size_t square_group_bytes(int n, int Dmax);
 
 // ------------------------------------------------------------ device views
 struct RowTable {

@@ -643,13 +643,17 @@ int square_max_degree(int n) {
   return D;
 }
 
-size_t square_scratch_bytes(int n, int Dmax, int64_t n_items) {
+size_t square_group_bytes(int n, int Dmax) {
   const int D = std::min(Dmax, square_max_degree(n));
   if (D <= square_smem_degree(n)) return 0;
-  const int64_t per = group_pairs(square_padded_terms(n, D)) * (int64_t)sizeof(p2);
+  return (size_t)group_pairs(square_padded_terms(n, D)) * sizeof(p2);
+}
+size_t square_scratch_bytes(int n, int Dmax, int64_t n_items, int64_t limit) {
+  const int64_t per = (int64_t)square_group_bytes(n, Dmax);
+  if (per == 0) return 0;
   // a group may be short, one per degree
   const int64_t groups = (n_items + 31) / 32 + kMaxRowDegree;
-  return (size_t)(per * std::max<int64_t>(1, std::min<int64_t>(groups, kSquareScratchBytes / per)));
+  return (size_t)(per * std::min<int64_t>(groups, limit / per));
 }
 
 cudaError_t launch_compose_square(const Launch& L, const Tables& T, const ComposeScratch& S,

@@ -1,0 +1,45 @@
+"""What a call does when device memory is short, on a runtime without a device."""
+from host_runtime import run
+
+COMPOSE = """
+def compose(h, n, D, B, hh, d=2, degrees=False):
+    M = bern.num_monomials(n, D)
+    keep = bern.num_monomials(n, min(2 * D, 16))
+    items = B * hh
+    launched()
+    rc = lib.bern_compose(h, n, B, hh, 16, 0.0, empty(items), empty(items * 4 * bern.COEF_STRIDE),
+                          empty(items * 4), empty(items) if degrees else None, d,
+                          empty(items * 4), empty(items * 4), empty(8), empty(8), M,
+                          empty(items * 4), empty(8), empty(8), keep, empty(items * 4))
+    return rc, launched()
+def count(names, what):
+    return sum(what in x for x in names)
+"""
+
+
+def test_squares_without_their_scratch_take_the_pair_lists(tmp_path):
+    """Inputs past shared memory (five variables, degree 8: 1287 terms): with no
+    scratch to be had the call goes on with the pair lists, with room for some of
+    the groups it takes several passes, and each state serves the calls after it."""
+    run(tmp_path, COMPOSE + """
+h = context()
+rc, k = compose(h, 5, 8, 4, 64)                       # eight groups and eight spare
+assert rc == 0 and count(k, "k_square_units") == 1 and count(k, "k_compose_pairs") == 0, (rc, k)
+lib.bern_destroy(h)
+
+h = context()
+rc, k = compose(h, 5, 8, 4, 64, d=1)                  # tables and queues
+assert rc == 0 and count(k, "k_square") == 0, (rc, k)
+rt.host_set_alloc_limit(300 << 10)                    # less than a group of 400 KB
+for _ in range(2):
+    rc, k = compose(h, 5, 8, 4, 64)
+    assert rc == 0 and count(k, "k_square_units") == 0 and count(k, "k_compose_pairs") == 1, (rc, k)
+rt.host_set_alloc_limit(2 << 20)                      # a few groups
+for _ in range(2):
+    rc, k = compose(h, 5, 8, 4, 64)
+    assert rc == 0 and count(k, "k_square_units") > 1 and count(k, "k_compose_pairs") == 0, (rc, k)
+rt.host_set_alloc_limit(1 << 40)
+rc, k = compose(h, 5, 8, 64, 64)                      # more items: asked for again
+assert rc == 0 and count(k, "k_square_units") == 1, (rc, k)
+lib.bern_destroy(h)
+""")
