@@ -1226,8 +1226,9 @@ int bern_compose(bern_ctx* c, int n, int64_t n_boxes, int h, int degree_cap, flo
                                          kHornerGlobalPerSM * std::max(1, c->sms));
   }
   ComposeScratch CS;
+  // order-2 items exist as launch_compose has it
   const size_t square_bytes =
-      prune_tau == 0.0f && global_d >= 2
+      prune_tau == 0.0f && (global_d == 2 || (degrees && global_d > 2))
           ? square_scratch_bytes(n, Dmax, n_boxes * h, c->square_scratch_limit)
           : 0;
   if ((rc = ensure_queues(c, std::max<int64_t>(1, n_boxes * h), &CS, horner_floats,
@@ -1350,7 +1351,8 @@ int bern_propagate_traced(bern_ctx* c, const bern_net* net, const float* boxes,
   ComposeScratch CS;
   size_t square_bytes = 0, square_group = 0;
   for (const auto& l : P.L)
-    if (l.hidden && P.tau == 0.0f && l.d >= 2 && !l.fused) {
+    if (l.hidden && P.tau == 0.0f && !l.fused &&
+        (l.d == 2 || (l.d > 2 && (P.per_neuron || P.learned)))) {
       square_bytes = std::max(square_bytes, square_scratch_bytes(P.n, l.D_pre, chunk * l.h_out,
                                                                  c->square_scratch_limit));
       square_group = std::max(square_group, square_group_bytes(P.n, l.D_pre));

@@ -16,6 +16,7 @@ long copies_left = -1;               // -1: all copies succeed
 int last_error = 0;
 std::map<const void*, std::string> names;
 std::string launched;                // one name per line
+std::string allocated;               // sizes in bytes, one per line
 constexpr int kNoMemory = 2, kUnknown = 999;
 int fail(int e) { return last_error = e; }
 }  // namespace
@@ -24,11 +25,13 @@ extern "C" {
 void host_set_alloc_limit(size_t bytes) { alloc_limit = bytes; }
 void host_fail_copies_after(long n) { copies_left = n; }
 const char* host_launched() { return launched.c_str(); }
-void host_clear() { launched.clear(); }
+const char* host_allocated() { return allocated.c_str(); }
+void host_clear() { launched.clear(), allocated.clear(); }
 
 int cudaMalloc(void** p, size_t n) {
   *p = nullptr;
   if (n > alloc_limit || !(*p = std::calloc(n ? n : 1, 1))) return fail(kNoMemory);
+  allocated += std::to_string(n) + "\n";
   return 0;
 }
 int cudaFree(void* p) { std::free(p); return 0; }

@@ -1,7 +1,8 @@
 """Runs a piece of Python against the library on host_cudart.cpp (no device, no
 kernel runs) in a process of its own.  The code finds `rt` (the runtime's
 controls), `lib` (the library, with its argument types), `bern`, `np`, `ctypes`,
-`launched()` (the kernels noted since the last call) and `empty(n)` (an address
+`launched()` (the kernels noted since the last call), `allocated()` (the sizes allocated since
+then) and `empty(n)` (an address
 of n zeroed bytes)."""
 import os
 import subprocess
@@ -16,7 +17,7 @@ sys.path.insert(0, %(root)r)
 rt = ctypes.CDLL(%(so)r, mode=ctypes.RTLD_GLOBAL)
 rt.host_set_alloc_limit.argtypes = [ctypes.c_size_t]
 rt.host_fail_copies_after.argtypes = [ctypes.c_long]
-rt.host_launched.restype = ctypes.c_char_p
+rt.host_launched.restype = rt.host_allocated.restype = ctypes.c_char_p
 from paper_2211_14438_gb300 import bern
 lib = bern.load()
 _keep = []
@@ -24,6 +25,8 @@ def launched():
     names = rt.host_launched().decode().split()
     rt.host_clear()
     return names
+def allocated():
+    return [int(x) for x in rt.host_allocated().decode().split()]
 def empty(n):
     _keep.append(np.zeros(max(1, n), np.uint8))
     return ctypes.c_void_p(_keep[-1].ctypes.data)

@@ -11,7 +11,9 @@ def compose(h, n, D, B, hh, d=2, degrees=False):
                           empty(items * 4), empty(items) if degrees else None, d,
                           empty(items * 4), empty(items * 4), empty(8), empty(8), M,
                           empty(items * 4), empty(8), empty(8), keep, empty(items * 4))
+    sizes.append(allocated())
     return rc, launched()
+sizes = []                                            # of each call
 def count(names, what):
     return sum(what in x for x in names)
 """
@@ -42,4 +44,19 @@ rt.host_set_alloc_limit(1 << 40)
 rc, k = compose(h, 5, 8, 64, 64)                      # more items: asked for again
 assert rc == 0 and count(k, "k_square_units") == 1, (rc, k)
 lib.bern_destroy(h)
+""")
+
+
+def test_no_scratch_where_nothing_is_squared(tmp_path):
+    """Order 3 for every neuron has no squares; per-neuron orders up to 3 may have."""
+    run(tmp_path, COMPOSE + """
+def sizes_of(d, degrees):
+    h = context()
+    assert compose(h, 5, 7, 4, 64, d=1)[0] == 0       # 792 terms: tables and queues
+    assert compose(h, 5, 7, 4, 64, d=d, degrees=degrees)[0] == 0
+    lib.bern_destroy(h)
+    return sizes[-1]
+scratch, = sizes_of(2, False)
+assert scratch in sizes_of(3, True)
+assert scratch not in sizes_of(3, False)
 """)
