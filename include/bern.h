@@ -179,7 +179,8 @@ int bern_set_pointer_mode(bern_ctx* ctx, int mode);
  * kernels (the wide-layer affine kernel: persistent register-blocked with
  * 4-, 2- or 1-row thread tiles, or 64x32 block tiles; the Bernstein
  * enclosure where it runs on grids: 8, 4 or 2 items per block) on its first
- * chunk, twice each, and keeps the fastest per shape.  All variants compute identical
+ * chunk, twice each, and keeps the fastest per shape: at most ten passes over the
+ * network, one where no step has variants.  All variants compute identical
  * results.  enable = 0 uses the built-in defaults. */
 int bern_set_autotune(bern_ctx* ctx, int enable);
 

@@ -919,7 +919,7 @@ int bern_set_autotune(bern_ctx* c, int enable) {
 int bern_force_variant(bern_ctx* c, const char* kind, int variant) {
   if (!c || !kind) return BERN_E_INVALID;
   const std::string k(kind);
-  const int nvar = k == "affine" ? 5 : (k == "enclose" ? 5 : 0);
+  const int nvar = k == "affine" || k == "enclose" ? kTuneVariants : 0;
   if (nvar == 0 || variant < -1 || variant >= nvar) return BERN_E_INVALID;
   cudaStreamSynchronize(c->stream);
   for (auto& g : c->graphs)
@@ -1360,7 +1360,7 @@ int bern_propagate_traced(bern_ctx* c, const bern_net* net, const float* boxes,
   if ((rc = ensure_queues(c, chunk * hmax, &CS, horner_floats, square_bytes, square_group)))
     return rc;
 
-  // autotune once per plan shape: probe every variant of every tunable kind
+  // autotune once per plan shape: probe every variant of the tunable launches
   // on the first chunk (plain launches, timed per launch), keep the fastest
   if (c->autotune) {
     std::string sig;
@@ -1383,35 +1383,34 @@ int bern_propagate_traced(bern_ctx* c, const bern_net* net, const float* boxes,
       const int64_t B = std::min(chunk, n_boxes);
       Chunk ch{(char*)c->ws.p, B};
       if ((rc = fill_degrees(c, P, ch, B))) return rc;
-      const char* kinds[] = {"affine", "enclose"};
-      const int nvar[] = {5, 5};
-      // two passes of each variant, the faster one counts: a kernel's first launch
-      // also loads it
-      for (int k = 0; k < 2; ++k) {
-        std::map<std::string, std::vector<float>> ms;
-        for (int v = 0; v < nvar[k]; ++v)
-          for (int pass = 0; pass < 2; ++pass) {
-            c->tuner.probe_kind = kinds[k];
-            c->tuner.probe_variant = v;
-            c->tuner.probe_ms.clear();
-            rc = run_chunk(c, c->stream, P, *T, CS, &dnet, d_boxes, B, ch, dres.lo, dres.hi, dres,
-                           nullptr);
-            c->tuner.probe_kind.clear();
-            if (rc) return rc;
-            for (const auto& kv : c->tuner.probe_ms) {
-              auto& w = ms[kv.first];
-              w.resize(nvar[k], -1.0f);
-              if ((int)kv.second.size() > v && kv.second[v] >= 0.0f)
-                w[v] = w[v] < 0.0f ? kv.second[v] : std::min(w[v], kv.second[v]);
-            }
+      // a pass of a variant times every launch that has it, of both kinds; the
+      // first finds which variants there are to choose at all.  Two passes of each,
+      // the faster one counts: a kernel's first launch also loads it
+      std::map<std::string, std::vector<float>> ms;
+      c->tuner.probe_mask = 1u;
+      for (int v = 0; v < kTuneVariants; ++v)
+        for (int pass = 0; pass < 2; ++pass) {
+          if (!((c->tuner.probe_mask >> v) & 1)) continue;
+          if (v == 0 && pass == 0) c->tuner.probe_mask = 0;
+          c->tuner.probe_variant = v;
+          c->tuner.probe_ms.clear();
+          rc = run_chunk(c, c->stream, P, *T, CS, &dnet, d_boxes, B, ch, dres.lo, dres.hi, dres,
+                         nullptr);
+          c->tuner.probe_variant = -1;
+          if (rc) return rc;
+          for (const auto& kv : c->tuner.probe_ms) {
+            auto& w = ms[kv.first];
+            w.resize(kTuneVariants, -1.0f);
+            if ((int)kv.second.size() > v && kv.second[v] >= 0.0f)
+              w[v] = w[v] < 0.0f ? kv.second[v] : std::min(w[v], kv.second[v]);
           }
-        c->tuner.probe_ms.clear();
-        for (const auto& kv : ms) {
-          int best = -1;
-          for (int v = 0; v < (int)kv.second.size(); ++v)
-            if (kv.second[v] >= 0.0f && (best < 0 || kv.second[v] < kv.second[best])) best = v;
-          if (best >= 0) c->tuner.best[kv.first] = best;
         }
+      c->tuner.probe_ms.clear();
+      for (const auto& kv : ms) {
+        int best = -1;
+        for (int v = 0; v < (int)kv.second.size(); ++v)
+          if (kv.second[v] >= 0.0f && (best < 0 || kv.second[v] < kv.second[best])) best = v;
+        if (best >= 0) c->tuner.best[kv.first] = best;
       }
       if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return map_cuda(e);
       c->tuned.insert(sig);

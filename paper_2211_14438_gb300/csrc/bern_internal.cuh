@@ -205,13 +205,13 @@ void build_lex_tables(int n, int l, std::vector<uint32_t>& pos,
 // ------------------------------------------------------------ launchers
 // Autotuning.  Launchers that have several valid variants for a shape ask
 // the tuner which one to run (by a key naming the kernel kind and shape).  In
-// a probe pass the tuner forces one variant of one kind and times every
-// launch of that kind with CUDA events; afterwards each key keeps its fastest
-// variant.  Every variant computes the same values in the same order.
+// a probe pass every launch that has the probed variant runs and times it with
+// CUDA events; afterwards each key keeps its fastest variant.  Every variant computes the same values in the same order.
+constexpr int kTuneVariants = 5;   // of each kind
 struct Tuner {
   std::map<std::string, int> best;                        // key -> variant
-  std::string probe_kind;                                 // empty: no probe pass
-  int probe_variant = -1;
+  int probe_variant = -1;                                 // -1: no probe pass
+  unsigned probe_mask = 0;                                // variants there were to choose
   std::map<std::string, std::vector<float>> probe_ms;     // key -> ms per variant
   std::map<std::string, int> forced;                      // kind -> variant (tests)
 };
@@ -231,16 +231,19 @@ struct Launch {
 // device's attribute); grids of persistent kernels are multiples of it.
 int device_sms(const Launch& L);
 
-// Variant of `kind` to run for `key` (dflt when untuned).
-int tune_variant(const Launch& L, const char* kind, const std::string& key, int dflt);
-// Probe timing around one launch of `kind`: tune_begin records the start event
-// when this kind is being probed; tune_end records, waits and adds the time.
+// Variant of `kind` to run for `key` (dflt when untuned), of those in the bit
+// mask `valid` that run a kernel of their own here; fills `t` for a probe pass.  A
+// forced variant comes back as it is, valid or not.
 struct TuneTimer {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   bool on = false;
 };
-void tune_begin(const Launch& L, const char* kind, TuneTimer& t);
-void tune_end(const Launch& L, const char* kind, const std::string& key, TuneTimer& t);
+int tune_variant(const Launch& L, const char* kind, const std::string& key, int dflt,
+                 unsigned valid, TuneTimer& t);
+// Probe timing around one launch: tune_begin records the start event; tune_end
+// records, waits and adds the time.
+void tune_begin(const Launch& L, TuneTimer& t);
+void tune_end(const Launch& L, const std::string& key, TuneTimer& t);
 
 // Layer-block layout: coefficient r of neuron m of box b at ((b*ld + r)*h + m);
 // term counts at b*h + m.

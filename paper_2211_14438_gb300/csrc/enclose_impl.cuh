@@ -291,11 +291,12 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
   int items = (int)std::min<int64_t>(8, (192 * 1024) / (2 * (int64_t)G * 4));
   const std::string key = "enclose/" + std::to_string(LB) + "/" + std::to_string(T.n) + "/" +
                           std::to_string(n_items);
-  const int v = tune_variant(L, "enclose", key, 0);
+  TuneTimer tt;
+  const int v = tune_variant(L, "enclose", key, 0,
+                             1u | (items > 4 ? 2u : 0u) | (items > 2 ? 4u : 0u), tt);
   items = std::min(items, 8 >> std::min(v, 2));
   if (items < 1) items = 1;
-  TuneTimer tt;
-  tune_begin(L, "enclose", tt);
+  tune_begin(L, tt);
   const size_t smem = (size_t)2 * items * G * sizeof(float);
   // the in-simplex prefix loop for four or more variables (their grids of
   // l >= 12, 13^4 cells and more, exceed kEncloseGridMax and run elsewhere);
@@ -316,7 +317,7 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
                                                ld, nterms, lo, hi, ro, L.status);
   ++*L.launches;
   const cudaError_t e = cudaGetLastError();
-  tune_end(L, "enclose", key, tt);
+  tune_end(L, key, tt);
   return e;
 }
 

@@ -1054,12 +1054,15 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
     const int64_t rows_in = std::min(in_ld, out_ld);
     const bool live = h_in >= kWideLiveInputs && rows_in > kWideLiveRows;
     const int rows_dflt = live && rows_in <= 64 ? 3 : 2;
-    int v = tune_variant(L, "affine", key, short_ok ? 4 : (wide_ok ? rows_dflt : 1));
+    TuneTimer tt;
+    int v = tune_variant(L, "affine", key, short_ok ? 4 : (wide_ok ? rows_dflt : 1),
+                         2u | (wide_ok ? 4u | 8u : 0u) | (wide4_ok ? 1u : 0u) |
+                             (short_ok ? 16u : 0u),
+                         tt);
     if (v == 4 && !short_ok) v = wide_ok ? 2 : 1;
     if (v != 1 && v != 4 && !wide_ok) v = short_ok ? 4 : 1;
     if (v == 0 && !wide4_ok) v = 2;
-    TuneTimer tt;
-    tune_begin(L, "affine", tt);
+    tune_begin(L, tt);
     cudaError_t e;
     if (v == 0 || v == 2 || v == 3) {
       const int rows = v == 0 ? 64 : (v == 2 ? 32 : 16);
@@ -1095,7 +1098,7 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
       e = launch_cfg<64, 32, 4, 2, 32>(L, n_boxes, h_out, h_in, W, b, in_up, in_lo, in_ld,
                                        in_nterms, out_up, out_lo, out_ld, out_nterms);
     }
-    tune_end(L, "affine", key, tt);
+    tune_end(L, key, tt);
     return e;
   }
   // Short polynomials into 17..31 neurons: a warp per box too, once every

@@ -138,14 +138,14 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
   if (blk_ok) {
     key = "enclose/" + std::to_string(lb) + "/" + std::to_string(T.n) + "/" +
           std::to_string(n_items);
-    const int v = tune_variant(L, "enclose", key, G >= kEncloseBlkGrid ? 3 : 0);
+    const int v = tune_variant(L, "enclose", key, G >= kEncloseBlkGrid ? 3 : 0, 31u, tt);
     blk = v >= 3;
     blk_wide = v == 4;
   }
   if (slab || G > kEncloseGridMax || blk) {
     // slabs, global-memory grids, or a block per polynomial: lo/hi, then the
     // ReLU step on the same items
-    if (blk) tune_begin(L, "enclose", tt);
+    if (blk) tune_begin(L, tt);
     cudaError_t e =
         slab ? launch_enclose_slab(L, T, lb, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi,
                                    ro.list, ro.count)
@@ -161,7 +161,7 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
       ++*L.launches;
       e = cudaGetLastError();
     }
-    if (blk) tune_end(L, "enclose", key, tt);
+    if (blk) tune_end(L, key, tt);
     return e;
   }
   if (G <= kSmallGrid && lb <= 7) {

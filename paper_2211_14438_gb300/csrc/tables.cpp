@@ -639,25 +639,30 @@ int device_sms(const Launch& L) {
   return sms;
 }
 
-int tune_variant(const Launch& L, const char* kind, const std::string& key, int dflt) {
+int tune_variant(const Launch& L, const char* kind, const std::string& key, int dflt,
+                 unsigned valid, TuneTimer& t) {
+  t.on = false;
   if (!L.tuner) return dflt;
-  if (!L.tuner->probe_kind.empty())
-    return L.tuner->probe_kind == kind ? L.tuner->probe_variant : dflt;
+  if (L.tuner->probe_variant >= 0) {
+    if ((valid & (valid - 1)) == 0) return dflt;   // nothing to choose
+    L.tuner->probe_mask |= valid;
+    t.on = (valid >> L.tuner->probe_variant) & 1;
+    return t.on ? L.tuner->probe_variant : dflt;
+  }
   auto f = L.tuner->forced.find(kind);
   if (f != L.tuner->forced.end()) return f->second;
   auto it = L.tuner->best.find(key);
   return it == L.tuner->best.end() ? dflt : it->second;
 }
 
-void tune_begin(const Launch& L, const char* kind, TuneTimer& t) {
-  t.on = L.tuner && L.tuner->probe_kind == kind;
+void tune_begin(const Launch& L, TuneTimer& t) {
   if (!t.on) return;
   cudaEventCreate(&t.e0);
   cudaEventCreate(&t.e1);
   cudaEventRecord(t.e0, L.stream);
 }
 
-void tune_end(const Launch& L, const char* kind, const std::string& key, TuneTimer& t) {
+void tune_end(const Launch& L, const std::string& key, TuneTimer& t) {
   if (!t.on) return;
   cudaEventRecord(t.e1, L.stream);
   cudaEventSynchronize(t.e1);
@@ -669,7 +674,6 @@ void tune_end(const Launch& L, const char* kind, const std::string& key, TuneTim
   const int var = L.tuner->probe_variant;
   if ((int)v.size() <= var) v.resize(var + 1, -1.0f);
   v[var] = (v[var] < 0.0f ? 0.0f : v[var]) + ms;
-  (void)kind;
 }
 
 }  // namespace bern
