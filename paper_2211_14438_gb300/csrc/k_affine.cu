@@ -1039,20 +1039,26 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
   const bool few_rows = std::min(in_ld, out_ld) <= 16;     // short polynomials: short tiles
   if (h_out >= 32) {
     // wide layers: autotuned among the persistent register-blocked kernel with
-    // 4-row (0), 2-row (2, the default) or 1-row (3, up to 64 rows) thread tiles, when its weights fit shared memory, block tiles (1), and
-    // for short polynomials a warp per box (4, their default)
+    // 4-row (0), 2-row (2) or 1-row (3) thread tiles, when its weights fit shared
+    // memory, block tiles (1), and for short polynomials a warp per box (4, their
+    // default)
     const std::string key = "affine/" + std::to_string(h_out) + "/" + std::to_string(h_in) +
                             "/" + std::to_string(in_ld) + "/" + std::to_string(n_boxes);
-    // 4-row thread tiles (64-row tiles) take the 2-row form where they do not fit
-    const bool wide_ok = wide_smem(h_out, h_in, 32) <= 200 * 1024;
+    const int64_t rows_in = std::min(in_ld, out_ld);
+    const bool live = h_in >= kWideLiveInputs && rows_in > kWideLiveRows;
+    // Weights that leave room for the smaller tiles only run one block on a
+    // multiprocessor, a box at a time: for batches (128 x 200, 165 rows, 608 boxes:
+    // 643 us against 980 us of block tiles, one box 218 against 22 us).
+    const size_t lists = 2 * (size_t)h_in * sizeof(int);
     const bool wide4_ok = wide_smem(h_out, h_in, 64) <= 200 * 1024;
+    const bool wide_ok = wide_smem(h_out, h_in, 64) - lists <= 200 * 1024 ||
+                         (n_boxes >= 4 * (int64_t)device_sms(L) &&
+                          wide_smem(h_out, h_in, 32) <= 200 * 1024);
     const size_t ssmem = short_smem(h_out, h_in);
     const bool short_ok = few_rows && ssmem <= 200 * 1024;
     // 1-row thread tiles from 33 to 64 rows (with lists): a 32-row tile is half empty at 35 rows,
     // and six blocks fit an SM instead of four (35 rows, 64 x 64, 5120 boxes: 132
     // against 150 us; 165 rows: 610 against 495 us)
-    const int64_t rows_in = std::min(in_ld, out_ld);
-    const bool live = h_in >= kWideLiveInputs && rows_in > kWideLiveRows;
     const int rows_dflt = live && rows_in <= 64 ? 3 : 2;
     TuneTimer tt;
     int v = tune_variant(L, "affine", key, short_ok ? 4 : (wide_ok ? rows_dflt : 1),
@@ -1061,7 +1067,7 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
                          tt);
     if (v == 4 && !short_ok) v = wide_ok ? 2 : 1;
     if (v != 1 && v != 4 && !wide_ok) v = short_ok ? 4 : 1;
-    if (v == 0 && !wide4_ok) v = 2;
+    if (v == 0 && !wide4_ok) v = 2;   // larger tiles that do not fit
     tune_begin(L, tt);
     cudaError_t e;
     if (v == 0 || v == 2 || v == 3) {
