@@ -163,14 +163,13 @@ k_affine(int h_out, int h_in, const float* __restrict__ W, const float* __restri
 // accumulates an 8 (neurons) x TR (rows) tile of the three sums per 64-neuron
 // slice: neurons 4 tm .. 4 tm + 3 and 32 + 4 tm .. 32 + 4 tm + 3, so the eight
 // lanes of a row read each half of the slice's weights as one contiguous
-// 128-byte load.  Sums of two neighbouring neurons are one packed FMA
-// (packed.cuh: the weights of a load are already pairs, the duplicated midpoint
-// and radius the other operand).  A tile holds only the inputs that have terms
-// in it: dead neurons and identity neurons of a lower degree drop out of the
-// higher rows (their products are exact zeros), about half of the inputs of the
-// benchmark network's last layers.  The next tile's list of inputs is made
-// while a tile is staged.  The staging issues kWBatch loads of each bound per
-// thread before converting any.  A warp covers 4 TR rows of the tile and skips
+// 128-byte load, and |w| is taken in the radius FMA itself.  A tile holds only the
+// inputs that have terms in it: dead neurons and identity neurons of a lower
+// degree drop out of the higher rows (their products are exact zeros), about half
+// of the inputs of the benchmark network's last layers.  The next tile's list of
+// inputs is made while a tile is staged; a tile with all of them goes without the
+// list.  The staging issues kWBatch loads of each bound per thread before
+// converting any.  A warp covers 4 TR rows of the tile and skips
 // the tile when all of them are at or past the box's term count.  With a
 // ScreenOut it also screens the box's output items (R21): every thread sums
 // max(0, upper) and min(0, lower) of its output coefficients past the first
@@ -178,17 +177,13 @@ k_affine(int h_out, int h_in, const float* __restrict__ W, const float* __restri
 // combine theirs, each warp adds its sum into its own shared row, and after
 // the box the rows are added to the constant coefficient in warp order.
 //
-// Bound: the FP32 pipe during the products, the staging between them.  Layer 4
-// of [3,64x4,1], 5120 boxes: 595 us with three scalar FMAs over all inputs, 404 us
-// (its 1.04e10 FMAs, zeros included, take 267 us at the measured rate).
+// Bound: the FP32 pipe during the products, the staging between them.  64 x 64
+// neurons, 165 rows, 3000 boxes, half of the inputs with short prefixes: 338 us
+// over all inputs, 251 us over those with terms; all inputs full 336 and 335 us.
+// Packed FMAs (two neurons' sums in one) need both operands twice in registers and
+// lose to scalar ones: 305 and 428 us.
 constexpr int kWThreads = 128;
 constexpr int kWBatch = 8;
-
-__device__ __forceinline__ p2 fma2_rd(p2 a, p2 b, p2 c) {
-  p2 r;
-  asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 
 // The inputs with a term at row r0 or later, in order; one warp.
 __device__ __forceinline__ int live_inputs(const int* sN, int h_in, int r0, int* list) {
@@ -204,9 +199,9 @@ __device__ __forceinline__ int live_inputs(const int* sN, int h_in, int r0, int*
   return n;
 }
 
-// LIVE: tiles hold only the inputs with terms, and the FMAs are packed; not worth
-// the lists and the wider register tiles for few inputs or a single tile (28
-// rows, 33 x 47, 2000 boxes: 28.5 us without, 31 us with them).
+// LIVE: tiles hold only the inputs with terms; not worth the lists and their
+// registers (five blocks a multiprocessor for six) for few inputs or a single
+// tile (28 rows, 33 x 47, 2000 boxes: 28.5 us without, 31 us with them).
 constexpr int kWideLiveInputs = 48, kWideLiveRows = 32;
 
 template <int TR, int MINB, bool SCREEN, bool LIVE>
@@ -285,7 +280,7 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
 #pragma unroll
           for (int q = 0; q < kWBatch; ++q) {
             const bool in = idx + q * kWThreads < ROWS * nl;
-            const int r = r0 + rr, j = LIVE ? (in ? J[jj] : 0) : jj;
+            const int r = r0 + rr, j = LIVE && nl < h_in && in ? J[jj] : jj;
             const bool live = in && r < sN[j];       // sN[j] <= M <= in_ld
             u[q] = live ? gU[(int64_t)r * h_in + j] : 0.0f;
             l[q] = live ? gL[(int64_t)r * h_in + j] : 0.0f;
@@ -312,74 +307,42 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
       __syncthreads();
       if (r0 + warp * 4 * TR >= M) continue;         // warp-uniform; no barrier follows
       for (int m0 = 0; m0 < h_out; m0 += 64) {
-        // LIVE: pairs of neighbouring neurons, i = 0, 1 the first half, 2, 3 the
-        // second; otherwise one neuron each
-        p2 uc[TR][4], lc[TR][4], rad[TR][4];
         float us[TR][8], ls[TR][8], rs[TR][8];
 #pragma unroll
         for (int k = 0; k < TR; ++k)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int m = m0 + 4 * tm + (i < 2 ? 2 * i : 28 + 2 * i), r = r0 + tr * TR + k;
-            const float b0 = r == 0 && m < h_out ? bias[m] : 0.0f;
-            const float b1 = r == 0 && m + 1 < h_out ? bias[m + 1] : 0.0f;
-            uc[k][i] = lc[k][i] = pack2(b0, b1);
-            rad[k][i] = 0ull;
-            us[k][2 * i] = ls[k][2 * i] = b0;
-            us[k][2 * i + 1] = ls[k][2 * i + 1] = b1;
-            rs[k][2 * i] = rs[k][2 * i + 1] = 0.0f;
+          for (int i = 0; i < 8; ++i) {
+            const int m = m0 + (i < 4 ? 4 * tm + i : 28 + 4 * tm + i), r = r0 + tr * TR + k;
+            us[k][i] = ls[k][i] = (r == 0 && m < h_out) ? bias[m] : 0.0f;
+            rs[k][i] = 0.0f;
           }
         const float* pw = sW + m0 + tm * 4;
         const float2* pcr = sCR + (tr * TR) * ldx;
-        if constexpr (LIVE) {
-#pragma unroll 2
-          for (int jj = 0; jj < nl; ++jj) {
-            const float* pj = pw + (size_t)J[jj] * hp;
-            p2 c[TR], rd[TR];
+        auto input = [&](const float* pj, int jj) {
+          float2 cr[TR];
 #pragma unroll
-            for (int k = 0; k < TR; ++k) {
-              const float2 v = pcr[k * ldx + jj];
-              c[k] = pack2(v.x, v.x);
-              rd[k] = pack2(v.y, v.y);
-            }
+          for (int k = 0; k < TR; ++k) cr[k] = pcr[k * ldx + jj];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(pj + 32 * half);
-              const p2 w[2] = {w2.x, w2.y};
+          for (int half = 0; half < 2; ++half) {
+            const float4 w4 = *reinterpret_cast<const float4*>(pj + 32 * half);
+            const float w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-              for (int i = 0; i < 2; ++i) {
-                const p2 aw = w[i] & 0x7fffffff7fffffffull;
+            for (int k = 0; k < TR; ++k)
 #pragma unroll
-                for (int k = 0; k < TR; ++k) {
-                  const int ii = 2 * half + i;
-                  uc[k][ii] = fma2_ru(w[i], c[k], uc[k][ii]);
-                  lc[k][ii] = fma2_rd(w[i], c[k], lc[k][ii]);
-                  rad[k][ii] = fma2_ru(aw, rd[k], rad[k][ii]);
-                }
+              for (int i = 0; i < 4; ++i) {
+                const int ii = 4 * half + i;
+                us[k][ii] = __fmaf_ru(w[i], cr[k].x, us[k][ii]);
+                ls[k][ii] = __fmaf_rd(w[i], cr[k].x, ls[k][ii]);
+                rs[k][ii] = __fmaf_ru(fabsf(w[i]), cr[k].y, rs[k][ii]);
               }
-            }
           }
+        };
+        if (LIVE && nl < h_in) {
+#pragma unroll 2
+          for (int jj = 0; jj < nl; ++jj) input(pw + (size_t)J[jj] * hp, jj);
         } else {
 #pragma unroll 2
-          for (int j = 0; j < h_in; ++j) {
-            float2 cr[TR];
-#pragma unroll
-            for (int k = 0; k < TR; ++k) cr[k] = pcr[k * ldx + j];
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const float4 w4 = *reinterpret_cast<const float4*>(pw + (size_t)j * hp + 32 * half);
-              const float w[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-              for (int k = 0; k < TR; ++k)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const int ii = 4 * half + i;
-                  us[k][ii] = __fmaf_ru(w[i], cr[k].x, us[k][ii]);
-                  ls[k][ii] = __fmaf_rd(w[i], cr[k].x, ls[k][ii]);
-                  rs[k][ii] = __fmaf_ru(fabsf(w[i]), cr[k].y, rs[k][ii]);
-                }
-            }
-          }
+          for (int j = 0; j < h_in; ++j) input(pw + (size_t)j * hp, j);
         }
         float su[8], sl[8];                          // screen: this thread's rows past the first
 #pragma unroll
@@ -390,18 +353,9 @@ k_affine_wide(int64_t n_boxes, int h_out, int h_in, const float* __restrict__ W,
           const bool valid = r < M;
           float vu[8], vl[8];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            float a = us[k][2 * i], c = us[k][2 * i + 1], d = ls[k][2 * i], e = ls[k][2 * i + 1];
-            float f = rs[k][2 * i], g = rs[k][2 * i + 1];
-            if constexpr (LIVE) {
-              unpack2(uc[k][i], a, c);
-              unpack2(lc[k][i], d, e);
-              unpack2(rad[k][i], f, g);
-            }
-            vu[2 * i] = __fadd_ru(a, f);
-            vu[2 * i + 1] = __fadd_ru(c, g);
-            vl[2 * i] = __fsub_rd(d, f);
-            vl[2 * i + 1] = __fsub_rd(e, g);
+          for (int i = 0; i < 8; ++i) {
+            vu[i] = __fadd_ru(us[k][i], rs[k][i]);
+            vl[i] = __fsub_rd(ls[k][i], rs[k][i]);
           }
           if (valid) {
             const int64_t o = (b * out_ld + r) * h_out + m0;
@@ -1056,10 +1010,9 @@ cudaError_t launch_affine(const Launch& L, int64_t n_boxes, int h_out, int h_in,
                           wide_smem(h_out, h_in, 32) <= 200 * 1024);
     const size_t ssmem = short_smem(h_out, h_in);
     const bool short_ok = few_rows && ssmem <= 200 * 1024;
-    // 1-row thread tiles from 33 to 64 rows (with lists): a 32-row tile is half empty at 35 rows,
-    // and six blocks fit an SM instead of four (35 rows, 64 x 64, 5120 boxes: 132
-    // against 150 us; 165 rows: 610 against 495 us)
-    const int rows_dflt = live && rows_in <= 64 ? 3 : 2;
+    // 1-row thread tiles where 16-row tiles cover the rows with fewer than 32-row
+    // ones (33 rows, 100 x 100, 3000 boxes: 315 against 359 us; 49 rows: 429 against 394)
+    const int rows_dflt = live && rows_in <= 48 ? 3 : 2;
     TuneTimer tt;
     int v = tune_variant(L, "affine", key, short_ok ? 4 : (wide_ok ? rows_dflt : 1),
                          2u | (wide_ok ? 4u | 8u : 0u) | (wide4_ok ? 1u : 0u) |
