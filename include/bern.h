@@ -194,8 +194,8 @@ int bern_set_autotune(bern_ctx* ctx, int enable);
  * (variants 0-2: 8, 4 or 2 items per block with a warp per polynomial; 3, 4:
  * a block of 128 or 320 threads per polynomial for shared-memory grids of
  * 256 cells or more at orders 3-16, else as 2; without effect on the
- * enclosures that use no grid: order 1, two and three variables up to order
- * 8, four and more up to order 10).  variant = -1 clears the
+ * enclosures that use no grid: order 1, up to three variables up to order 8,
+ * four and more up to order 10).  variant = -1 clears the
  * force.
  * Drops captured graphs.  Returns BERN_E_INVALID for an unknown kind or a
  * variant out of range. */

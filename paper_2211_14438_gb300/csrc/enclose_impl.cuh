@@ -300,8 +300,8 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
   const size_t smem = (size_t)2 * items * G * sizeof(float);
   // the in-simplex prefix loop for four or more variables (their grids of
   // l >= 12, 13^4 cells and more, exceed kEncloseGridMax and run elsewhere);
-  // fewer variables come here from order 8 on (one) and 9 on (two and three),
-  // their lower orders run in k_enclose_small and k_enclose_tail.cu
+  // fewer variables come here from order 9 on, their lower orders run in
+  // k_enclose_tail.cu
   auto kern = k_enclose<LB, (LB < 8), 0>;
   if constexpr (LB > 8)
     if (T.n == 3) kern = k_enclose<LB, false, 3>;
@@ -321,7 +321,7 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
   return e;
 }
 
-// Tiny grids ((l+1)^n <= 64: order 0, and one variable up to order 7): one lane per polynomial, the lane's grid
+// Tiny grids (order 0: one cell): one lane per polynomial, the lane's grid
 // interleaved with its warp's (element g of lane L at grid[g*32 + L]); a warp
 // takes 32 items of one bound, a block 4 groups of 32 items (both bounds).
 constexpr int kSmallGrid = 64;

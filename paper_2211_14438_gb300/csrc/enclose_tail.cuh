@@ -106,6 +106,83 @@ __device__ __forceinline__ p2 scale_pair(float l, float u, float2 sc) {
   return pack2(__fmul_ru(l, l >= 0.0f ? sc.y : sc.x), __fmul_ru(u, u >= 0.0f ? sc.y : sc.x));
 }
 
+// The terms above the order (ranks `first` on), each in [min(0, a), max(0, a)] on
+// the box: the sums of the upper ends and of the negated lower ends, rounded up, as
+// (negated lower, upper).  pu, pl: an item's coefficients, of which this thread adds
+// every step-th, eight in flight.
+//
+// Bound: the loads.  One at a time by a thread per item, or by lanes that read a
+// neuron's rows at a stride, order 2 on 3003 terms of six variables took 91 us for
+// 64 items (33 us now), on degree 16 in three variables 362 us for 32,768 (133).
+__device__ __forceinline__ p2 sum_remainder(const float* __restrict__ pu,
+                                            const float* __restrict__ pl, int h, int first,
+                                            int step, int nt) {
+  float ru = 0.0f, rl = 0.0f;
+  for (int r = first; r < nt; r += 8 * step) {
+    float u[8], l[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int k = r + q * step;
+      u[q] = k < nt ? pu[(int64_t)k * h] : 0.0f;
+      l[q] = k < nt ? pl[(int64_t)k * h] : 0.0f;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      ru = __fadd_ru(ru, fmaxf(u[q], 0.0f));
+      rl = __fadd_ru(rl, fmaxf(-l[q], 0.0f));
+    }
+  }
+  return pack2(rl, ru);
+}
+
+// The forms below are out of line: the kernels of 2 to 5 us also wait for their
+// instructions, and most calls have no such terms.
+//
+// Of one item by its thread.
+__device__ __noinline__ inline p2 thread_remainder(const float* __restrict__ pu,
+                                                   const float* __restrict__ pl, int h, int first,
+                                                   int nt) {
+  return sum_remainder(pu, pl, h, first, 1, nt);
+}
+
+// Of the items of a warp's first iw lanes (a power of two; base and nt theirs): that
+// of item lane % iw, its rows split over 32 / iw lanes.
+__device__ __noinline__ inline p2 warp_remainder(const float* __restrict__ pre_up,
+                                                 const float* __restrict__ pre_lo, int h,
+                                                 int first, int iw, int64_t base, int nt) {
+  const int lane = threadIdx.x & 31, my = lane & (iw - 1);
+  base = __shfl_sync(0xffffffffu, base, my);
+  nt = __shfl_sync(0xffffffffu, nt, my);
+  p2 v = sum_remainder(pre_up + base, pre_lo + base, h, first + lane / iw, 32 / iw, nt);
+  for (int o = iw; o < 32; o <<= 1) v = add2_ru(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// Of a block's `ib` items (s_base, s_nt: block and term count of each) into s_rl and
+// s_ru.  Called by all NT threads of the block, thread my_r * ib + my on item `my`;
+// neighbouring threads read neighbouring neurons of one row, and the item's NT / ib
+// partial sums are added in halves.
+template <int NT>
+__device__ __noinline__ void remainder_sums(const float* __restrict__ pre_up,
+                                            const float* __restrict__ pre_lo, int h, int first,
+                                            int ib, const int64_t* s_base, const int* s_nt,
+                                            p2* s_part, float* s_rl, float* s_ru) {
+  const int tid = threadIdx.x, my = tid % ib, my_r = tid / ib, rb = NT / ib;
+  p2 v = 0ull;
+  if (my_r < rb)
+    v = sum_remainder(pre_up + s_base[my], pre_lo + s_base[my], h, first + my_r, rb, s_nt[my]);
+  s_part[tid] = v;
+  __syncthreads();
+  int half = 1;
+  while (half < rb) half <<= 1;
+  for (half >>= 1; half > 0; half >>= 1) {
+    if (my_r < half && my_r + half < rb)
+      s_part[tid] = add2_ru(s_part[tid], s_part[tid + half * ib]);
+    __syncthreads();
+  }
+  if (tid < ib) unpack2(s_part[tid], s_rl[tid], s_ru[tid]);
+}
+
 // Whether (n, lb) runs the register kernels, and their launcher.
 bool enclose_tail_ok(int n, int lb);
 cudaError_t launch_enclose_tail(const Launch& L, const Tables& T, int lb, int64_t n_items, int h,

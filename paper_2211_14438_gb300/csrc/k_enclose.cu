@@ -1,7 +1,7 @@
 // Bernstein enclosure (a2) and ReLU coefficients (a3): dispatch over the
-// effective Bernstein order.  The per-order kernels are instantiated here
-// (orders 0-8) and in k_enclose_hi.cu (9-16); orders above 16 use the
-// runtime-order kernel below.
+// effective Bernstein order.  The grid kernels are instantiated here (orders 0
+// and 2-8) and in k_enclose_hi.cu (9-16); orders above 16 use the runtime-order
+// kernel below.
 #include <string>
 
 #include "enclose_tail.cuh"
@@ -122,7 +122,7 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
   int G;
   const int lb = effective_order(T.n, order, budget, &G, L.ews != nullptr);
   if (lb > T.rscale_max || T.rscale[lb] == nullptr) return cudaErrorInvalidValue;
-  // Order 1, and two and three variables up to order kTailMaxOrder: the last two
+  // Order 1, and up to three variables up to order kTailMaxOrder: the last two
   // passes in registers (k_enclose_tail.cu)
   if (enclose_tail_ok(T.n, lb))
     return launch_enclose_tail(L, T, lb, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
@@ -164,16 +164,8 @@ static cudaError_t launch_enclose_impl(const Launch& L, const Tables& T, int64_t
     if (blk) tune_end(L, key, tt);
     return e;
   }
-  if (G <= kSmallGrid && lb <= 7) {
-#define BERN_SMALL_CASE(X) \
-  case X: return launch_small<X>(L, T, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
-    switch (lb) {
-      BERN_SMALL_CASE(0) BERN_SMALL_CASE(2) BERN_SMALL_CASE(3) BERN_SMALL_CASE(4)
-      BERN_SMALL_CASE(5) BERN_SMALL_CASE(6) BERN_SMALL_CASE(7)
-      default: break;
-    }
-#undef BERN_SMALL_CASE
-  }
+  if (lb == 0)
+    return launch_small<0>(L, T, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
 #define BERN_ENC_CASE(X) \
   case X: return launch_lb<X>(L, T, G, n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro);
   switch (lb) {

@@ -453,6 +453,7 @@ k_enclose_regs(Tables T, LexView X, const float2* __restrict__ rs, int64_t n_ite
   __shared__ float s_rl[IB], s_ru[IB];
   __shared__ int64_t s_item[IB], s_base[IB];
   __shared__ int s_nt[IB];
+  __shared__ p2 s_part[kRegThreads];
   const int tid = threadIdx.x;
   for (int x = tid; x < R * R; x += kRegThreads)
     s_bin[x] = pack2(binomf(x / R, x % R), binomf(x / R, x % R));
@@ -464,6 +465,7 @@ k_enclose_regs(Tables T, LexView X, const float2* __restrict__ rs, int64_t n_ite
   const int64_t n_list = list ? (int64_t)*count : n_items;
   for (int64_t i0 = (int64_t)blockIdx.x * IB; i0 < n_list; i0 += (int64_t)gridDim.x * IB) {
     __syncthreads();                                 // the previous items are finished
+    bool above = false;
     if (tid < IB) {
       const int64_t item = i0 + tid < n_list ? (list ? (int64_t)list[i0 + tid] : i0 + tid) : -1;
       int nt = item >= 0 ? nterms[item] : 0;
@@ -477,16 +479,12 @@ k_enclose_regs(Tables T, LexView X, const float2* __restrict__ rs, int64_t n_ite
       s_nt[tid] = nt;
       s_bl[tid] = float_key(-CUDART_INF_F);
       s_bu[tid] = float_key(-CUDART_INF_F);
-      // terms above the order: their one-sided ranges
-      float ru = 0.0f, rl = 0.0f;
-      for (int r = MN; r < nt; ++r) {
-        ru = __fadd_ru(ru, fmaxf(pre_up[s_base[tid] + (int64_t)r * h], 0.0f));
-        rl = __fadd_ru(rl, fmaxf(-pre_lo[s_base[tid] + (int64_t)r * h], 0.0f));
-      }
-      s_rl[tid] = rl;
-      s_ru[tid] = ru;
+      s_rl[tid] = 0.0f;
+      s_ru[tid] = 0.0f;
+      above = nt > MN;
     }
-    __syncthreads();
+    if (__syncthreads_or(above))
+      remainder_sums<kRegThreads>(pre_up, pre_lo, h, MN, IB, s_base, s_nt, s_part, s_rl, s_ru);
     if (my_r < RB) {
       const int nt = s_nt[my];
       const float* pu = pre_up + s_base[my];
@@ -564,13 +562,14 @@ k_enclose_expand(Tables T, LexView X, ExpandShape sh, const float2* __restrict__
                  const float* __restrict__ pre_lo, int64_t ld, const int32_t* __restrict__ nterms,
                  float* __restrict__ lo, float* __restrict__ hi, const int* list, const int* count,
                  int* status) {
-  constexpr int R = LB + 1, NW = NT / 32, IBMAX = NT / R, BOT = expand_bottom<LB>();
+  constexpr int R = LB + 1, IBMAX = NT / R, BOT = expand_bottom<LB>();
   extern __shared__ p2 sm[];
   __shared__ p2 s_bin[R * R];
   __shared__ int s_bl[IBMAX], s_bu[IBMAX], s_nt[IBMAX], s_any;
   __shared__ float s_rl[IBMAX], s_ru[IBMAX];
   __shared__ int64_t s_item[IBMAX], s_base[IBMAX];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ p2 s_part[NT];
+  const int tid = threadIdx.x, lane = tid & 31;
   const int n = sh.n, ib = sh.ib, Mn = sh.M[n];
   uint16_t* tab = reinterpret_cast<uint16_t*>(sm);
   for (int x = tid; x < R * R; x += NT) s_bin[x] = pack2(binomf(x / R, x % R), binomf(x / R, x % R));
@@ -615,23 +614,8 @@ k_enclose_expand(Tables T, LexView X, ExpandShape sh, const float2* __restrict__
       if (my_r == 0 && nt > Mn) s_any = 1;
     }
     __syncthreads();
-    if (s_any) {
-      // terms above the order: their one-sided ranges, a warp per item
-      for (int i = warp; i < ib; i += NW) {
-        float ru = 0.0f, rl = 0.0f;
-        for (int r = lane; r < s_nt[i]; r += 32) {
-          if (r < Mn) continue;
-          ru = __fadd_ru(ru, fmaxf(pre_up[s_base[i] + (int64_t)r * h], 0.0f));
-          rl = __fadd_ru(rl, fmaxf(-pre_lo[s_base[i] + (int64_t)r * h], 0.0f));
-        }
-        ru = warp_dsum<true>(ru);
-        rl = warp_dsum<true>(rl);
-        if (lane == 0) {
-          s_ru[i] = ru;
-          s_rl[i] = rl;
-        }
-      }
-    }
+    if (s_any)
+      remainder_sums<NT>(pre_up, pre_lo, h, Mn, ib, s_base, s_nt, s_part, s_rl, s_ru);
     int ns = ib;                                     // slabs of the level above
     for (int m = n - 1; m >= BOT; --m) {
       const int rows = sh.M[m], sa = sh.stride[m + 1], sb = sh.stride[m];

@@ -1,4 +1,4 @@
-// a2 (Sec. 5.1 Step 1 with Def. 2) for two and three variables at the orders
+// a2 (Sec. 5.1 Step 1 with Def. 2) for one to three variables at the orders
 // whose last two passes fit a thread's registers, and for order 1.
 //
 // The passes of enclose_impl.cuh run from the last variable to the first, so
@@ -50,7 +50,8 @@ k_enclose_tail3(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
   __shared__ float s_rl[IB], s_ru[IB];
   __shared__ int64_t s_item[IB], s_base[IB];
   __shared__ int s_nt[IB], s_any;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ p2 s_part[kTailThreads];
+  const int tid = threadIdx.x;
   for (int x = tid; x < R * R; x += kTailThreads)
     s_bin[x] = pack2(binomf(x / R, x % R), binomf(x / R, x % R));
   for (int r = tid; r < M3; r += kTailThreads) {
@@ -97,23 +98,8 @@ k_enclose_tail3(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
       if (my_r == 0 && nt > M3) s_any = 1;
     }
     __syncthreads();
-    if (s_any) {
-      // terms above the order: their one-sided ranges, a warp per item
-      for (int i = warp; i < IB; i += kTailThreads / 32) {
-        float ru = 0.0f, rl = 0.0f;
-        for (int r = lane; r < s_nt[i]; r += 32) {
-          if (r < M3) continue;
-          ru = __fadd_ru(ru, fmaxf(pre_up[s_base[i] + (int64_t)r * h], 0.0f));
-          rl = __fadd_ru(rl, fmaxf(-pre_lo[s_base[i] + (int64_t)r * h], 0.0f));
-        }
-        ru = warp_dsum<true>(ru);
-        rl = warp_dsum<true>(rl);
-        if (lane == 0) {
-          s_ru[i] = ru;
-          s_rl[i] = rl;
-        }
-      }
-    }
+    if (s_any)
+      remainder_sums<kTailThreads>(pre_up, pre_lo, h, M3, IB, s_base, s_nt, s_part, s_rl, s_ru);
     if (tid < IB * R && i0 + tid / R < n_list) {
       float bl = -CUDART_INF_F, bu = -CUDART_INF_F;
       tail_max<LB>(s_c + tid / R * MS, tid % R, s_bin, bl, bu);
@@ -136,52 +122,65 @@ k_enclose_tail3(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
   }
 }
 
-// Two variables: a thread per item, its coefficients straight into registers
+// One and two variables: a thread per item, its coefficients straight into registers
 // (rank of (j_1, j_2): s (s + 1) / 2 + j_2, s = j_1 + j_2).  Neighbouring
-// threads take neighbouring items.
-template <int LB>
-__global__ void __launch_bounds__(128)
+// threads take neighbouring items, each its own terms above the order: at most 150
+// rows, and lanes that share them cost calls without any (order 8, 1024 items 5.3
+// us for 4.7).
+constexpr int kTail2Threads = 128;
+template <int NV, int LB>
+__global__ void __launch_bounds__(kTail2Threads)
 k_enclose_tail2(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
                 const float* __restrict__ pre_up, const float* __restrict__ pre_lo, int64_t ld,
                 const int32_t* __restrict__ nterms, float* __restrict__ lo,
                 float* __restrict__ hi, EncloseOpts ro, int* status) {
-  constexpr int R = LB + 1, M2 = R * (R + 1) / 2;
+  constexpr int R = LB + 1, M2 = NV == 1 ? R : R * (R + 1) / 2;
   const int64_t n_list = ro.list ? (int64_t)*ro.count : n_items;
-  for (int64_t at = (int64_t)blockIdx.x * 128 + threadIdx.x; at < n_list;
-       at += (int64_t)gridDim.x * 128) {
-    const int64_t item = ro.list ? (int64_t)ro.list[at] : at;
+  for (int64_t at_list = (int64_t)blockIdx.x * kTail2Threads + threadIdx.x; at_list < n_list;
+       at_list += (int64_t)gridDim.x * kTail2Threads) {
+    const int64_t item = ro.list ? (int64_t)ro.list[at_list] : at_list;
     int nt = nterms[item];
     if (nt < 0 || nt > ld || nt > T.mexps) {
       atomicOr(status, kStatusInvalid);
       nt = 0;
     }
     const int64_t b = item / h;
-    const float* pu = pre_up + (b * ld) * h + (item - b * h);
-    const float* pl = pre_lo + (b * ld) * h + (item - b * h);
+    const int64_t base = (b * ld) * h + (item - b * h);
+    const float* pu = pre_up + base;
+    const float* pl = pre_lo + base;
+    // rank r of degree s, exponent j of t_2
     p2 q[M2];
+    auto at = [](int s, int j) { return NV == 1 ? s : lex2(LB, s - j) + j; };
 #pragma unroll
     for (int s = 0; s <= LB; ++s)
 #pragma unroll
-      for (int j = 0; j <= s; ++j) {
-        const int r = s * (s + 1) / 2 + j;
-        q[lex2(LB, s - j) + j] = r < nt ? pack2(-pl[(int64_t)r * h], pu[(int64_t)r * h])
-                                        : pack2(0.0f, 0.0f);
+      for (int j = 0; j <= (NV == 1 ? 0 : s); ++j) {
+        const int r = NV == 1 ? s : s * (s + 1) / 2 + j;
+        q[at(s, j)] = r < nt ? pack2(-pl[(int64_t)r * h], pu[(int64_t)r * h]) : pack2(0.0f, 0.0f);
       }
 #pragma unroll
     for (int s = 0; s <= LB; ++s)
 #pragma unroll
-      for (int j = 0; j <= s; ++j) {
+      for (int j = 0; j <= (NV == 1 ? 0 : s); ++j) {
         float l, u;
-        unpack2(q[lex2(LB, s - j) + j], l, u);
-        q[lex2(LB, s - j) + j] = scale_pair(l, u, __ldg(rs + s * (s + 1) / 2 + j));
+        unpack2(q[at(s, j)], l, u);
+        q[at(s, j)] = scale_pair(l, u, __ldg(rs + (NV == 1 ? s : s * (s + 1) / 2 + j)));
       }
-    float ru = 0.0f, rl = 0.0f;
-    for (int r = M2; r < nt; ++r) {
-      ru = __fadd_ru(ru, fmaxf(pu[(int64_t)r * h], 0.0f));
-      rl = __fadd_ru(rl, fmaxf(-pl[(int64_t)r * h], 0.0f));
-    }
     float bl = -CUDART_INF_F, bu = -CUDART_INF_F;
-    pair_max<LB>(q, bl, bu);
+    if constexpr (NV == 1) {
+      pair_transform<LB>(q);
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        float l, u;
+        unpack2(q[i], l, u);
+        bl = fmaxf(bl, l);
+        bu = fmaxf(bu, u);
+      }
+    } else {
+      pair_max<LB>(q, bl, bu);
+    }
+    float ru = 0.0f, rl = 0.0f;
+    if (nt > M2) unpack2(thread_remainder(pu, pl, h, M2, nt), rl, ru);
     const float l = -__fadd_ru(bl, rl), u = __fadd_ru(bu, ru);
     lo[item] = l;
     hi[item] = u;
@@ -197,18 +196,26 @@ k_enclose_tail2(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
 // Order 1: the coefficients are the values at the vertices, and with the
 // passes' rounding from the last variable to the first the largest is
 // a_0 plus the positive linear coefficients in that order.  A thread per
-// item.
-__global__ void __launch_bounds__(256)
+// item, 32 to a warp; SPLIT: iw to a warp, whose lanes share the terms above the
+// order.
+constexpr int kOrder1Threads = 256;
+template <bool SPLIT>
+__global__ void __launch_bounds__(kOrder1Threads)
 k_enclose_order1(Tables T, int64_t n_items, int h, const float* __restrict__ pre_up,
                  const float* __restrict__ pre_lo, int64_t ld,
                  const int32_t* __restrict__ nterms, float* __restrict__ lo,
-                 float* __restrict__ hi, EncloseOpts ro, int* status) {
+                 float* __restrict__ hi, EncloseOpts ro, int iw, int* status) {
   const int n = T.n;
   const int64_t n_list = ro.list ? (int64_t)*ro.count : n_items;
-  for (int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; at < n_list;
-       at += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t item = ro.list ? (int64_t)ro.list[at] : at;
-    int nt = nterms[item];
+  // SPLIT: warp-uniform, lane 0's item
+  const int per = SPLIT ? iw * (kOrder1Threads / 32) : kOrder1Threads;
+  const int lane = threadIdx.x & 31;
+  for (int64_t i0 = (int64_t)blockIdx.x * per + (SPLIT ? (int)(threadIdx.x >> 5) * iw : threadIdx.x);
+       i0 < n_list; i0 += (int64_t)gridDim.x * per) {
+    const int64_t at = SPLIT ? i0 + lane : i0;
+    const bool mine = !SPLIT || (lane < iw && at < n_list);
+    const int64_t item = !mine ? 0 : ro.list ? (int64_t)ro.list[at] : at;
+    int nt = mine ? nterms[item] : 0;
     if (nt < 0 || nt > ld || nt > T.mexps) {
       atomicOr(status, kStatusInvalid);
       nt = 0;
@@ -232,13 +239,16 @@ k_enclose_order1(Tables T, int64_t n_items, int h, const float* __restrict__ pre
       u = __fadd_ru(u, fmaxf(cu[k], 0.0f));
       l = __fadd_rd(l, fminf(cl[k], 0.0f));
     }
-    float ru = 0.0f, rl = 0.0f;
-    for (int r = n + 1; r < nt; ++r) {
-      ru = __fadd_ru(ru, fmaxf(pre_up[base + (int64_t)r * h], 0.0f));
-      rl = __fadd_rd(rl, fminf(pre_lo[base + (int64_t)r * h], 0.0f));
+    float ru = 0.0f, rl = 0.0f;                      // rl: negated
+    if constexpr (SPLIT) {
+      if (__any_sync(0xffffffffu, nt > n + 1))
+        unpack2(warp_remainder(pre_up, pre_lo, h, n + 1, iw, base, nt), rl, ru);
+      if (!mine) continue;
+    } else {
+      if (nt > n + 1) unpack2(thread_remainder(pre_up + base, pre_lo + base, h, n + 1, nt), rl, ru);
     }
     u = __fadd_ru(u, ru);
-    l = __fadd_rd(l, rl);
+    l = __fsub_rd(l, rl);
     lo[item] = l;
     hi[item] = u;
     if (!(isfinite(l) && isfinite(u))) atomicOr(status, kStatusNonFinite);
@@ -253,8 +263,7 @@ k_enclose_order1(Tables T, int64_t n_items, int h, const float* __restrict__ pre
 }  // namespace
 
 bool enclose_tail_ok(int n, int lb) {
-  return lb == 1 || (n == 2 && lb >= 2 && lb <= kTailMaxOrder) ||
-         (n == 3 && lb >= 2 && lb <= kTailMaxOrder);
+  return lb == 1 || (n <= 3 && lb >= 2 && lb <= kTailMaxOrder);
 }
 
 cudaError_t launch_enclose_tail(const Launch& L, const Tables& T, int lb, int64_t n_items, int h,
@@ -264,19 +273,27 @@ cudaError_t launch_enclose_tail(const Launch& L, const Tables& T, int lb, int64_
   const int64_t sms = device_sms(L);
   ++*L.launches;
   if (lb == 1) {
-    const int64_t blocks = std::min<int64_t>((n_items + 255) / 256, sms * 8);
-    k_enclose_order1<<<(unsigned)blocks, 256, 0, L.stream>>>(T, n_items, h, pre_up, pre_lo, ld,
-                                                             nterms, lo, hi, ro, L.status);
+    // Fewer items a warp where rows past the order call for more lanes an item and
+    // the items do not give eight warps a multiprocessor
+    int iw = 32;
+    while (iw > 1 && ld > T.n + 1 + 64 && n_items < 8 * sms * iw) iw >>= 1;
+    const int64_t per = iw * (kOrder1Threads / 32);
+    const int64_t blocks = std::min<int64_t>((n_items + per - 1) / per, sms * 8);
+    auto kern = iw < 32 ? k_enclose_order1<true> : k_enclose_order1<false>;
+    kern<<<(unsigned)blocks, kOrder1Threads, 0, L.stream>>>(T, n_items, h, pre_up, pre_lo, ld,
+                                                            nterms, lo, hi, ro, iw, L.status);
     return cudaGetLastError();
   }
-  if (T.n == 2) {
-    const int64_t blocks = std::min<int64_t>((n_items + 127) / 128, sms * 16);
+  if (T.n <= 2) {
+    const int64_t blocks =
+        std::min<int64_t>((n_items + kTail2Threads - 1) / kTail2Threads, sms * 16);
 #define BERN_T2(X)                                                                              \
-  case X:                                                                                       \
-    k_enclose_tail2<X><<<(unsigned)blocks, 128, 0, L.stream>>>(T, T.rscale[X], n_items, h, pre_up, \
-                                                               pre_lo, ld, nterms, lo, hi, ro,  \
-                                                               L.status);                       \
-    return cudaGetLastError();
+  case X: {                                                                                     \
+    auto kern = T.n == 1 ? k_enclose_tail2<1, X> : k_enclose_tail2<2, X>;                       \
+    kern<<<(unsigned)blocks, kTail2Threads, 0, L.stream>>>(T, T.rscale[X], n_items, h, pre_up,   \
+                                                           pre_lo, ld, nterms, lo, hi, ro, L.status); \
+    return cudaGetLastError();                                                                  \
+  }
     switch (lb) {
       BERN_T2(2) BERN_T2(3) BERN_T2(4) BERN_T2(5) BERN_T2(6) BERN_T2(7) BERN_T2(8)
       default: return cudaErrorInvalidValue;
@@ -286,9 +303,8 @@ cudaError_t launch_enclose_tail(const Launch& L, const Tables& T, int lb, int64_
 #define BERN_T3(X)                                                                              \
   case X: {                                                                                     \
     const int64_t need = (n_items + tail_items<X>() - 1) / tail_items<X>();                     \
-    k_enclose_tail3<X><<<(unsigned)std::min<int64_t>(need, sms * 16), kTailThreads, 0,           \
-                         L.stream>>>(T, T.rscale[X], n_items, h, pre_up, pre_lo, ld, nterms, lo, \
-                                     hi, ro, L.status);                                         \
+    k_enclose_tail3<X><<<(unsigned)std::min<int64_t>(need, sms * 16), kTailThreads, 0, L.stream>>>(           \
+        T, T.rscale[X], n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro, L.status);          \
     return cudaGetLastError();                                                                  \
   }
   switch (lb) {
