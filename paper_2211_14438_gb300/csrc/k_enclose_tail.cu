@@ -24,7 +24,11 @@ namespace bern {
 namespace {
 
 // Threads of a block of the three-variable kernel; a block takes as many items
-// as give every thread one (item, digit of t_3) task.
+// as give every thread one (item, digit of t_3) task, or one where the items are
+// so few that all threads do best to load its coefficients: up to four of them a
+// multiprocessor, two from order 7 on, whose one wave of blocks holds no more (order
+// 5, 64 items 4.5 us in full blocks, 3.2 in blocks of their own; 1024 items 4.6 and
+// 4.9; order 8, 600 items 5.8 and 6.9).
 constexpr int kTailThreads = 128;
 template <int LB>
 constexpr int tail_items() {
@@ -34,14 +38,14 @@ constexpr int tail_items() {
 // Three variables: the scaled coefficients of the block's items sit in shared
 // memory in lexicographic order (rows of t_3), a thread takes one digit i_3
 // of one item's two polynomials.
-template <int LB>
+template <int LB, int IB>
 __global__ void __launch_bounds__(kTailThreads, (LB >= 7 ? 4 : (LB >= 5 ? 6 : 8)))
 k_enclose_tail3(Tables T, const float2* __restrict__ rs, int64_t n_items, int h,
                 const float* __restrict__ pre_up, const float* __restrict__ pre_lo, int64_t ld,
                 const int32_t* __restrict__ nterms, float* __restrict__ lo,
                 float* __restrict__ hi, EncloseOpts ro, int* status) {
   constexpr int R = LB + 1, M3 = R * (R + 1) * (R + 2) / 6, MS = M3 | 1;
-  constexpr int IB = tail_items<LB>(), RB = kTailThreads / IB;   // rows loaded at a time
+  constexpr int RB = kTailThreads / IB;                        // rows loaded at a time
   __shared__ p2 s_c[IB * MS];
   __shared__ p2 s_bin[R * R];
   __shared__ float2 s_sc[M3];
@@ -300,10 +304,12 @@ cudaError_t launch_enclose_tail(const Launch& L, const Tables& T, int lb, int64_
     }
 #undef BERN_T2
   }
+  const bool few = n_items <= (lb <= 6 ? 4 : 2) * sms;
 #define BERN_T3(X)                                                                              \
   case X: {                                                                                     \
-    const int64_t need = (n_items + tail_items<X>() - 1) / tail_items<X>();                     \
-    k_enclose_tail3<X><<<(unsigned)std::min<int64_t>(need, sms * 16), kTailThreads, 0, L.stream>>>(           \
+    const int64_t ib = few ? 1 : tail_items<X>(), need = (n_items + ib - 1) / ib;               \
+    auto kern = few ? k_enclose_tail3<X, 1> : k_enclose_tail3<X, tail_items<X>()>;              \
+    kern<<<(unsigned)std::min<int64_t>(need, sms * 16), kTailThreads, 0, L.stream>>>(           \
         T, T.rscale[X], n_items, h, pre_up, pre_lo, ld, nterms, lo, hi, ro, L.status);          \
     return cudaGetLastError();                                                                  \
   }
