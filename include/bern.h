@@ -195,8 +195,7 @@ int bern_set_autotune(bern_ctx* ctx, int enable);
  * a block of 128 or 320 threads per polynomial for shared-memory grids of
  * 256 cells or more at orders 3-16, else as 2; without effect on the
  * enclosures that use no grid: order 1, up to three variables up to order 8,
- * four and more up to order 10).  variant = -1 clears the
- * force.
+ * four and more up to order 9).  variant = -1 clears the force.
  * Drops captured graphs.  Returns BERN_E_INVALID for an unknown kind or a
  * variant out of range. */
 int bern_force_variant(bern_ctx* ctx, const char* kind, int variant);

@@ -148,7 +148,7 @@ constexpr int kProdStride = kMaxTableDegree + 1;   // prod[Dq * kProdStride + Ds
 // 24 on; off[m] the C(m-1+l, m-1) + 1 row offsets of m variables (a row: the
 // monomials sharing all exponents but the last); wt[m] the products
 // prod_k C(l, j_k) of m variables, rounded up.
-constexpr int kSlabMaxOrder = 10;
+constexpr int kSlabMaxOrder = 9;
 struct LexView {
   const uint32_t* pos = nullptr;
   const int32_t* off[kMaxVars + 1] = {};

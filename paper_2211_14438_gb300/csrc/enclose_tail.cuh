@@ -10,7 +10,7 @@
 namespace bern {
 
 // Largest order of the register passes of two and three variables: 45 pairs
-// of coefficients at order 8 (66 at order 10, the slab kernel's largest).
+// of coefficients at order 8 (55 at order 9, the slab kernel's largest).
 constexpr int kTailMaxOrder = 8;
 
 // Lexicographic order of the exponents of total degree <= l, the last exponent
@@ -113,7 +113,7 @@ __device__ __forceinline__ p2 scale_pair(float l, float u, float2 sc) {
 //
 // Bound: the loads.  One at a time by a thread per item, or by lanes that read a
 // neuron's rows at a stride, order 2 on 3003 terms of six variables took 91 us for
-// 64 items (33 us now), on degree 16 in three variables 362 us for 32,768 (133).
+// 64 items (11 us now), on degree 16 in three variables 362 us for 32,768 (66).
 __device__ __forceinline__ p2 sum_remainder(const float* __restrict__ pu,
                                             const float* __restrict__ pl, int h, int first,
                                             int step, int nt) {

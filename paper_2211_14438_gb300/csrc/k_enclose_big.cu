@@ -1,8 +1,8 @@
 // a2 for Bernstein grids larger than shared memory (Sec. 5.1 Step 1 with
 // Def. 2, the full tensor-product grid of order l in every variable):
 // (l+1)^n cells up to the caller's budget, e.g. 13^5 = 371,293 cells for five
-// inputs at order 12; orders up to 10 of four and more variables run in
-// k_enclose_slab.cu, order 10 of six here.  One block per polynomial works on its own slice of a
+// inputs at order 12; lower orders of four and more variables run in
+// k_enclose_slab.cu (up to kSlabMaxOrder).  One block per polynomial works on its own slice of a
 // global workspace (resident in L2 while the block runs): the scaled
 // coefficients are scattered to their grid cells, then the per-variable
 // triangular transforms run from the last variable to the first, the threads

@@ -35,6 +35,10 @@
 // Bound: FP32 issue in the register passes (610 of about 1000 instructions of
 // a digit at order 8 are packed FMAs; the FP32 pipe is 48% busy).
 //
+// Order 10 stays on the grids: its 66 pairs of coefficients do not fit a thread's
+// registers beside the passes (four variables, 32,768 items 7.2 ms for 2.6 ms, five
+// 36 for 26 ms; order 9 1.56 for 1.65 and 6.3 for 19.2 ms).
+//
 // Three forms, by what fits where (launch_enclose_slab): order 2, and orders 3
 // and 4 of few variables, fix every digit above t_3 in registers
 // (k_enclose_regs); up to the shared memory of a quarter SM all slabs of a
@@ -737,7 +741,7 @@ cudaError_t launch_expand(const Launch& L, const Tables& T, const LexView& X, co
 
 #define BERN_SLAB_CASES                                                                       \
   BERN_SLAB(2, 32) BERN_SLAB(3, 32) BERN_SLAB(4, 64) BERN_SLAB(5, 128) BERN_SLAB(6, 256)      \
-  BERN_SLAB(7, 256) BERN_SLAB(8, 256) BERN_SLAB(9, 256) BERN_SLAB(10, 256)
+  BERN_SLAB(7, 256) BERN_SLAB(8, 256) BERN_SLAB(9, 256)
 
 bool enclose_slab_ok(const Tables& T, int lb) {
   if (!T.lex || T.n < 4 || lb < 2 || lb > kSlabMaxOrder || !T.lex[lb].pos) return false;

@@ -20,3 +20,20 @@ assert lib.bern_affine(h, %d, %d, %d, empty(8), empty(8), empty(8), empty(8), %d
 names = launched()
 assert len(names) == 1 and %r in names[0], names
 """ % (boxes, h_out, h_in, rows, rows, kernel))
+
+
+@pytest.mark.parametrize("n,l,kernels", [
+    (4, 10, "enclose"), (5, 10, "k_enclose_big"), (4, 9, "k_enclose_slab"), (5, 9, "k_enclose_slab"),
+    (6, 9, "k_enclose_slab"),
+    (8, 4, "k_enclose_slab"), (6, 5, "k_enclose_slab"), (4, 8, "k_enclose_expand")])
+def test_enclose(tmp_path, n, l, kernels):
+    """Orders and variables at the ends of the enclosure's forms."""
+    run(tmp_path, """
+h = context()
+n, l = %d, %d
+assert lib.bern_enclose(h, n, 2, 3, l, 0, empty(8), empty(8), bern.num_monomials(n, l), empty(8),
+                        empty(8), empty(8)) == 0
+names = launched()
+assert len(names) == 1 and %r in names[0], names
+assert l < 10 or "slab" not in names[0], names
+""" % (n, l, kernels))
