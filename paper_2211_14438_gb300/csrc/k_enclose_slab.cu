@@ -41,7 +41,7 @@
 //
 // Three forms, by what fits where (launch_enclose_slab): order 2, and orders 3
 // and 4 of few variables, fix every digit above t_3 in registers
-// (k_enclose_regs); up to the shared memory of a quarter SM all slabs of a
+// (k_enclose_regs); up to the shared memory of half an SM all slabs of a
 // level are made at once, without bounds (k_enclose_expand); above, digit by
 // digit with pruning (k_enclose_slab).  Measured against the grid kernels on
 // the layers of the [6,100x3,2] network, 2048 boxes: order 2 344 -> 85 us,
@@ -542,6 +542,10 @@ cudaError_t launch_regs(const Launch& L, const Tables& T, const LexView& X, int6
 // grids have too few slabs per item to fill a block, and too little behind a
 // slab to pay for its bound.
 constexpr int64_t kExpandBytes = 52 * 1024;   // shared memory of a block: four per SM
+// Of a block with one item: two per SM.  Digit by digit, a small item is a chain of
+// barriers (order 3 in eight variables, one item 99 us on the grid, 232 us in slabs,
+// 12 us here, 32,768 items 36, 3.6 and 1.2 ms).
+constexpr int64_t kExpandOneBytes = 110 * 1024;
 
 struct ExpandShape {
   int n, ib;                   // items per block
@@ -706,7 +710,8 @@ bool expand_shape(int n, ExpandShape* s) {
     if (slabs > 4096) return false;
   }
   s->slabs = (int)slabs;
-  const int64_t fit = (kExpandBytes / (int64_t)sizeof(p2) - tab) / (a + b);
+  int64_t fit = (kExpandBytes / (int64_t)sizeof(p2) - tab) / (a + b);
+  if (fit < 1 && tab + a + b <= kExpandOneBytes / (int64_t)sizeof(p2)) fit = 1;
   if (fit < 1) return false;
   const int64_t fill = std::max<int64_t>(1, NT / (slabs * R));   // items whose tasks fill the block
   s->ib = (int)std::min<int64_t>(fit, fill);

@@ -24,7 +24,7 @@ assert len(names) == 1 and %r in names[0], names
 
 @pytest.mark.parametrize("n,l,kernels", [
     (4, 10, "enclose"), (5, 10, "k_enclose_big"), (4, 9, "k_enclose_slab"), (5, 9, "k_enclose_slab"),
-    (6, 9, "k_enclose_slab"),
+    (6, 9, "k_enclose_slab"), (7, 4, "k_enclose_expand"), (8, 3, "k_enclose_expand"),
     (8, 4, "k_enclose_slab"), (6, 5, "k_enclose_slab"), (4, 8, "k_enclose_expand")])
 def test_enclose(tmp_path, n, l, kernels):
     """Orders and variables at the ends of the enclosure's forms."""
