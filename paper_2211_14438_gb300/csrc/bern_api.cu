@@ -32,14 +32,23 @@ struct DevBuf {
     if (want <= bytes) return cudaSuccess;
     release();
     cudaError_t e = cudaMalloc(&p, want);
-    if (e == cudaSuccess) bytes = want;
+    if (e == cudaSuccess)
+      bytes = want;
+    else
+      cudaGetLastError();   // returned here: not the error of a later launch
     return e;
   }
 };
 
+// A copy to the device, its error returned and not left for a later launch.
+cudaError_t copy_in(void* dst, const void* src, size_t size) {
+  const cudaError_t e = cudaMemcpy(dst, src, size, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 struct TableSet {
   int dmax = -1;
-  DevBuf exps, mcount;
   std::vector<DevBuf> bufs;
   Tables view{};
   // product tables of the Horner kernel, built on demand; prod_arr is the
@@ -48,6 +57,22 @@ struct TableSet {
   std::vector<ProdTable> prod_host;
   DevBuf prod_arr;
   std::vector<LexView> lex;         // by order, host array of Tables::lex
+  // A buffer of this set with a copy of src (16 bytes at least), or the error of
+  // either step.
+  template <class P>
+  cudaError_t upload(const void* src, size_t size, P** dst) {
+    DevBuf b;
+    cudaError_t e = b.reserve(std::max<size_t>(16, size));
+    if (e != cudaSuccess) return e;
+    bufs.push_back(b);
+    if (size) e = copy_in(b.p, src, size);
+    *dst = (P*)b.p;
+    return e;
+  }
+  template <class T, class P>
+  cudaError_t upload(const std::vector<T>& v, P** dst) {
+    return upload(v.data(), v.size() * sizeof(T), dst);
+  }
 };
 
 struct GraphEntry {
@@ -159,28 +184,19 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
   const int De = exps_degree(n);
   std::vector<uint8_t> ex;
   graded_monomials(n, De, ex);
-  cudaError_t e = ts.exps.reserve(ex.size());
+  cudaError_t e = ts.upload(ex, &ts.view.exps);
   if (e != cudaSuccess) return map_cuda(e);
-  cudaMemcpy(ts.exps.p, ex.data(), ex.size(), cudaMemcpyHostToDevice);
   std::vector<int32_t> mc(kMaxTableDegree + 1);
   for (int D = 0; D <= kMaxTableDegree; ++D) {
     int64_t m = num_monomials(n, D);
     mc[D] = (m < 0 || m > INT32_MAX) ? INT32_MAX : (int32_t)m;
   }
-  e = ts.mcount.reserve(mc.size() * sizeof(int32_t));
-  if (e != cudaSuccess) return map_cuda(e);
-  cudaMemcpy(ts.mcount.p, mc.data(), mc.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-  ts.view.exps = (const uint8_t*)ts.exps.p;
-  ts.view.mcount = (const int32_t*)ts.mcount.p;
+  if ((e = ts.upload(mc, &ts.view.mcount)) != cudaSuccess) return map_cuda(e);
   ts.view.mexps = num_monomials(n, De);
   {
     std::vector<uint8_t> dof;
     build_degree_of(n, De, dof);
-    DevBuf b;
-    if ((e = b.reserve(dof.size())) != cudaSuccess) return map_cuda(e);
-    cudaMemcpy(b.p, dof.data(), dof.size(), cudaMemcpyHostToDevice);
-    ts.view.deg_of = (const uint8_t*)b.p;
-    ts.bufs.push_back(b);
+    if ((e = ts.upload(dof, &ts.view.deg_of)) != cudaSuccess) return map_cuda(e);
   }
   // reciprocal brackets and grid indices up to the largest order of any
   // enclosure; line tables only for the shared-memory kernels' orders
@@ -189,26 +205,11 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
   for (int l = 0; l <= ts.view.rscale_max; ++l) {
     std::vector<float> rs;
     build_rscale(n, l, rs);
-    DevBuf b;
-    if ((e = b.reserve(rs.size() * sizeof(float))) != cudaSuccess) return map_cuda(e);
-    cudaMemcpy(b.p, rs.data(), rs.size() * sizeof(float), cudaMemcpyHostToDevice);
-    ts.view.rscale[l] = (const float2*)b.p;
-    ts.bufs.push_back(b);
+    if ((e = ts.upload(rs, &ts.view.rscale[l])) != cudaSuccess) return map_cuda(e);
     std::vector<int32_t> gi, li;
     build_enclose_tables(n, l, gi, li, l <= lines_max);
-    DevBuf bg, bl;
-    if ((e = bg.reserve(gi.size() * sizeof(int32_t))) != cudaSuccess) return map_cuda(e);
-    if (!li.empty() && (e = bl.reserve(li.size() * sizeof(int32_t))) != cudaSuccess) {
-      bg.release();
-      return map_cuda(e);
-    }
-    cudaMemcpy(bg.p, gi.data(), gi.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-    if (!li.empty())
-      cudaMemcpy(bl.p, li.data(), li.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-    ts.view.gidx[l] = (const int32_t*)bg.p;
-    ts.view.lines[l] = (const int2*)bl.p;
-    ts.bufs.push_back(bg);
-    ts.bufs.push_back(bl);
+    if ((e = ts.upload(gi, &ts.view.gidx[l])) != cudaSuccess) return map_cuda(e);
+    if (!li.empty() && (e = ts.upload(li, &ts.view.lines[l])) != cudaSuccess) return map_cuda(e);
   }
   // the slab enclosure's tables, all arrays of one order in one buffer
   if (n >= 4) {
@@ -231,11 +232,8 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
         at_off[m] = put(off[m].data(), off[m].size());
         at_wt[m] = put(wt[m].data(), wt[m].size());
       }
-      DevBuf b;
-      if ((e = b.reserve(img.size() * sizeof(uint32_t))) != cudaSuccess) return map_cuda(e);
-      cudaMemcpy(b.p, img.data(), img.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
-      ts.bufs.push_back(b);
-      const uint32_t* d = (const uint32_t*)b.p;
+      const uint32_t* d;
+      if ((e = ts.upload(img, &d)) != cudaSuccess) return map_cuda(e);
       ts.lex[l].pos = d + at_pos;
       for (int m = 0; m <= n; ++m) {
         if (!off[m].empty()) ts.lex[l].off[m] = (const int32_t*)(d + at_off[m]);
@@ -252,20 +250,12 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
     rt.m_in = ri.m_in;
     rt.n_out_rows = ri.n_out_rows;
     rt.row_split = ri.row_split;
-    auto up = [&](const std::vector<int32_t>& v, const void** dst) -> cudaError_t {
-      DevBuf b;
-      cudaError_t e2 = b.reserve(std::max<size_t>(16, v.size() * sizeof(int32_t)));
-      if (e2 != cudaSuccess) return e2;
-      if (!v.empty()) cudaMemcpy(b.p, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-      *dst = b.p;
-      ts.bufs.push_back(b);
-      return cudaSuccess;
-    };
-    if ((e = up(ri.pos_in, (const void**)&rt.pos_in)) != cudaSuccess) return map_cuda(e);
-    if ((e = up(ri.hdr, (const void**)&rt.hdr)) != cudaSuccess) return map_cuda(e);
-    if ((e = up(ri.in_off, (const void**)&rt.in_off)) != cudaSuccess) return map_cuda(e);
-    if ((e = up(ri.pairs, (const void**)&rt.pairs)) != cudaSuccess) return map_cuda(e);
-    if ((e = up(ri.out_ranks, (const void**)&rt.out_ranks)) != cudaSuccess) return map_cuda(e);
+    if ((e = ts.upload(ri.pos_in, &rt.pos_in)) != cudaSuccess ||
+        (e = ts.upload(ri.hdr, &rt.hdr)) != cudaSuccess ||
+        (e = ts.upload(ri.in_off, &rt.in_off)) != cudaSuccess ||
+        (e = ts.upload(ri.pairs, &rt.pairs)) != cudaSuccess ||
+        (e = ts.upload(ri.out_ranks, &rt.out_ranks)) != cudaSuccess)
+      return map_cuda(e);
   }
   // squaring units up to the largest degree asked for, or what shared memory
   // holds
@@ -275,47 +265,37 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
     if (!build_square_table(n, D, im)) return BERN_E_UNSUPPORTED;
     // units first: they are read as int4
     const size_t wu = im.units.size(), wp = im.pos.size(), ww = im.words.size();
-    DevBuf b;
-    if ((e = b.reserve((wu + wp + ww + im.ranks.size() + 4) * sizeof(int32_t))) != cudaSuccess)
-      return map_cuda(e);
-    ts.bufs.push_back(b);
-    int32_t* d = (int32_t*)b.p;
-    cudaMemcpy(d, im.units.data(), wu * sizeof(int32_t), cudaMemcpyHostToDevice);
-    cudaMemcpy(d + wu, im.pos.data(), wp * sizeof(int32_t), cudaMemcpyHostToDevice);
-    cudaMemcpy(d + wu + wp, im.words.data(), ww * sizeof(int32_t), cudaMemcpyHostToDevice);
-    cudaMemcpy(d + wu + wp + ww, im.ranks.data(), im.ranks.size() * sizeof(int32_t),
-               cudaMemcpyHostToDevice);
+    std::vector<int32_t> img(im.units);
+    img.insert(img.end(), im.pos.begin(), im.pos.end());
+    img.insert(img.end(), im.words.begin(), im.words.end());
+    img.insert(img.end(), im.ranks.begin(), im.ranks.end());
+    const int32_t* d;
+    if ((e = ts.upload(img, &d)) != cudaSuccess) return map_cuda(e);
     ts.view.sqt[D] = SquareTable{im.m_pad, im.n_units, d + wu, (const int4*)d,
                                  (const uint32_t*)(d + wu + wp), d + wu + wp + ww};
   }
   for (int D = 0; D <= dmax; ++D) {
     PairList pl;
     if (!build_square_pairs(n, D, pl)) return BERN_E_UNSUPPORTED;
-    DevBuf bp, bq;
-    if ((e = bp.reserve(pl.ptr.size() * sizeof(int32_t))) != cudaSuccess) return map_cuda(e);
-    if ((e = bq.reserve(std::max<size_t>(4, pl.pairs.size() * sizeof(uint32_t)))) != cudaSuccess)
+    if ((e = ts.upload(pl.ptr, &ts.view.sq[D].ptr)) != cudaSuccess ||
+        (e = ts.upload(pl.pairs, &ts.view.sq[D].pairs)) != cudaSuccess)
       return map_cuda(e);
-    cudaMemcpy(bp.p, pl.ptr.data(), pl.ptr.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-    if (!pl.pairs.empty())
-      cudaMemcpy(bq.p, pl.pairs.data(), pl.pairs.size() * sizeof(uint32_t),
-                 cudaMemcpyHostToDevice);
-    ts.view.sq[D].ptr = (const int32_t*)bp.p;
-    ts.view.sq[D].pairs = (const uint32_t*)bq.p;
-    ts.bufs.push_back(bp);
-    ts.bufs.push_back(bq);
   }
   if (!ts.prod_arr.p) {
     ts.prod_host.assign((size_t)kProdStride * kProdStride, ProdTable{nullptr, nullptr});
     if ((e = ts.prod_arr.reserve(ts.prod_host.size() * sizeof(ProdTable))) != cudaSuccess)
       return map_cuda(e);
-    cudaMemcpy(ts.prod_arr.p, ts.prod_host.data(), ts.prod_host.size() * sizeof(ProdTable),
-               cudaMemcpyHostToDevice);
+    e = copy_in(ts.prod_arr.p, ts.prod_host.data(), ts.prod_host.size() * sizeof(ProdTable));
+    if (e != cudaSuccess) {
+      ts.prod_arr.release();
+      return map_cuda(e);
+    }
   }
   ts.view.prod = (const ProdTable*)ts.prod_arr.p;
-  ts.dmax = dmax;
-  ts.view.dmax = dmax;
   e = cudaGetLastError();
   if (e != cudaSuccess) return map_cuda(e);
+  ts.dmax = dmax;
+  ts.view.dmax = dmax;
   *out = &ts.view;
   return BERN_OK;
 }
@@ -334,9 +314,8 @@ int ensure_prod_tables(bern_ctx* c, int n, int Dmax, int dmax, int cap) {
   std::vector<std::pair<int, int>> added;
   auto finish = [&](int rc_in) -> int {
     if (added.empty()) return rc_in;
-    const cudaError_t e = cudaMemcpy(ts.prod_arr.p, ts.prod_host.data(),
-                                     ts.prod_host.size() * sizeof(ProdTable),
-                                     cudaMemcpyHostToDevice);
+    const cudaError_t e = copy_in(ts.prod_arr.p, ts.prod_host.data(),
+                                  ts.prod_host.size() * sizeof(ProdTable));
     if (e == cudaSuccess) return rc_in;
     for (const auto& key : added) {
       ts.prod_host[(size_t)key.first * kProdStride + key.second] = ProdTable{nullptr, nullptr};
@@ -359,14 +338,15 @@ int ensure_prod_tables(bern_ctx* c, int n, int Dmax, int dmax, int cap) {
       DevBuf bp, bq;
       cudaError_t e = bp.reserve(ptr.size() * sizeof(int32_t));
       if (e == cudaSuccess) e = bq.reserve(std::max<size_t>(8, pairs.size() * sizeof(int32_t)));
+      if (e == cudaSuccess)
+        e = copy_in(bp.p, ptr.data(), ptr.size() * sizeof(int32_t));
+      if (e == cudaSuccess && !pairs.empty())
+        e = copy_in(bq.p, pairs.data(), pairs.size() * sizeof(int32_t));
       if (e != cudaSuccess) {
         bp.release();
         bq.release();
         return finish(map_cuda(e));
       }
-      cudaMemcpy(bp.p, ptr.data(), ptr.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-      if (!pairs.empty())
-        cudaMemcpy(bq.p, pairs.data(), pairs.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
       ts.prod[key] = std::make_pair(bp, bq);
       ts.prod_host[(size_t)Dq * kProdStride + D] = ProdTable{(const int32_t*)bp.p, (const int2*)bq.p};
       added.push_back(key);
@@ -388,7 +368,6 @@ cudaError_t ensure_square_scratch(bern_ctx* c, size_t bytes, size_t group) {
   for (size_t want = bytes;; want = std::max(group, want / 2)) {
     const cudaError_t e = b.reserve(want);
     if (e != cudaErrorMemoryAllocation) return e;
-    cudaGetLastError();             // not this call's error
     if (want == group) return cudaSuccess;
   }
 }
@@ -877,8 +856,6 @@ int bern_destroy(bern_ctx* c) {
   for (auto& g : c->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   for (auto& kv : c->tables) {
-    kv.second.exps.release();
-    kv.second.mcount.release();
     for (auto& b : kv.second.bufs) b.release();
     for (auto& p : kv.second.prod) {
       p.second.first.release();

@@ -13,6 +13,7 @@ struct Dim3 { unsigned x, y, z; };
 namespace {
 size_t alloc_limit = (size_t)-1;
 long copies_left = -1;               // -1: all copies succeed
+int copies = 0;
 int last_error = 0;
 std::map<const void*, std::string> names;
 std::string launched;                // one name per line
@@ -24,6 +25,7 @@ int fail(int e) { return last_error = e; }
 extern "C" {
 void host_set_alloc_limit(size_t bytes) { alloc_limit = bytes; }
 void host_fail_copies_after(long n) { copies_left = n; }
+int host_count_copies() { int n = copies; copies = 0; return n; }
 const char* host_launched() { return launched.c_str(); }
 const char* host_allocated() { return allocated.c_str(); }
 void host_clear() { launched.clear(), allocated.clear(); }
@@ -39,6 +41,7 @@ int cudaMemGetInfo(size_t* f, size_t* t) { *f = *t = (size_t)1 << 30; return 0; 
 int cudaMemcpy(void* d, const void* s, size_t n, int) {
   if (copies_left == 0) return fail(kUnknown);
   if (copies_left > 0) --copies_left;
+  ++copies;
   std::memcpy(d, s, n);
   return 0;
 }

@@ -60,3 +60,36 @@ scratch, = sizes_of(2, False)
 assert scratch in sizes_of(3, True)
 assert scratch not in sizes_of(3, False)
 """)
+
+
+def test_tables_whose_copy_failed_are_built_again(tmp_path):
+    """A copy of a table to the device fails, the first, the last or any between: the
+    call says so, and the next one does not run on what is there."""
+    run(tmp_path, COMPOSE + """
+def tries(n, D, d):
+    h = context()
+    rt.host_count_copies()
+    rc, k = compose(h, n, D, 1, 3, d=d)
+    total = rt.host_count_copies()
+    assert rc == 0 and total > 10
+    lib.bern_destroy(h)
+    for left in sorted({0, 1, total // 3, total // 2, total - 2, total - 1}):
+        h = context()
+        launched()
+        rt.host_fail_copies_after(left)
+        rc, k = compose(h, n, D, 1, 3, d=d)
+        assert rc != 0 and not k, (left, rc, k)
+        rt.host_fail_copies_after(-1)
+        first = rt.host_count_copies()
+        rc, k = compose(h, n, D, 1, 3, d=d)
+        assert rc == 0 and k, (left, rc, k)
+        # what a failed build had copied is copied again; the product tables of order
+        # 3 that were complete stay
+        again = rt.host_count_copies()
+        assert again >= total - 1 if d == 2 else first + again >= total, (left, total, first, again)
+        rc, k = compose(h, n, D, 1, 3, d=d)
+        assert rc == 0 and rt.host_count_copies() == 0
+        lib.bern_destroy(h)
+tries(4, 2, 2)
+tries(2, 2, 3)
+""")
