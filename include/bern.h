@@ -413,8 +413,8 @@ int bern_enclose(bern_ctx* ctx, int n, int64_t n_boxes, int h, int order,
 /* Lin step, Sec. 5.3 (parameter Lin): for every neuron of a post-activation
  * block, the least-squares multilinear fit A of each bound on [0,1]^n is
  * written to lin_up / lin_lo (a layer block with stride lin_ld >=
- * M(n, min(n, order)); term counts lin_nterms = min(nterms, that)), the
- * residual post - A (rounded up for the upper bound, down for the lower)
+ * M(n, min(n, order)); term counts lin_nterms = min(nterms, that); A's terms
+ * past them are left out), the residual post - A (rounded up for the upper bound, down for the lower)
  * OVERWRITES post_up / post_lo, its Bernstein enclosure of order `order`
  * goes to res_lo (min over the lower residual) and res_hi (max over the
  * upper one), and A's constant is shifted by it outward: lin_up >= post_up

@@ -15,7 +15,8 @@
 //   a_T = 2^|T| sum_{S contains T} (-1)^(|S|-|T|) c_S.
 // c_S is exactly 0 unless some term contains every variable of S (a factor
 // e_k = 0 in its weight vanishes otherwise), so the fit of a degree-D
-// polynomial has degree <= min(n, D).
+// polynomial has degree <= min(n, D).  Below the order min(n, D) the fit block holds
+// the terms of A up to that order only; the others stay in the residual.
 //
 // Soundness does not depend on the fit: A enters the bound exactly as stored
 // (float32).  The residual coefficients are rounded up (upper) or down
@@ -129,10 +130,10 @@ k_lin_project_thread(Tables T, int64_t n_items, int h, int64_t mlin, int mw,
         if ((S & Tm) == Tm) a += (__popc(S ^ Tm) & 1) ? -c[S] : c[S];
       a *= (float)(1 << __popc(Tm));
       const int r = s_rank[Tm];
-      if (r < nt) {
+      if (r < ntl) {                       // terms the fit block does not hold stay in P
         const float p = P[(int64_t)r * h];
         P[(int64_t)r * h] = up ? __fsub_ru(p, a) : __fsub_rd(p, a);
-        if (r < ntl) A[(int64_t)r * h] = a;
+        A[(int64_t)r * h] = a;
       }
     }
     if (up) lin_nt[item] = ntl;
@@ -199,7 +200,7 @@ k_lin_project(Tables T, int64_t n_items, int h, int64_t mlin, float* __restrict_
     sa[Tm] = a * (float)(1 << __popc(Tm));
   }
   __syncwarp();
-  for (int r = lane; r < nt; r += 32) {
+  for (int r = lane; r < ntl; r += 32) {   // terms the fit block does not hold stay in P
     const uint8_t* e = T.exps + (int64_t)r * n;
     bool ml = true;
     int mask = 0;
@@ -212,7 +213,7 @@ k_lin_project(Tables T, int64_t n_items, int h, int64_t mlin, float* __restrict_
       const float p = P[(int64_t)r * h];
       P[(int64_t)r * h] = up ? __fsub_ru(p, a) : __fsub_rd(p, a);
     }
-    if (r < ntl) A[(int64_t)r * h] = a;
+    A[(int64_t)r * h] = a;
   }
   if (up && lane == 0) lin_nt[item] = ntl;
 }
