@@ -274,6 +274,7 @@ int ensure_tables(bern_ctx* c, int n, int dmax, const Tables** out) {
     ts.view.sqt[D] = SquareTable{im.m_pad, im.n_units, d + wu, (const int4*)d,
                                  (const uint32_t*)(d + wu + wp), d + wu + wp + ww};
   }
+  // pair lists of every degree: the squares without a scratch take them too
   for (int D = 0; D <= dmax; ++D) {
     PairList pl;
     if (!build_square_pairs(n, D, pl)) return BERN_E_UNSUPPORTED;

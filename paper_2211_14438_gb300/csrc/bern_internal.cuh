@@ -198,7 +198,7 @@ void build_rscale(int n, int l, std::vector<float>& out);
 void build_enclose_tables(int n, int l, std::vector<int32_t>& gidx, std::vector<int32_t>& lines,
                           bool with_lines = true);
 // Host images of the slab enclosure's tables for (n, l), n >= 4: pos, and
-// off[m] (m = 4..n) and wt[m] (m = 3..n-1).
+// off[m] (m = 4..n) and wt[m] (m = 4..n-1).
 void build_lex_tables(int n, int l, std::vector<uint32_t>& pos,
                       std::vector<std::vector<int32_t>>& off, std::vector<std::vector<float>>& wt);
 

@@ -324,7 +324,6 @@ cudaError_t launch_lb(const Launch& L, const Tables& T, int G, int64_t n_items, 
 // Tiny grids (order 0: one cell): one lane per polynomial, the lane's grid
 // interleaved with its warp's (element g of lane L at grid[g*32 + L]); a warp
 // takes 32 items of one bound, a block 4 groups of 32 items (both bounds).
-constexpr int kSmallGrid = 64;
 template <int LB, bool UP>
 __device__ float enclose_lane(const float* __restrict__ P, int ps, int nt, int n,
                               const Tables& T, const float2* __restrict__ rs, float* grid) {

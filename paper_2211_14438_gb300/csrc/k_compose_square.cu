@@ -22,8 +22,9 @@
 // scaling), the diagonal pair s by s once, everything rounds up.
 //
 // s lies in shared memory (32 lanes x M pairs) up to kSquareSmemTerms terms; for
-// longer inputs a first kernel writes it to a scratch [M][32] per group, which
-// the L2 holds, and the units of a group are spread over blocks.
+// longer inputs a first kernel writes it to a scratch [M][32] per group (1 MB with
+// 3003 terms, up to 512 MB of groups in a pass; some hundred of them stay in the L2),
+// and the units of a group are spread over blocks.
 //
 // Bound: instruction issue (n = 6, D = 4: 22,155 products, 2,575 tile or row
 // pairs and 3,003 outputs of both bounds per group; 52% of the issue slots, ALU the
@@ -216,12 +217,13 @@ __device__ __forceinline__ p2 put(const SquareOut& o, p2 sq, p2 lin, int K, p2& 
 }
 
 // A unit's header with the first 32 words of its pairs and its output ranks (at
-// most 28 of a tile, 17 of a row), one per lane.
+// most 21 of a tile, 17 of a row), one per lane.
 struct UnitHead {
   int4 un;
   uint32_t words;
   int32_t rank;
 };
+static_assert(kTileDegree == 5, "the tiles of square_unit");
 static_assert(tri_size(kTileDegree) <= 32 && 2 * kRowLen - 1 <= 32, "a lane per output");
 __device__ __forceinline__ UnitHead unit_head(const SquareTable& R, int4 un) {
   const int lane = threadIdx.x & 31;
@@ -272,8 +274,6 @@ __device__ __forceinline__ p2 tile_unit(const SquareTable& R, const UnitHead& hd
         tile_run<E, (E >= 2 ? 1 : 0)>(s, mine, m, k, w, acc);
       else if (E >= 4 && d1 == 2)
         tile_run<E, (E >= 4 ? 2 : 0)>(s, mine, m, k, w, acc);
-      else if (E >= 6 && d1 == 3)
-        tile_run<E, (E >= 6 ? 3 : 0)>(s, mine, m, k, w, acc);
     }
     if (k0 + 32 < un.y) mine = next;         // the diagonal's word may be the next chunk's first
   }
@@ -320,7 +320,6 @@ __device__ __forceinline__ p2 square_unit(const SquareTable& R, const UnitHead& 
       case 3: return tile_unit<3, TRUNC>(R, hd, s, out, rem);
       case 4: return tile_unit<4, TRUNC>(R, hd, s, out, rem);
       case 5: return tile_unit<5, TRUNC>(R, hd, s, out, rem);
-      case 6: if constexpr (kTileDegree >= 6) return tile_unit<6, TRUNC>(R, hd, s, out, rem);
       default: break;
     }
   } else {

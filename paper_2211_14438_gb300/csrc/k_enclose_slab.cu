@@ -17,7 +17,8 @@
 //   c_0 + sum_J max(0, w_J c_J),   w_J = prod_k C(l, j_k),
 // and no computed one exceeds that by more than delta sum_J |w_J c_J|, where
 // delta covers the roundings of the m remaining passes (m l additions, each of
-// at most 2^-23 of a partial sum that sum |w c| bounds) four times over.  A
+// at most 2^-23 of a partial sum that sum |w c| bounds) twice over, and four times
+// where a coefficient is positive.  A
 // slab whose bound is not above the largest coefficient found so far adds
 // nothing to the maximum.  The search starts from the value at the vertex that
 // the linear terms point to (summed rounding down, so it is not above the
@@ -130,7 +131,7 @@ __device__ __forceinline__ void slab_row(const p2* __restrict__ src, int len, p2
 }
 
 template <int LB, int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? (LB >= 9 ? 1 : 2) : (NT == 128 ? 5 : (NT == 64 ? 12 : 24)))
+__global__ void __launch_bounds__(NT, NT == 256 ? (LB >= 9 ? 1 : 2) : (NT == 128 ? 5 : 12))
 k_enclose_slab(Tables T, LexView X, SlabShape sh, const float2* __restrict__ rs, int64_t n_items,
                int h, const float* __restrict__ pre_up, const float* __restrict__ pre_lo,
                int64_t ld, const int32_t* __restrict__ nterms, float* __restrict__ lo,
@@ -340,7 +341,7 @@ cudaError_t launch_slab(const Launch& L, const Tables& T, const LexView& X, int6
     if (e != cudaSuccess) return e;
   }
   const int by_smem = (int)((226 * 1024) / (smem + 3072));
-  const int per_sm = std::max(1, std::min(NT == 256 ? 2 : (NT == 128 ? 5 : (NT == 64 ? 12 : 24)), by_smem));
+  const int per_sm = std::max(1, std::min(NT == 256 ? 2 : (NT == 128 ? 5 : 12), by_smem));
   const int64_t blocks = std::min<int64_t>((int64_t)device_sms(L) * per_sm, n_items);
   kern<<<(unsigned)blocks, NT, smem, L.stream>>>(T, X, sh, T.rscale[LB], n_items, h, pre_up,
                                                  pre_lo, ld, nterms, lo, hi, list, count,
@@ -753,13 +754,14 @@ cudaError_t launch_expand(const Launch& L, const Tables& T, const LexView& X, co
 }  // namespace
 
 #define BERN_SLAB_CASES                                                                       \
-  BERN_SLAB(2, 32) BERN_SLAB(3, 32) BERN_SLAB(4, 64) BERN_SLAB(5, 128) BERN_SLAB(6, 256)      \
-  BERN_SLAB(7, 256) BERN_SLAB(8, 256) BERN_SLAB(9, 256)
+  BERN_SLAB(4, 64) BERN_SLAB(5, 128) BERN_SLAB(6, 256) BERN_SLAB(7, 256) BERN_SLAB(8, 256)    \
+  BERN_SLAB(9, 256)
 
 bool enclose_slab_ok(const Tables& T, int lb) {
   if (!T.lex || T.n < 4 || lb < 2 || lb > kSlabMaxOrder || !T.lex[lb].pos) return false;
   SlabShape sh;
   switch (lb) {
+    case 2: case 3: return true;   // registers, or the expansion
 #define BERN_SLAB(X, NT) case X: return shape_of<X, NT>(T.n, &sh);
     BERN_SLAB_CASES
 #undef BERN_SLAB
@@ -787,7 +789,7 @@ cudaError_t launch_enclose_slab(const Launch& L, const Tables& T, int lb, int64_
       return launch_expand<X, NT>(L, T, T.lex[X], es, n_items, h, pre_up, pre_lo, ld, nterms,  \
                                   lo, hi, list, count);                                        \
   }
-  BERN_EXPAND(2, 128) BERN_EXPAND(3, 128) BERN_EXPAND(4, 128) BERN_EXPAND(5, 128)
+  BERN_EXPAND(3, 128) BERN_EXPAND(4, 128) BERN_EXPAND(5, 128)
   BERN_EXPAND(6, 256) BERN_EXPAND(7, 256) BERN_EXPAND(8, 256)
 #undef BERN_EXPAND
   switch (lb) {

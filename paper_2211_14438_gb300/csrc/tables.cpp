@@ -533,7 +533,7 @@ void build_lex_tables(int n, int l, std::vector<uint32_t>& pos,
   binom[0] = 1.0;
   for (int j = 1; j <= l; ++j) binom[j] = binom[j - 1] * (l - j + 1) / j;
   std::map<uint64_t, uint32_t> at;
-  for (int m = 3; m <= n; ++m) {
+  for (int m = 4; m <= n; ++m) {
     std::vector<uint8_t> ex;
     lex_monomials(m, l, ex);
     const size_t rows = ex.size() / m;
@@ -546,14 +546,14 @@ void build_lex_tables(int n, int l, std::vector<uint32_t>& pos,
         if ((double)f < w) f = std::nextafterf(f, INFINITY);
         wt[m].push_back(f);
       }
-      if (m >= 4 && e[m - 1] == 0) off[m].push_back((int32_t)r);
+      if (e[m - 1] == 0) off[m].push_back((int32_t)r);
       if (m == n) {
         uint32_t mask = 0;
         for (int k = 0; k < n; ++k) mask |= (e[k] ? 1u : 0u) << k;
         at[pack_key(e, n)] = (uint32_t)r | mask << 24;
       }
     }
-    if (m >= 4) off[m].push_back((int32_t)rows);
+    off[m].push_back((int32_t)rows);
   }
   std::vector<uint8_t> ex;
   graded_monomials(n, l, ex);
