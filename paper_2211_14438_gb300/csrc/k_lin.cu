@@ -120,6 +120,13 @@ k_lin_project_thread(Tables T, int64_t n_items, int h, int64_t mlin, int mw,
     }
 #pragma unroll
     for (int S = 0; S < NS; ++S) c[S] = (c[S] + q[0][S]) + (q[1][S] + q[2][S]);
+    // terms the fit block does not hold stay in P; all loads before the first store
+    float p[NS];
+#pragma unroll
+    for (int Tm = 0; Tm < NS; ++Tm) {
+      const int r = s_rank[Tm];
+      p[Tm] = r < ntl ? P[(int64_t)r * h] : 0.0f;
+    }
     for (int r = 0; r < ntl; ++r) A[(int64_t)r * h] = 0.0f;
     // power-basis coefficients a_T from the supersets S of T
 #pragma unroll
@@ -130,9 +137,8 @@ k_lin_project_thread(Tables T, int64_t n_items, int h, int64_t mlin, int mw,
         if ((S & Tm) == Tm) a += (__popc(S ^ Tm) & 1) ? -c[S] : c[S];
       a *= (float)(1 << __popc(Tm));
       const int r = s_rank[Tm];
-      if (r < ntl) {                       // terms the fit block does not hold stay in P
-        const float p = P[(int64_t)r * h];
-        P[(int64_t)r * h] = up ? __fsub_ru(p, a) : __fsub_rd(p, a);
+      if (r < ntl) {
+        P[(int64_t)r * h] = up ? __fsub_ru(p[Tm], a) : __fsub_rd(p[Tm], a);
         A[(int64_t)r * h] = a;
       }
     }
