@@ -35,8 +35,8 @@ namespace bern {
 // queue is a list of sorted runs, and a warp's 32 consecutive entries are mostly
 // neighbouring neurons of one box.
 __global__ void __launch_bounds__(kQueueThreads)
-k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int sq_dmax, ComposeScratch S,
-                int* status) {
+k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int sq_smem, int sq_dmax,
+                ComposeScratch S, int* status) {
   const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int q = -1;
   if (item < n_items) {
@@ -67,8 +67,9 @@ k_compose_queue(Tables T, ComposeArgs A, int64_t n_items, int sq_dmax, ComposeSc
         } else if (d == 1) {
           q = kQLinear;
           nt = Mout;
-        } else if (D <= sq_dmax) {
-          q = D;
+        } else if (D <= sq_smem ||
+                   (D <= sq_dmax && !(A.coef[item * kCoefStride + 2] < 0.0f))) {
+          q = D;   // past shared memory, a caller's concave polynomial takes the pair lists
           nt = Mout;
         } else if (D <= T.dmax) {
           q = kQPairs;
@@ -335,13 +336,14 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
          num_monomials(T.n, Dmax + 1) <= pre_cap)
     ++Dmax;
   // long inputs take the squaring kernels where the caller gave them a scratch
-  const int sq_dmax = std::min(std::min(T.sqt_dmax, Dmax),
-                               S.tws ? square_max_degree(T.n) : square_smem_degree(T.n));
+  const int sq_smem = std::min(std::min(T.sqt_dmax, Dmax), square_smem_degree(T.n));
+  const int sq_dmax =
+      S.tws ? std::min(std::min(T.sqt_dmax, Dmax), square_max_degree(T.n)) : sq_smem;
   cudaError_t e = cudaMemsetAsync(S.qcount, 0, kComposeQueues * sizeof(int), L.stream);
   if (e != cudaSuccess) return e;
   k_compose_queue<<<(unsigned)((n_items + kQueueThreads - 1) / kQueueThreads), kQueueThreads, 0,
                     L.stream>>>(
-      T, A, n_items, sq_dmax, S, L.status);
+      T, A, n_items, sq_smem, sq_dmax, S, L.status);
   ++*L.launches;
   // order-2 items exist only with order 2 somewhere in the plan (with pruning
   // they go to the Horner kernel)
@@ -362,8 +364,9 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
                        0, L.stream>>>(A, S, 32 * device_sms(L), L.status);
     ++*L.launches;
   }
-  // pair-list kernel for order-2 items beyond the squaring kernels
-  if (order2 && Dmax > sq_dmax) {
+  // pair-list kernel for order-2 items beyond the squaring kernels, and for concave
+  // ones beyond those in shared memory
+  if (order2 && Dmax > sq_smem) {
     const size_t psmem = 2 * (size_t)pre_cap * sizeof(float);
     if (psmem > 200 * 1024) return cudaErrorInvalidValue;
     if (psmem > 48 * 1024) {

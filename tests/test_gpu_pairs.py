@@ -93,3 +93,18 @@ def test_long_squares_in_several_passes(n, D, cap):
     assert parts[3] > whole[3]
     for a, b in zip(parts[:3], whole[:3]):
         assert np.array_equal(a, b)
+
+
+def test_concave_polynomials_of_long_inputs():
+    """A caller's coefficients with a_2 < 0: past shared memory such items take the
+    pair lists, their neighbours the squares by tiles, both as without a scratch."""
+    n, D, B, h = 5, 8, 2, 40
+    p = _problem(n, D, B, h, 16)
+    convex = _run(n, D, B, h, 16, p)                  # raises where an item is refused
+    p["coef"][:, ::4, 2] *= -1.0
+    got, lists = _run(n, D, B, h, 16, p), _run(n, D, B, h, 16, p, 0)
+    for a, b, c in zip(got[:2], lists[:2], convex[:2]):
+        assert np.array_equal(a[..., ::4], b[..., ::4])
+        keep = np.arange(h) % 4 != 0
+        assert np.array_equal(a[..., keep], c[..., keep])
+        assert not np.array_equal(a[..., ::4], c[..., ::4])
