@@ -473,24 +473,34 @@ __device__ __forceinline__ int find_group(const ComposeScratch& S, int dlo, int 
   return -1;
 }
 
-// Inputs in shared memory.  WPG = kSquareWarps: a block per group, half of its
-// warps loading each bound, all taking the units in turn.  WPG = 1: a warp per
-// group, without block barriers, for short inputs of many groups.
+// Inputs in shared memory, WPG warps to a group: they share the loads and then the
+// units in turn.  A block per group for long inputs or few groups, fewer warps for
+// short inputs of many groups (down to one, without barriers).
 constexpr int kSquareWarps = 8;
 constexpr int kSquareBlocks = 2;
 constexpr int kLoadParts = 4;                // partial sums of |s| (as the fused layer's)
 
 template <int WPG>
+__device__ __forceinline__ void group_sync(int group) {
+  if constexpr (WPG == kSquareWarps)
+    __syncthreads();
+  else if constexpr (WPG > 1)
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(32 * WPG) : "memory");
+  else
+    __syncwarp();
+}
+
+template <int WPG>
 __global__ void __launch_bounds__(32 * kSquareWarps, kSquareBlocks)
 k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstride, int* status) {
-  static_assert(WPG == 1 || WPG == 2 * kLoadParts, "a warp per group, or one per bound and part");
+  static_assert(2 * kLoadParts % WPG == 0, "the loads of both bounds over the warps of a group");
   constexpr int GPB = kSquareWarps / WPG;    // groups of a block
   extern __shared__ __align__(16) p2 smem2[];
-  __shared__ float s_l1[2][kLoadParts][32];
-  __shared__ p2 s_rem[kSquareWarps][32], s_c0[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = warp % WPG;
-  p2* mine = smem2 + (size_t)(32 * (warp / WPG) + lane) * sstride;
-  for (int task = blockIdx.x * GPB + warp / WPG;; task += gridDim.x * GPB) {
+  __shared__ float s_l1[WPG > 1 ? GPB : 1][2][kLoadParts][32];
+  __shared__ p2 s_rem[kSquareWarps][32], s_c0[GPB][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = warp % WPG, g = warp / WPG;
+  p2* mine = smem2 + (size_t)(32 * g + lane) * sstride;
+  for (int task = blockIdx.x * GPB + g;; task += gridDim.x * GPB) {
     int group = task;
     const int D = find_group(S, dlo, dhi, group);
     if (D < 0) break;
@@ -498,10 +508,12 @@ k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstrid
     const SquareItem it = square_item(A, S, D, group * 32 + lane, status);
     p2 l1 = 0ull;
     if constexpr (WPG > 1) {
-      const int up = w / kLoadParts, part = w - up * kLoadParts;
-      s_l1[up][part][lane] = load_s(A, R, it, up ? A.pre_up : A.pre_lo, part, kLoadParts,
-                                    reinterpret_cast<float*>(mine) + up, 1);
-      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < 2 * kLoadParts / WPG; ++i) {
+        const int k = w + i * WPG, up = k / kLoadParts, part = k - up * kLoadParts;
+        s_l1[g][up][part][lane] = load_s(A, R, it, up ? A.pre_up : A.pre_lo, part, kLoadParts,
+                                         reinterpret_cast<float*>(mine) + up, 1);
+      }
     } else {
 #pragma unroll
       for (int part = 0; part < kLoadParts; ++part) {
@@ -511,8 +523,8 @@ k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstrid
                                reinterpret_cast<float*>(mine), 1);
         l1 = part == 0 ? pack2(l, u) : add2_ru(l1, pack2(l, u));
       }
-      __syncwarp();
     }
+    group_sync<WPG>(g);
     const SquareOut out = square_out(T, A, it, D);
     p2 rem = 0ull, c0 = 0ull;
     if (2 * D <= A.cap)
@@ -521,22 +533,21 @@ k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstrid
       square_units<true>(R, w, WPG, SmemRow{mine}, out, rem, c0);
     if constexpr (WPG > 1) {
       s_rem[warp][lane] = rem;
-      if (warp == 0) s_c0[lane] = c0;        // unit 0 holds the constant
-      __syncthreads();
-      if (warp == 0) {
-        l1 = pack2(s_l1[0][0][lane], s_l1[1][0][lane]);
+      if (w == 0) s_c0[g][lane] = c0;        // unit 0 holds the constant
+      group_sync<WPG>(g);
+      if (w == 0) {
+        l1 = pack2(s_l1[g][0][0][lane], s_l1[g][1][0][lane]);
 #pragma unroll
         for (int i = 1; i < kLoadParts; ++i)
-          l1 = add2_ru(l1, pack2(s_l1[0][i][lane], s_l1[1][i][lane]));
+          l1 = add2_ru(l1, pack2(s_l1[g][0][i][lane], s_l1[g][1][i][lane]));
 #pragma unroll
-        for (int i = 1; i < kSquareWarps; ++i) rem = add2_ru(rem, s_rem[i][lane]);
-        if (it.valid) put_constant(A, it, out, s_c0[lane], l1, rem, status);
+        for (int i = 1; i < WPG; ++i) rem = add2_ru(rem, s_rem[warp + i][lane]);
+        if (it.valid) put_constant(A, it, out, s_c0[g][lane], l1, rem, status);
       }
-      __syncthreads();                       // the next task reuses the shared inputs
     } else {
       if (it.valid) put_constant(A, it, out, c0, l1, rem, status);
-      __syncwarp();
     }
+    group_sync<WPG>(g);                      // the next task reuses the shared inputs
   }
 }
 
@@ -552,6 +563,7 @@ k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstrid
 // together (100 groups, n = 6, D = 8: 7.1 ms, 6.9 with 8 tasks, 6.4 with 16 and
 // 6.3 with 32, whose remainders cost that again).
 constexpr int kSquareWarpTerms = 32;         // padded terms of a warp per group
+constexpr int kSquarePairTerms = 50;         // of two warps per group
 constexpr int kSquareChunks = 16;
 constexpr int kUnitWarps = 16;                // one block per multiprocessor
 constexpr int kSquareParts = kSquareChunks * kUnitWarps;
@@ -661,10 +673,19 @@ cudaError_t launch_compose_square(const Launch& L, const Tables& T, const Compos
   const int dmx = std::min(std::min(Dmax, T.sqt_dmax), square_max_degree(T.n));
   // A warp per group where every input of the layer is short and there is a group
   // for every resident warp: order 2 on degree 2 in three variables, 327,680
-  // items, 41 us with a block per group, 26 us; from degree 4 in three variables
-  // on (44 padded terms) the block is faster, 149 against 169 us.
-  const bool warps = square_padded_terms(T.n, dsm) <= kSquareWarpTerms &&
-                     n_items >= (int64_t)32 * kSquareWarps * kSquareBlocks * device_sms(L);
+  // items, 41 us with a block per group, 26 us.
+  const int pad = square_padded_terms(T.n, dsm);
+  const int64_t resident = (int64_t)32 * kSquareWarps * kSquareBlocks * device_sms(L);
+  const bool one = pad <= kSquareWarpTerms && n_items >= resident;
+  // Two warps for inputs about as long (degrees 7 and 8 in two variables, 4 in three),
+  // whose 13 to 17 units eight warps share badly: degree 8 in two variables, 327,680
+  // items of which 1/5, 1/2 and all are squared in place, 8 / 4 / 2 / 1 warps a group
+  // (us): 151 / 146 / 149 / 168, 220 / 193 / 184 / 199, 347 / 278 / 237 / 238.  From
+  // seven eighths of the resident warps on (70,400 items, all: 83 / - / 64; 44,800,
+  // 1/3: 33 / 30 / 40), and where the cap keeps all outputs: the sum over the
+  // others has a part per warp.
+  const bool two = pad > kSquareWarpTerms && pad <= kSquarePairTerms &&
+                   2 * dsm <= A.cap && n_items >= resident / 8 * 7;
   auto launch = [&](auto kern, int wpg, int dlo, int dhi) -> cudaError_t {
     // the per-lane stride is an odd number of 16-byte units, so that lanes
     // reading the same position hit distinct banks
@@ -681,7 +702,8 @@ cudaError_t launch_compose_square(const Launch& L, const Tables& T, const Compos
     ++*L.launches;
     return cudaGetLastError();
   };
-  const cudaError_t e = warps ? launch(k_square<1>, 1, 0, dsm)
+  const cudaError_t e = one   ? launch(k_square<1>, 1, 0, dsm)
+                        : two ? launch(k_square<2>, 2, 0, dsm)
                               : launch(k_square<kSquareWarps>, kSquareWarps, 0, dsm);
   if (e != cudaSuccess) return e;
   if (dmx > dsm && S.tws) {
