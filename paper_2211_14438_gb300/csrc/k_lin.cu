@@ -206,9 +206,9 @@ k_lin_project(Tables T, int64_t n_items, int h, int64_t mlin, float* __restrict_
     sa[Tm] = a * (float)(1 << __popc(Tm));
   }
   __syncwarp();
-  for (int r = lane; r < ntl; r += 32) {   // terms the fit block does not hold stay in P
+  for (int r = lane; r < nt; r += 32) {
     const uint8_t* e = T.exps + (int64_t)r * n;
-    bool ml = true;
+    bool ml = r < ntl;                     // terms the fit block does not hold stay in P
     int mask = 0;
     for (int k = 0; k < n; ++k) {
       if (e[k] > 1) ml = false;
@@ -219,7 +219,7 @@ k_lin_project(Tables T, int64_t n_items, int h, int64_t mlin, float* __restrict_
       const float p = P[(int64_t)r * h];
       P[(int64_t)r * h] = up ? __fsub_ru(p, a) : __fsub_rd(p, a);
     }
-    A[(int64_t)r * h] = a;
+    if (r < ntl) A[(int64_t)r * h] = a;
   }
   if (up && lane == 0) lin_nt[item] = ntl;
 }
