@@ -204,11 +204,14 @@ __device__ __forceinline__ void compose_linear(const ComposeArgs& A, const Compo
 
 // Eight entries a warp once that leaves each scheduler one or more warps (5120
 // boxes of [3,64x4,1] with learned orders, the four layers: 23, 29, 49 and 88 us
-// at an entry a warp, now 9, 11, 14 and 19 us), one below.
+// at an entry a warp, now 9, 11, 14 and 19 us), one below; calls of fewer
+// neurons take a kernel without the other form, whose instructions a call of 20
+// neurons waits 1 us for.
+template <bool MANY>
 __global__ void __launch_bounds__(256)
 k_compose_linear(ComposeArgs A, ComposeScratch S, int few, int* status) {
   const int n_lin = S.qcount[kQLinear];
-  if (n_lin < few)
+  if (!MANY || n_lin < few)
     compose_linear<1>(A, S, n_lin, status);
   else
     compose_linear<8>(A, S, n_lin, status);
@@ -360,8 +363,10 @@ cudaError_t launch_compose(const Launch& L, const Tables& T, const ComposeScratc
   // order-1 items exist only with order 1 somewhere in the plan (with pruning
   // they go to the Horner kernel)
   if (tau == 0.0f && (degrees != nullptr || global_d == 1)) {
-    k_compose_linear<<<(unsigned)std::min<int64_t>((n_items + 7) / 8, device_sms(L) * 16), 256,
-                       0, L.stream>>>(A, S, 32 * device_sms(L), L.status);
+    const int few = 32 * device_sms(L);
+    auto kern = n_items < few ? k_compose_linear<false> : k_compose_linear<true>;
+    kern<<<(unsigned)std::min<int64_t>((n_items + 7) / 8, device_sms(L) * 16), 256, 0, L.stream>>>(
+        A, S, few, L.status);
     ++*L.launches;
   }
   // pair-list kernel for order-2 items beyond the squaring kernels, and for concave
