@@ -564,6 +564,7 @@ k_square(Tables T, ComposeArgs A, ComposeScratch S, int dlo, int dhi, int sstrid
 // 6.3 with 32, whose remainders cost that again).
 constexpr int kSquareWarpTerms = 32;         // padded terms of a warp per group
 constexpr int kSquarePairTerms = 50;         // of two warps per group
+constexpr int kSquareFewTerms = 12;
 constexpr int kSquareChunks = 16;
 constexpr int kUnitWarps = 16;                // one block per multiprocessor
 constexpr int kSquareParts = kSquareChunks * kUnitWarps;
@@ -682,10 +683,11 @@ cudaError_t launch_compose_square(const Launch& L, const Tables& T, const Compos
   // items of which 1/5, 1/2 and all are squared in place, 8 / 4 / 2 / 1 warps a group
   // (us): 151 / 146 / 149 / 168, 220 / 193 / 184 / 199, 347 / 278 / 237 / 238.  From
   // seven eighths of the resident warps on (70,400 items, all: 83 / - / 64; 44,800,
-  // 1/3: 33 / 30 / 40), and where the cap keeps all outputs: the sum over the
-  // others has a part per warp.
-  const bool two = pad > kSquareWarpTerms && pad <= kSquarePairTerms &&
-                   2 * dsm <= A.cap && n_items >= resident / 8 * 7;
+  // 1/3: 33 / 30 / 40), inputs of a few units already from half of them on (degree 2 in
+  // two variables, 44,800 items, all: 27 / - / 17 / 15 us; 19,200, 2/5: 14.5 / - / 14.7),
+  // and where the cap keeps all outputs: the sum over the others has a part per warp.
+  const bool two = !one && pad <= kSquarePairTerms && 2 * dsm <= A.cap &&
+                   n_items >= (pad <= kSquareFewTerms ? resident / 2 : resident / 8 * 7);
   auto launch = [&](auto kern, int wpg, int dlo, int dhi) -> cudaError_t {
     // the per-lane stride is an odd number of 16-byte units, so that lanes
     // reading the same position hit distinct banks

@@ -1,5 +1,5 @@
-"""Squares of medium inputs (33 to 50 padded terms): whether two warps or a block take
-a group depends on the neurons of the call, and changes nothing."""
+"""Squares of short and medium inputs (up to 50 padded terms): whether a warp, two or a
+block take a group depends on the neurons of the call, and changes nothing."""
 import numpy as np
 import pytest
 
@@ -8,7 +8,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n,D,B,h,share", [
     (2, 7, 1100, 64, 1.0), (2, 8, 1100, 64, 1.0), (2, 8, 2600, 60, 0.3), (2, 8, 1101, 63, 0.5),
-    (3, 4, 1100, 64, 1.0), (3, 4, 1101, 63, 0.01)])
+    (3, 4, 1100, 64, 1.0), (3, 4, 1101, 63, 0.01), (2, 3, 700, 64, 1.0), (1, 1, 701, 63, 0.6),
+    (1, 8, 1400, 64, 1.0)])
 @pytest.mark.parametrize("place", [False, True])
 def test_forms_of_medium_squares(n, D, B, h, share, place):
     import torch
