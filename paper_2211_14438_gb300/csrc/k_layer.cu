@@ -11,7 +11,7 @@
 // so a post-activation polynomial never goes to HBM: the block reads the
 // layer block pre[M x h] of its box once and writes next[M' x h'] once, whole
 // 32-byte sectors at a time.  The arithmetic is that of the per-step kernels
-// (k_stable_screen, k_enclose, k_compose_rows / k_compose_linear,
+// (k_stable_screen, k_enclose, k_square / k_compose_linear,
 // k_affine_wide): every value is rounded in the same direction, in the same
 // order, except the cap-truncation remainder (summed per warp here) and the
 // next layer's affine step, whose sum runs over the live neurons in index
